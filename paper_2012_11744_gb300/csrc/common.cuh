@@ -37,6 +37,16 @@ struct Geo {
     }
 };
 
+// Children of coarse cell I of cn along an axis of fn fine cells halved
+// (f = 2) or kept (f = 1): f of them, three in the last cell of an odd axis.
+__host__ __device__ inline int child_count(int I, int cn, int fn, int f) { return I == cn - 1 ? fn - f * I : f; }
+
+// The coarse cell (of cn) that holds fine cell i along such an axis.
+__host__ __device__ inline int parent_of(int i, int cn, int f) {
+    const int I = i >> (f - 1);
+    return I < cn ? I : cn - 1;
+}
+
 // Coefficient set of one level: face arrays and a uniform scale (1/h^2 for
 // arrays holding beta itself, 1 for arrays that are already scaled), and an
 // optional per-cell diagonal excess sig in the units of the face arrays: the

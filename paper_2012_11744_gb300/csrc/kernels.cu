@@ -654,9 +654,16 @@ void launch_convert_scaled(int64_t n, const double* in, double scale, float* out
 // at fine index f_a*I_a along a and f_b*I_b + {0..f_b-1} along the other
 // axes b; its coefficient is their mean times (h_fine/h_coarse)^2 along a
 // (the arrays hold beta/h_a^2).  Wall faces stay 0.
+// Where an axis of odd length is halved, the last coarse cell along it has
+// three children: a face is covered by the faces of all of them (summed; the
+// divisor stays the product of the factors, as in the restriction, which
+// keeps the operator symmetric), and the flux through the last interior face
+// and through the periodic seam crosses a longer distance between centres:
+// r_last and r_seam are the fine distance over the coarse one, each in its
+// level's cell widths (1 where all cells are alike).
 template <typename T>
 __global__ void coarse_beta_kernel(Geo fg, Coef<T> cf, Geo cg, int fa0, int fa1, int fa2,
-                                   int axis, double ratio, T* __restrict__ out) {
+                                   int axis, double ratio, double r_last, double r_seam, T* __restrict__ out) {
     const int n0 = cg.nx + (axis == 0 ? cg.wx : 0);
     const int n1 = cg.ny + (axis == 1 ? cg.wy : 0);
     const int n2 = cg.nz + (axis == 2 ? cg.wz : 0);
@@ -665,6 +672,7 @@ __global__ void coarse_beta_kernel(Geo fg, Coef<T> cf, Geo cg, int fa0, int fa1,
     const T* src = axis == 0 ? cf.bx : (axis == 1 ? cf.by : cf.bz);
     const int fn0 = fg.nx + (axis == 0 ? fg.wx : 0);
     const int fn1 = fg.ny + (axis == 1 ? fg.wy : 0);
+    const int fn[3] = {fg.nx, fg.ny, fg.nz}, cn[3] = {cg.nx, cg.ny, cg.nz};
     PARIS_EW_FOR(t, total) {
         const int I = (int)(t % n0);
         const int J = (int)((t / n0) % n1);
@@ -672,8 +680,13 @@ __global__ void coarse_beta_kernel(Geo fg, Coef<T> cf, Geo cg, int fa0, int fa1,
         const int C3[3] = {I, J, K};
         int lo[3], cnt[3];
         for (int b = 0; b < 3; ++b) {
-            if (b == axis) { lo[b] = C3[b] * fac[b]; cnt[b] = 1; }
-            else { lo[b] = C3[b] * fac[b]; cnt[b] = fac[b]; }
+            lo[b] = C3[b] * fac[b];
+            cnt[b] = b == axis ? 1 : child_count(C3[b], cn[b], fn[b], fac[b]);
+        }
+        const int F = C3[axis];
+        if (F == cn[axis]) {  // the far wall: closed
+            out[t] = T(0);
+            continue;
         }
         double sum = 0.0;
         for (int dk = 0; dk < cnt[2]; ++dk)
@@ -682,18 +695,23 @@ __global__ void coarse_beta_kernel(Geo fg, Coef<T> cf, Geo cg, int fa0, int fa1,
                     int64_t fi = ((int64_t)(lo[2] + dk) * fn1 + (lo[1] + dj)) * fn0 + (lo[0] + di);
                     sum += (double)src[fi];
                 }
-        double mean = sum / (double)(cnt[0] * cnt[1] * cnt[2]);
-        out[t] = (T)(mean * ratio * (double)cf.scale);
+        const double mean = sum / (double)((fa0 * fa1 * fa2) / fac[axis]);
+        const double r = F == 0 ? r_seam : (F == cn[axis] - 1 ? r_last : 1.0);
+        out[t] = (T)(mean * ratio * (double)cf.scale * r);
     }
 }
 
 template <typename T>
 void launch_coarse_beta(const Geo& fine, const Coef<T>& cf, const Geo& coarse, const int f[3],
-                        const double hc2_over_hf2[3], T* out[3], cudaStream_t st) {
+                        const double wf[3], const double wc[3], T* out[3], cudaStream_t st) {
     for (int a = 0; a < 3; ++a) {
         int64_t n = coarse.nface(a);
+        // distances over the seam: half of the first and of the last cell's width; the
+        // last interior coarse face lies between fine cells of width 1 when the axis is halved
+        const double df = 0.5 * (1.0 + wf[a]), dc = 0.5 * (1.0 + wc[a]);
         coarse_beta_kernel<T><<<elementwise_blocks(n), kRedThreads, 0, st>>>(
-            fine, cf, coarse, f[0], f[1], f[2], a, 1.0 / hc2_over_hf2[a], out[a]);
+            fine, cf, coarse, f[0], f[1], f[2], a, 1.0 / ((double)f[a] * f[a]), (f[a] == 2 ? 1.0 : df) / dc, df / dc,
+            out[a]);
         count_launch();
     }
 }
@@ -710,10 +728,12 @@ __global__ void coarse_sig_kernel(Geo fg, const T* __restrict__ sf, double scale
         const int I = (int)(t % cg.nx);
         const int J = (int)((t / cg.nx) % cg.ny);
         const int K = (int)(t / ((int64_t)cg.nx * cg.ny));
+        const int n0 = child_count(I, cg.nx, fg.nx, fa0), n1 = child_count(J, cg.ny, fg.ny, fa1);
+        const int n2 = child_count(K, cg.nz, fg.nz, fa2);
         double sum = 0.0;
-        for (int dk = 0; dk < fa2; ++dk)
-            for (int dj = 0; dj < fa1; ++dj)
-                for (int di = 0; di < fa0; ++di)
+        for (int dk = 0; dk < n2; ++dk)
+            for (int dj = 0; dj < n1; ++dj)
+                for (int di = 0; di < n0; ++di)
                     sum += (double)sf[fg.cidx(I * fa0 + di, J * fa1 + dj, K * fa2 + dk)];
         out[t] = (T)(sum / (double)(fa0 * fa1 * fa2) * scale);
     }
@@ -1174,10 +1194,10 @@ void launch_jacobi(const Geo& g, const Coef<T>& cf, const T* w, const T* f, cons
 // Coarse right-hand side: the average over the children of the fine residual
 // f - A x (restriction R = P^T / #children for the piecewise-constant P),
 // each child's A x on its faces on the coarse cell's surface only (the
-// faces between children cancel in the sum; apply_A_faces).  FULL: the
-// 2 x 2 x 2 children of full coarsening, the loops unrolled so that the
-// loads of all eight children are in flight together (the sum keeps its
-// order).
+// faces between children cancel in the sum; apply_A_faces).  FULL: every
+// axis halved, the loops over the 2 x 2 x 2 children unrolled so that the
+// loads of all eight are in flight together (the sum keeps its order); the
+// cells of three children at the end of an odd axis take the plain loops.
 template <typename T, typename TB, bool I32, bool SIG = false, bool FULL = false>
 __global__ void restrict_residual_kernel(Geo fg, const TB* __restrict__ bx, const TB* __restrict__ by,
                                          const TB* __restrict__ bz, T scale, const T* __restrict__ f,
@@ -1189,28 +1209,37 @@ __global__ void restrict_residual_kernel(Geo fg, const TB* __restrict__ bx, cons
     const int K = blockIdx.z;
     if (I >= cg.nx || J >= cg.ny) return;
     if (FULL) fa0 = fa1 = fa2 = 2;
+    const int n0 = child_count(I, cg.nx, fg.nx, fa0), n1 = child_count(J, cg.ny, fg.ny, fa1);
+    const int n2 = child_count(K, cg.nz, fg.nz, fa2);
     T sum = T(0);
+    auto child = [&](int di, int dj, int dk, unsigned mask) {
+        const int i = I * fa0 + di, j = J * fa1 + dj, k = K * fa2 + dk;
+        Stencil<T> s;
+        int64_t c;
+        if (I32) {
+            int c32;
+            load_stencil_fast<T>(fg, bx, by, bz, i, j, k, s, c32);
+            c = c32;
+        } else {
+            c = fg.cidx(i, j, k);
+            load_stencil_as<T>(fg, bx, by, bz, i, j, k, s);
+        }
+        T ax = apply_A_faces(s, x, x[c], scale, mask);
+        if (SIG) ax = fma(scale * sig[c], x[c], ax);
+        sum += f[c] - ax;
+    };
+    if (FULL && n0 + n1 + n2 == 6) {  // eight children: their loads in flight together
 #pragma unroll
-    for (int dk = 0; dk < (FULL ? 2 : fa2); ++dk)
+        for (int dk = 0; dk < 2; ++dk)
 #pragma unroll
-        for (int dj = 0; dj < (FULL ? 2 : fa1); ++dj)
+            for (int dj = 0; dj < 2; ++dj)
 #pragma unroll
-            for (int di = 0; di < (FULL ? 2 : fa0); ++di) {
-                const int i = I * fa0 + di, j = J * fa1 + dj, k = K * fa2 + dk;
-                Stencil<T> s;
-                int64_t c;
-                if (I32) {
-                    int c32;
-                    load_stencil_fast<T>(fg, bx, by, bz, i, j, k, s, c32);
-                    c = c32;
-                } else {
-                    c = fg.cidx(i, j, k);
-                    load_stencil_as<T>(fg, bx, by, bz, i, j, k, s);
-                }
-                T ax = apply_A_faces(s, x, x[c], scale, surface_faces(di, dj, dk, fa0, fa1, fa2));
-                if (SIG) ax = fma(scale * sig[c], x[c], ax);
-                sum += f[c] - ax;
-            }
+                for (int di = 0; di < 2; ++di) child(di, dj, dk, surface_faces(di, dj, dk, 2, 2, 2));
+    } else {
+        for (int dk = 0; dk < n2; ++dk)
+            for (int dj = 0; dj < n1; ++dj)
+                for (int di = 0; di < n0; ++di) child(di, dj, dk, surface_faces(di, dj, dk, n0, n1, n2));
+    }
     fc[cg.cidx(I, J, K)] = sum / T(fa0 * fa1 * fa2);
 }
 
@@ -1267,8 +1296,7 @@ __global__ void prolong_add_kernel(Geo fg, Geo cg, int fa0, int fa1, int fa2,
     const int j = blockIdx.y * kTY + threadIdx.y;
     const int k = blockIdx.z;
     if (i >= fg.nx || j >= fg.ny) return;
-    // factors are 1 or 2: halving is a shift
-    x[fg.cidx(i, j, k)] += xc[cg.cidx(i >> (fa0 - 1), j >> (fa1 - 1), k >> (fa2 - 1))];
+    x[fg.cidx(i, j, k)] += xc[cg.cidx(parent_of(i, cg.nx, fa0), parent_of(j, cg.ny, fa1), parent_of(k, cg.nz, fa2))];
 }
 
 // x_fine += x_coarse[parent] for four x-consecutive fine cells per thread
@@ -1280,7 +1308,7 @@ __global__ void prolong_add4_kernel(Geo fg, Geo cg, const float* __restrict__ xc
     const int k = blockIdx.z;
     if (4 * q >= fg.nx || j >= fg.ny) return;
     const int64_t c = fg.cidx(4 * q, j, k);
-    const int64_t cc = cg.cidx(2 * q, j >> 1, k >> 1);
+    const int64_t cc = cg.cidx(2 * q, parent_of(j, cg.ny, 2), parent_of(k, cg.nz, 2));
     float4 v = *reinterpret_cast<const float4*>(x + c);
     const float a = xc[cc], b = xc[cc + 1];
     v.x += a;
@@ -1812,7 +1840,7 @@ cudaError_t stream_rates(const float* a, const float* b, const float* c, float* 
     template void launch_convert_beta<T>(const Geo&, const double* [3], double, T* [3],        \
                                          cudaStream_t);                                        \
     template void launch_coarse_beta<T>(const Geo&, const Coef<T>&, const Geo&, const int[3],  \
-                                        const double[3], T* [3], cudaStream_t);                \
+                                        const double[3], const double[3], T* [3], cudaStream_t); \
     template void launch_inv_diag<T>(const Geo&, const Coef<T>&, T*, cudaStream_t);            \
     template void launch_coarse_inverse<T>(const Geo&, const Coef<T>&, double*, cudaStream_t); \
     template void launch_coarse_solve<T>(const Geo&, const double*, const T*, T*, cudaStream_t, bool); \

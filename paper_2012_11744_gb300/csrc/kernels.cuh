@@ -378,7 +378,7 @@ void launch_convert_beta(const Geo& g, const double* b64[3], double scale, T* ou
 void launch_convert_scaled(int64_t n, const double* in, double scale, float* out, cudaStream_t st);
 template <typename T>
 void launch_coarse_beta(const Geo& fine, const Coef<T>& cf, const Geo& coarse, const int f[3],
-                        const double hc2_over_hf2[3], T* out[3], cudaStream_t st);
+                        const double wf[3], const double wc[3], T* out[3], cudaStream_t st);
 template <typename T>
 void launch_inv_diag(const Geo& g, const Coef<T>& cf, T* w, cudaStream_t st);
 // dense (A + a 1 1^T)^{-1} of the coarsest operator, FP64, one CTA

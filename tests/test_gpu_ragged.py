@@ -1,0 +1,63 @@
+"""Grids with odd axes (GPU): every axis is halved level by level, the last
+cell of an odd axis made of three, down to a dense coarsest level, and the
+solve lands on the oracle's solution."""
+import numpy as np
+import pytest
+
+import oracle
+import paris_inputs as pi
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+P, W = pi.PERIODIC, pi.WALL
+# odd finest axes, axes that turn odd after one and two halvings, long thin boxes, periodic odd axes
+GRIDS = [pi.Grid(45, 31, 27, 1 / 45, (W, W, W)), pi.Grid(50, 26, 34, 1 / 50, (W, P, W)),
+         pi.Grid(33, 33, 33, 1 / 33, (P, P, P)), pi.Grid(36, 20, 44, 1 / 44, (P, W, P)),
+         pi.Grid(5, 6, 203, 1 / 203, (W, W, W)), pi.Grid(131, 3, 9, 1 / 131, (P, W, W))]
+ids = lambda g: f"{g.nx}x{g.ny}x{g.nz}_{''.join('pw'[b] for b in g.bc)}"
+
+
+@pytest.fixture(scope="module")
+def paris():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2012_11744_gb300 as m
+    return m
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+@pytest.mark.parametrize("precision", ["FP64", "MIXED"])
+@pytest.mark.parametrize("grid", GRIDS, ids=ids)
+def test_odd_axes_match_oracle(paris, grid, precision):
+    """p and u to 1e-8 of the oracle's (the parity bar of the other grids),
+    without falling back to the other precision."""
+    pr = pi.random_problem(grid, seed=41, rho1=1000.0)
+    ref = oracle.projection_step(grid, pr.C, pr.rho1, pr.rho2, pr.dt, pr.u, pr.v, pr.w)
+    with paris.Context(grid, opts=paris.default_opts(precision=getattr(paris, precision))) as ctx:
+        u, p = [dev(x) for x in (pr.u, pr.v, pr.w)], torch.zeros(grid.shape, dtype=torch.float64, device="cuda")
+        st = ctx.projection_step(dev(pr.C), pr.rho1, pr.rho2, pr.dt, *u, p)
+    assert st["converged"] == 1 and st["fell_back"] == 0, st
+    assert np.abs(p.cpu().numpy() - ref.p).max() <= 1e-8 * np.abs(ref.p).max()
+    umax = max(np.abs(x).max() for x in (pr.u, pr.v, pr.w))
+    for a in range(3):
+        assert np.abs(u[a].cpu().numpy() - ref.u[a]).max() <= 1e-8 * umax
+
+
+@pytest.mark.parametrize("grid", [GRIDS[0], GRIDS[4], pi.Grid(41, 48, 57, 1 / 57, (W, P, W))], ids=ids)
+def test_tail_and_fused_sweep_bit_identical_on_odd_levels(paris, grid):
+    """The single-block tail and the fused sweep do the arithmetic of the
+    per-level kernels on levels with odd axes too (periodic axes even on
+    every smoothed level, where a colour pass has one result)."""
+    pr = pi.random_problem(grid, seed=43, rho1=1000.0)
+    out = []
+    for kw in ({"coarse_tail": 1}, {"coarse_tail": 0}, {"smoother": paris.SMOOTH_RBGS}):
+        with paris.Context(grid, opts=paris.default_opts(level0_density=0, **kw)) as ctx:
+            u, p = [dev(x) for x in (pr.u, pr.v, pr.w)], torch.zeros(grid.shape, dtype=torch.float64, device="cuda")
+            ctx.projection_step(dev(pr.C), pr.rho1, pr.rho2, pr.dt, *u, p)
+            out.append(p.cpu().numpy())
+    np.testing.assert_array_equal(out[0], out[1])
+    np.testing.assert_array_equal(out[0], out[2])
