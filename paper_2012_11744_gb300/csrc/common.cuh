@@ -252,6 +252,29 @@ __device__ inline double f2d_scaled(float v, int s) {
     return __hiloint2double((int)(sign | ((unsigned)de << 20) | (frac >> 3)), (int)(frac << 29));
 }
 
+// 1/s for s > 0 without an FP64 division and without FP64<->FP32
+// conversions (both run at the FP64 rate, 1/64 of the FP32 rate on this
+// GPU): an FP32 estimate is formed from the leading bits of s by re-biasing
+// the exponent in integer arithmetic (20 of the 52 fraction bits kept, so
+// the estimate is within 2^-20 of s), inverted with the FP32 approximate
+// reciprocal (1 ulp), re-biased back into an FP64 y0 with |1 - s y0| < 2^-19.
+// One third-order Newton-Raphson step y0 (1 + e + e^2), e = 1 - s y0,
+// leaves a truncation error e^3 < 2^-57 relative, below half an ulp, so the
+// result is within one ulp of the correctly rounded 1/s.  Values of s
+// outside the exponent window [2^-123, 2^117) (or s <= 0, NaN) take the
+// FP64 division.
+__device__ inline double recip64(double s) {
+    const int hi = __double2hiint(s);
+    if (hi < (900 << 20) || hi >= (1140 << 20)) return 1.0 / s;
+    const float sf = __int_as_float((hi - (896 << 20)) << 3);
+    float yf;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(sf));
+    const unsigned yb = (unsigned)__float_as_int(yf);
+    const double y0 = __hiloint2double((int)((yb >> 3) + (896u << 20)), (int)(yb << 29));
+    const double e = fma(-s, y0, 1.0);
+    return fma(y0, fma(e, e, e), y0);
+}
+
 // Programmatic dependent launch: a kernel launched with launch_pdl may start
 // while the kernel before it on the stream is finishing; it waits here for
 // that kernel's completion (and its memory) before touching anything the
@@ -335,6 +358,72 @@ __device__ inline void block_reduce_skc(S sum, unsigned long long key, unsigned 
         partials[3 * block + 1] = key_value(tk);
         partials[3 * block + 2] = (double)tc;
     }
+}
+
+// Block reduction of NS FP64 sums, one magnitude key (max) and one count,
+// stored as the NS + 2 partials (first sum, key_value(max), count, further
+// sums) of this block.  The threads' sums go through shared memory to one
+// warp, which adds the warps' lanes up and shuffles: 12 FP64 warp
+// instructions a sum instead of the 40 of a shuffle tree in every warp, which
+// on this GPU (FP64 at 1/64 of the FP32 rate) took as long as a quarter of the
+// work of a block of the viscous kernels.  Fixed order.
+template <int NS>
+__device__ inline void block_reduce_sums_kc(const double (&sum)[NS], unsigned long long key, unsigned cnt,
+                                            double* partials, int64_t block, int tid) {
+    __shared__ double sh_s[NS][kRedThreads];
+    __shared__ unsigned long long sh_k[kRedThreads / 32];
+    __shared__ unsigned sh_c[kRedThreads / 32];
+    const unsigned all = 0xffffffffu;
+    const int lane = tid & 31, wid = tid >> 5;
+#pragma unroll
+    for (int q = 0; q < NS; ++q) sh_s[q][tid] = sum[q];
+    const unsigned khi = __reduce_max_sync(all, (unsigned)(key >> 32));
+    const unsigned klo = __reduce_max_sync(all, (unsigned)(key >> 32) == khi ? (unsigned)key : 0u);
+    cnt = __reduce_add_sync(all, cnt);
+    if (lane == 0) {
+        sh_k[wid] = ((unsigned long long)khi << 32) | klo;
+        sh_c[wid] = cnt;
+    }
+    __syncthreads();
+    if (wid != 0) return;
+    double t[NS];
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+        t[q] = sh_s[q][lane];
+#pragma unroll
+        for (int w = 1; w < kRedThreads / 32; ++w) t[q] += sh_s[q][32 * w + lane];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < NS; ++q) t[q] += __shfl_xor_sync(all, t[q], o);
+    if (lane == 0) {
+        unsigned long long tk = 0;
+        unsigned tc = 0;
+        for (int w = 0; w < kRedThreads / 32; ++w) {
+            tk = sh_k[w] > tk ? sh_k[w] : tk;
+            tc += sh_c[w];
+        }
+        double* out = partials + (NS + 2) * block;
+        out[0] = t[0];
+        out[1] = key_value(tk);
+        out[2] = (double)tc;
+#pragma unroll
+        for (int q = 1; q < NS; ++q) out[2 + q] = t[q];
+    }
+}
+
+// Block reduction of one FP64 sum, the block's only partial (as above).
+__device__ inline void block_reduce_sum(double sum, double* partials, int64_t block, int tid) {
+    __shared__ double sh[kRedThreads];
+    sh[tid] = sum;
+    __syncthreads();
+    if (tid >= 32) return;
+    double t = sh[tid];
+#pragma unroll
+    for (int w = 1; w < kRedThreads / 32; ++w) t += sh[32 * w + tid];
+    t = warp_sum(t);
+    if (tid == 0) partials[block] = t;
 }
 
 }  // namespace paris

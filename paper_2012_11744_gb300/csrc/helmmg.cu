@@ -426,19 +426,6 @@ __global__ void __launch_bounds__(kTX* kTY) hmg_setup_kernel(HelmGeo g, const do
     finalize_last_block(partials, (int64_t)gridDim.x * gridDim.y * gridDim.z, fin, tid);
 }
 
-// the component's wall faces of its own axis: u* = 0 there
-__global__ void hmg_wall_zero_kernel(HelmGeo g, double* __restrict__ us) {
-    const int c = g.comp, a1 = c == 0 ? 1 : 0, a2 = c == 2 ? 1 : 2;
-    const int64_t plane = (int64_t)g.e[a1] * g.e[a2];
-    const int64_t se[3] = {1, g.e[0], (int64_t)g.e[0] * g.e[1]};
-    for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < 2 * plane; w += (int64_t)gridDim.x * blockDim.x) {
-        const int side = w >= plane;
-        const int64_t rem = w - side * plane;
-        const int64_t i2 = rem / g.e[a1], i1 = rem - i2 * g.e[a1];
-        us[i1 * se[a1] + i2 * se[a2] + (int64_t)side * (g.e[c] - 1) * se[c]] = 0.0;
-    }
-}
-
 // FP64 operator on the unknowns of x stored with strides st (the face array
 // of u*, or a Krylov vector): returns sigma x_c - Lap_h x at (i, j, k)
 __device__ __forceinline__ double hop64(const HelmGeo& g, const double* __restrict__ x, int64_t c,
@@ -623,12 +610,7 @@ int64_t launch_hmg_setup(const HelmGeo& g, const double* un, const double* nu, d
     const dim3 gr = hgrid(g.m, kZ);
     hmg_setup_kernel<<<gr, dim3(kTX, kTY), 0, st>>>(g, un, nu, tau, sig64, sig32, us, partials, fin);
     count_launch();
-    if (g.wall) {
-        const int c = g.comp, a1 = c == 0 ? 1 : 0, a2 = c == 2 ? 1 : 2;
-        const int64_t n = 2 * (int64_t)g.e[a1] * g.e[a2];
-        hmg_wall_zero_kernel<<<elementwise_blocks(n), kRedThreads, 0, st>>>(g, us);
-        count_launch();
-    }
+    launch_helm_wall_zero(g, us, st);
     return (int64_t)gr.x * gr.y * gr.z;
 }
 

@@ -143,8 +143,24 @@ int elementwise_blocks(int64_t n) {
     return (int)b;
 }
 
+int march_planes(int64_t tiles, int nz, int per_sm) {
+    const int64_t cap = (int64_t)device_sms() * per_sm;
+    int best = nz;
+    int64_t least = INT64_MAX;
+    for (int p = nz < 64 ? nz : 64; p >= (nz < kMinMarch ? nz : kMinMarch); --p) {
+        if ((nz + p - 1) / p > 65535) break;  // gridDim.z
+        const int64_t blocks = tiles * ((nz + p - 1) / p);
+        const int64_t cost = ((blocks + cap - 1) / cap) * (p + 2);
+        if (cost < least) {
+            least = cost;
+            best = p;
+        }
+    }
+    return best;
+}
+
 int64_t max_reduce_blocks(const Geo& g) {
-    const int64_t tiles = nblocks_of(tile_grid(g, kZ));
+    const int64_t tiles = nblocks_of(tile_grid(g, kMinMarch));
     const int64_t ew = elementwise_blocks(g.ncell());
     return tiles > ew ? tiles : ew;
 }
@@ -165,29 +181,6 @@ void finalize(const double* partials, int64_t nblocks, int nv, int maxmask, Scal
 }
 
 // ------------------------------------------------------- face coefficients ---
-
-// 1/s for s > 0 without an FP64 division and without FP64<->FP32
-// conversions (both run at the FP64 rate, 1/64 of the FP32 rate on this
-// GPU): an FP32 estimate is formed from the leading bits of s by re-biasing
-// the exponent in integer arithmetic (20 of the 52 fraction bits kept, so
-// the estimate is within 2^-20 of s), inverted with the FP32 approximate
-// reciprocal (1 ulp), re-biased back into an FP64 y0 with |1 - s y0| < 2^-19.
-// One third-order Newton-Raphson step y0 (1 + e + e^2), e = 1 - s y0,
-// leaves a truncation error e^3 < 2^-57 relative, below half an ulp, so the
-// result is within one ulp of the correctly rounded 1/s.  Values of s
-// outside the exponent window [2^-123, 2^117) (or s <= 0, NaN) take the
-// FP64 division.
-__device__ inline double recip64(double s) {
-    const int hi = __double2hiint(s);
-    if (hi < (900 << 20) || hi >= (1140 << 20)) return 1.0 / s;
-    const float sf = __int_as_float((hi - (896 << 20)) << 3);
-    float yf;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(sf));
-    const unsigned yb = (unsigned)__float_as_int(yf);
-    const double y0 = __hiloint2double((int)((yb >> 3) + (896u << 20)), (int)(yb << 29));
-    const double e = fma(-s, y0, 1.0);
-    return fma(y0, fma(e, e, e), y0);
-}
 
 constexpr int kFSeg = 16;  // planes per thread of the face-coefficient kernel
 

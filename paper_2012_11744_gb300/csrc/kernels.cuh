@@ -189,6 +189,13 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 int device_sms();
 // Grid of the element-wise kernels (kEW elements per thread).
 int elementwise_blocks(int64_t n);
+// Planes per block of a kernel whose 32 x 8 tiles march along z, `tiles`
+// tiles a plane, per_sm blocks resident on an SM: the number that fills the
+// chip in the fewest, fullest waves (a block's start and its reduction count as
+// two planes' work).  A fixed number leaves the last wave nearly empty at some
+// sizes (128^3 doubles at 8 planes: 1.35 waves) and the chip at others.
+int march_planes(int64_t tiles, int nz, int per_sm);
+constexpr int kMinMarch = 2;  // the fewest it returns (one on a single plane)
 // Most blocks any reducing kernel launches on a grid of this size (the
 // number of partial-sum slots a caller must provide, per value).
 int64_t max_reduce_blocks(const Geo& g);
@@ -316,20 +323,25 @@ int64_t launch_hmg_scale_d2f(int64_t n, const double* r, const Scal* s, float* r
 void launch_hmg_accumulate(const HelmGeo& g, const float* e, const Scal* s, double* us, cudaStream_t st);
 int64_t helm_unknowns(const HelmGeo& g);
 int64_t helm_faces(const HelmGeo& g);
-// us = un on the unknowns, 0 on the wall faces; partials (|b|^2, max|b|,
-// non-finite count, 0) of b = un/(tau nu)
-int64_t launch_helm_init(const HelmGeo& g, const double* un, const double* nu, double tau, double* us,
-                         double* partials, cudaStream_t st, FinSpec fin);
-// r = b - A x, z = r/diag(A); partials (r.r, max|r|, non-finite count, r.z)
-int64_t launch_helm_residual(const HelmGeo& g, const double* un, const double* nu, double tau, const double* x,
-                             double* r, double* z, double* partials, cudaStream_t st, FinSpec fin);
+// sig = 1/(tau nu) and w = 1/(sig + diag(-Lap_h)) on the unknowns; us = un
+// there, 0 on the wall faces; partials (|b|^2, max|b|, non-finite count) of
+// b = sig un
+void launch_helm_init(const HelmGeo& g, const double* un, const double* nu, double tau, double* sig, double* w,
+                      double* us, double* partials, cudaStream_t st, FinSpec fin);
+// us = 0 on the wall faces of the component's own axis
+void launch_helm_wall_zero(const HelmGeo& g, double* us, cudaStream_t st);
+// r = b - A x; partials (r.r, max|r|, non-finite count, r.z) with z = w r
+void launch_helm_residual(const HelmGeo& g, const double* un, const double* sig, const double* w, const double* x,
+                          double* r, double* partials, cudaStream_t st, FinSpec fin);
 // q = A d; partials d.q
-int64_t launch_helm_matvec_dot(const HelmGeo& g, const double* nu, double tau, const double* d, double* q,
-                               double* partials, cudaStream_t st, FinSpec fin);
-// x += alpha d, r -= alpha q, z = r/diag(A); partials as launch_helm_residual
-int64_t launch_helm_update(const HelmGeo& g, const double* nu, double tau, const Scal* s, const double* d,
-                           const double* q, double* x, double* r, double* z, double* partials, cudaStream_t st,
-                           FinSpec fin);
+void launch_helm_matvec_dot(const HelmGeo& g, const double* sig, const double* d, double* q, double* partials,
+                            cudaStream_t st, FinSpec fin);
+// x += alpha d, r -= alpha q; partials as launch_helm_residual
+void launch_helm_update(const HelmGeo& g, const double* w, const Scal* s, const double* d, const double* q,
+                        double* x, double* r, double* partials, cudaStream_t st, FinSpec fin);
+// d = w r + beta d (first: d = w r)
+void launch_helm_direction(int64_t n, const Scal* s, const double* w, const double* r, double* d, bool first,
+                           cudaStream_t st);
 // nu_f = (mu_L + mu_R)/(rho_L + rho_R) on the component's faces, 0 on its wall faces
 void launch_helm_face_nu(const HelmGeo& g, const Geo& g0, const double* C, double mu1, double mu2, double rho1,
                          double rho2, double* nu, cudaStream_t st);

@@ -1747,8 +1747,10 @@ paris_status paris_viscous_solve(paris_ctx* c, int comp, const double* nu, doubl
     if (st) *st = paris_stats{};
     const HelmGeo g = helm_geo(c->g0, comp, c->grid.h);
     CK(cudaMemsetAsync(c->scal, 0, sizeof(Scal), c->st));
+    double *r = c->r, *d = c->d, *q = c->q;
+    double *sig = c->f, *w = c->rhs;  // 1/(tau nu) and 1/diag, formed once a solve
     if (tau == 0.0) {  // u* = u^n
-        launch_helm_init(g, un, nu, 1.0, us, c->partials, c->st, no_fin());
+        launch_helm_init(g, un, nu, 1.0, sig, w, us, c->partials, c->st, no_fin());
         CK(cudaGetLastError());
         CK(cudaStreamSynchronize(c->st));
         if (st) st->converged = 1;
@@ -1756,9 +1758,8 @@ paris_status paris_viscous_solve(paris_ctx* c, int comp, const double* nu, doubl
     }
     const auto met = [tol](const Scal& h) { return h.rr <= tol * tol * h.bnorm2 && h.rinf <= tol * h.binf; };
     const FinSpec rnorms{c->scal, 4, 2, FIN_RNORMS_RHO, 0.0};
-    double *r = c->r, *z = c->z, *d = c->d, *q = c->q;
-    launch_helm_init(g, un, nu, tau, us, c->partials, c->st, FinSpec{c->scal, 4, 0xA, FIN_BNORMS, 0.0});
-    launch_helm_residual(g, un, nu, tau, us, r, z, c->partials, c->st, rnorms);
+    launch_helm_init(g, un, nu, tau, sig, w, us, c->partials, c->st, FinSpec{c->scal, 3, 2, FIN_BNORMS, 0.0});
+    launch_helm_residual(g, un, sig, w, us, r, c->partials, c->st, rnorms);
     CK(cudaGetLastError());
     paris_status s = read_scal(c);
     if (s != PARIS_OK) return s;
@@ -1766,22 +1767,30 @@ paris_status paris_viscous_solve(paris_ctx* c, int comp, const double* nu, doubl
     bool converged = c->scal_h->bnorm2 == 0.0 || met(*c->scal_h);
     bool nonfinite = c->scal_h->nonfinite > 0;
     while (!converged && !nonfinite && iters < max_iter) {
-        std::swap(d, z);  // first direction d = z: exchange the buffers
         bool inner = false;
+        // the next direction and its product go in behind the norms' copy, so
+        // the GPU works on while the host reads them; after the last
+        // iteration they go unused (d and q only)
+        auto next_product = [&](bool first) {
+            launch_helm_direction(helm_unknowns(g), c->scal, w, r, d, first, c->st);
+            launch_helm_matvec_dot(g, sig, d, q, c->partials, c->st, FinSpec{c->scal, 1, 0, FIN_ALPHA, 0.0});
+        };
+        next_product(true);
         while (iters < max_iter) {
-            launch_helm_matvec_dot(g, nu, tau, d, q, c->partials, c->st, FinSpec{c->scal, 1, 0, FIN_ALPHA, 0.0});
-            launch_helm_update(g, nu, tau, c->scal, d, q, us, r, z, c->partials, c->st, rnorms);
+            launch_helm_update(g, w, c->scal, d, q, us, r, c->partials, c->st, rnorms);
+            s = read_scal_async(c);
+            if (s != PARIS_OK) return s;
+            if (iters + 1 < max_iter) next_product(false);
             CK(cudaGetLastError());
-            s = read_scal(c);
+            s = read_scal_wait(c);
             if (s != PARIS_OK) return s;
             ++iters;
             if (c->scal_h->nonfinite > 0) { nonfinite = true; break; }
             if (met(*c->scal_h)) { inner = true; break; }
-            launch_xpby<double>(helm_unknowns(g), c->scal, z, d, c->st);  // d = z + beta d
         }
         if (nonfinite) break;
         // verify with the true residual; restart from it if the recurrence drifted
-        launch_helm_residual(g, un, nu, tau, us, r, z, c->partials, c->st, rnorms);
+        launch_helm_residual(g, un, sig, w, us, r, c->partials, c->st, rnorms);
         CK(cudaGetLastError());
         s = read_scal(c);
         if (s != PARIS_OK) return s;

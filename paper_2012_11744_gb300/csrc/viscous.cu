@@ -12,176 +12,300 @@
 // cell away, Sec. 2.2).
 //
 // u^n, nu and u* are full face arrays (the library's face layout); the
-// Krylov vectors r, z, d, q hold only the unknowns, x fastest.  The Jacobi
-// step z = r / diag is fused into the kernels that produce r, which also
-// reduce r . r, max |r|, the non-finite count and r . z.
+// Krylov vectors r, d, q and the per-unknown sigma = 1/(tau nu) and
+// w = 1/diag hold only the unknowns, x fastest.
+//
+// What bounds these kernels is the FP64 pipe (1/64 of the FP32 rate on this
+// GPU, 0.58e12 instructions a second), so everything that does not change
+// during a solve is formed once: sigma and w by one setup pass, where each
+// product and update used to divide by tau nu and by the diagonal (a division
+// is about ten FP64 instructions).  A Laplacian is five additions of
+// neighbours and one fused step with the integer diagonal count; maxima and
+// non-finite tests are integer comparisons; z = w r is formed where it is
+// used and never stored.  That leaves 9 FP64 instructions per unknown for the
+// product, 5 for the update and 2 for the direction.  At 128^3 (ncu, cold
+// caches): product 97 -> 56 us, update 118 -> 41 us a launch, the FP64 pipe 80 %
+// busy while the product's blocks run; a step of three components 55.3 ->
+// 26.0 ms.  The product's threads own z-columns of a 32 x 8 tile (no index
+// divisions), the column's values carried from plane to plane.
+#include <algorithm>
+
 #include "kernels.cuh"
 
 namespace paris {
 
 namespace {
 
-__device__ __forceinline__ void helm_pos(const HelmGeo& g, int64_t p, int (&pos)[3]) {
-    const int64_t t = p / g.m[0];
-    pos[0] = (int)(p - t * g.m[0]);
-    pos[1] = (int)(t % g.m[1]);
-    pos[2] = (int)(t / g.m[1]);
-}
+constexpr int kTX = 32, kTY = 8;  // tile of the marching kernels
+constexpr int kPerSM = 4;         // their resident blocks per SM (at most 64 registers)
 
-// index in the full face array of the unknown at pos
-__device__ __forceinline__ int64_t helm_face(const HelmGeo& g, const int (&pos)[3]) {
-    return g.off + pos[0] + (int64_t)g.e[0] * (pos[1] + (int64_t)g.e[1] * pos[2]);
-}
+// The column (i, j) of unknowns over planes [k0, k1) of an array x with
+// strides st: base points at (i, j, 0).  next(k) returns Lap_h x / ih2 at
+// plane k: the neighbours present (or wrapped) summed, minus the diagonal
+// count times the value: 2 an axis, one more at a no-slip end (ghost value
+// minus the end value), 0 along a periodic axis of one point.
+struct HelmColumn {
+    const double* base;
+    int64_t sz, oxm, oxp, oym, oyp;  // plane stride; offsets of the x and y neighbours
+    bool hxm, hxp, hym, hyp;         // which of them exist
+    int m2, kz;                      // planes and the kind of the z axis
+    double dxy;                      // diagonal count of the x and y axes
+    double zm, zc;
 
-// Lap_h x at the entry c of x (position pos, value xc); st: strides of x
-__device__ __forceinline__ double helm_lap(const HelmGeo& g, const double* __restrict__ x, int64_t c,
-                                           const int64_t (&st)[3], const int (&pos)[3], double xc) {
-    double s = 0.0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int m = g.m[a];
-        const int kind = g.kind[a];
-        const double end = kind == HELM_ZERO ? 0.0 : -xc;  // beyond a wall
-        const double lo = pos[a] > 0 ? x[c - st[a]] : (kind == HELM_PERIODIC ? x[c + (int64_t)(m - 1) * st[a]] : end);
-        const double hi = pos[a] < m - 1 ? x[c + st[a]] : (kind == HELM_PERIODIC ? x[c - (int64_t)(m - 1) * st[a]] : end);
-        s += (lo + hi) - 2.0 * xc;
+    __device__ __forceinline__ HelmColumn(const HelmGeo& g, const double* x, const int64_t (&st)[3], int i, int j,
+                                          int k0) {
+        base = x + i * st[0] + j * st[1];
+        sz = st[2];
+        auto axis = [&](int a, int p, bool& hm, bool& hp, int64_t& om, int64_t& op) {
+            const int m = g.m[a];
+            const bool per = g.kind[a] == HELM_PERIODIC;
+            hm = per ? m > 1 : p > 0;
+            hp = per ? m > 1 : p < m - 1;
+            om = p > 0 ? -st[a] : (int64_t)(m - 1) * st[a];
+            op = p < m - 1 ? st[a] : -(int64_t)(m - 1) * st[a];
+            return (double)count(g.kind[a], m, p);
+        };
+        dxy = axis(0, i, hxm, hxp, oxm, oxp) + axis(1, j, hym, hyp, oym, oyp);
+        m2 = g.m[2];
+        kz = g.kind[2];
+        zc = base[k0 * sz];
+        zm = below(k0);
     }
-    return s * g.ih2;
-}
+    __device__ __forceinline__ static int count(int kind, int m, int p) {
+        if (kind == HELM_PERIODIC) return m > 1 ? 2 : 0;
+        return 2 + (kind == HELM_NOSLIP ? (p == 0) + (p == m - 1) : 0);
+    }
+    __device__ __forceinline__ double below(int k) const {
+        if (k > 0) return base[(k - 1) * sz];
+        return kz == HELM_PERIODIC && m2 > 1 ? base[(m2 - 1) * sz] : 0.0;
+    }
+    __device__ __forceinline__ double above(int k) const {
+        if (k < m2 - 1) return base[(k + 1) * sz];
+        return kz == HELM_PERIODIC && m2 > 1 ? base[0] : 0.0;
+    }
+    __device__ __forceinline__ double next(int k, double& xc) {
+        const double* c = base + k * sz;
+        const double xm = hxm ? c[oxm] : 0.0, xp = hxp ? c[oxp] : 0.0;
+        const double ym = hym ? c[oym] : 0.0, yp = hyp ? c[oyp] : 0.0;
+        const double zp = above(k);
+        xc = zc;
+        const double dg = dxy + (double)count(kz, m2, k);
+        const double s = ((xm + xp) + (ym + yp)) + (zm + zp);
+        zm = zc;
+        zc = zp;
+        return fma(-dg, xc, s);
+    }
+};
 
-// diagonal of diag(1/(tau nu)) - Lap_h at pos
-__device__ __forceinline__ double helm_diag(const HelmGeo& g, const int (&pos)[3], double inv_tnu) {
-    double d = 0.0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int m = g.m[a];
-        if (g.kind[a] == HELM_PERIODIC) {
-            d += m > 1 ? 2.0 : 0.0;  // one point along a periodic axis is its own neighbour
-        } else {
-            d += 2.0;
-            if (g.kind[a] == HELM_NOSLIP) d += (pos[a] == 0 ? 1.0 : 0.0) + (pos[a] == m - 1 ? 1.0 : 0.0);
+__device__ __forceinline__ int64_t helm_block() {
+    return ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+}
+__device__ __forceinline__ int64_t helm_blocks() { return (int64_t)gridDim.x * gridDim.y * gridDim.z; }
+
+// sigma = 1/(tau nu) and w = 1/(sigma + diag(-Lap_h)) on the unknowns;
+// u* = u^n there (the initial guess), 0 on the component's wall faces;
+// partials of |b|^2, max |b| and the non-finite count (a nu that is not
+// positive counts), with b = sigma u^n
+__global__ void __launch_bounds__(kTX* kTY, kPerSM) helm_init_kernel(HelmGeo g, const double* __restrict__ un,
+                                                            const double* __restrict__ nu, double tau,
+                                                            double* __restrict__ sig, double* __restrict__ w,
+                                                            double* __restrict__ us, double* partials, int zper, FinSpec fin) {
+    const int i = blockIdx.x * kTX + threadIdx.x, j = blockIdx.y * kTY + threadIdx.y;
+    const int tid = threadIdx.y * kTX + threadIdx.x;
+    double l2[1] = {0.0};
+    unsigned long long bk = 0;
+    unsigned nf = 0;
+    if (i < g.m[0] && j < g.m[1]) {
+        const int k0 = blockIdx.z * zper, k1 = min(k0 + zper, g.m[2]);
+        const int dxy = HelmColumn::count(g.kind[0], g.m[0], i) + HelmColumn::count(g.kind[1], g.m[1], j);
+        for (int k = k0; k < k1; ++k) {
+            const int64_t p = ((int64_t)k * g.m[1] + j) * g.m[0] + i;
+            const int64_t f = g.off + i + (int64_t)g.e[0] * (j + (int64_t)g.e[1] * k);
+            const double v = un[f], nv = nu[f];
+            us[f] = v;
+            const double s = recip64(tau * nv);
+            sig[p] = s;
+            w[p] = recip64(fma((double)(dxy + HelmColumn::count(g.kind[2], g.m[2], k)), g.ih2, s));
+            const double b = s * v;
+            l2[0] = fma(b, b, l2[0]);
+            const unsigned long long kb = abs_key(b);
+            bk = kb > bk ? kb : bk;
+            nf += (key_nonfinite(kb) || !(nv > 0.0)) ? 1u : 0u;
         }
     }
-    return inv_tnu + d * g.ih2;
+    block_reduce_sums_kc<1>(l2, bk, nf, partials, helm_block(), tid);
+    finalize_last_block(partials, helm_blocks(), fin, tid);
 }
 
-// u* = u^n on the unknowns (the initial guess), 0 on the component's wall
-// faces; partials of |b|^2, max |b|, the non-finite count (a nu that is not
-// positive counts) and 0, with b = u^n / (tau nu)
-__global__ void helm_init_kernel(HelmGeo g, int64_t n, const double* __restrict__ un,
-                                 const double* __restrict__ nu, double tau, double* __restrict__ us,
-                                 double* partials, FinSpec fin) {
-    double l2 = 0.0, mx = 0.0;
-    unsigned nf = 0;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    for (int64_t p = t0; p < n; p += stride) {
-        int pos[3];
-        helm_pos(g, p, pos);
-        const int64_t f = helm_face(g, pos);
-        const double v = un[f];
-        const double nv = nu[f];
-        us[f] = v;
-        const double b = v / (tau * nv);
-        l2 = fma(b, b, l2);
-        mx = fmax(mx, fabs(b));
-        nf += (isfinite(b) && nv > 0.0) ? 0u : 1u;
-    }
-    // the two wall planes of the component's own axis (none along a periodic axis)
-    if (g.wall) {
-        const int c = g.comp, a1 = c == 0 ? 1 : 0, a2 = c == 2 ? 1 : 2;
-        const int64_t plane = (int64_t)g.e[a1] * g.e[a2];
-        const int64_t se[3] = {1, g.e[0], (int64_t)g.e[0] * g.e[1]};
-        for (int64_t w = t0; w < 2 * plane; w += stride) {
-            const int side = w >= plane;
-            const int64_t rem = w - side * plane;
-            const int64_t i2 = rem / g.e[a1];
-            const int64_t i1 = rem - i2 * g.e[a1];
-            us[i1 * se[a1] + i2 * se[a2] + (int64_t)side * (g.e[c] - 1) * se[c]] = 0.0;
-        }
-    }
-    double acc[4] = {l2, mx, (double)nf, 0.0};
-    const int op[4] = {0, 1, 0, 1};
-    block_reduce_store<4>(acc, op, partials, blockIdx.x, threadIdx.x);
-    finalize_last_block(partials, gridDim.x, fin, threadIdx.x);
-}
-
-// r = u^n/(tau nu) - (x/(tau nu) - Lap_h x), z = r / diag; partials of
-// r . r, max |r|, the non-finite count, r . z
-__global__ void helm_residual_kernel(HelmGeo g, int64_t n, const double* __restrict__ un,
-                                     const double* __restrict__ nu, double tau, const double* __restrict__ x,
-                                     double* __restrict__ r, double* __restrict__ z, double* partials,
-                                     FinSpec fin) {
-    double l2 = 0.0, mx = 0.0, rz = 0.0;
-    unsigned nf = 0;
+// the two wall planes of the component's own axis: u* = 0 there
+__global__ void helm_wall_zero_kernel(HelmGeo g, double* __restrict__ us) {
+    const int c = g.comp, a1 = c == 0 ? 1 : 0, a2 = c == 2 ? 1 : 2;
+    const int64_t plane = (int64_t)g.e[a1] * g.e[a2];
     const int64_t se[3] = {1, g.e[0], (int64_t)g.e[0] * g.e[1]};
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-        int pos[3];
-        helm_pos(g, p, pos);
-        const int64_t f = helm_face(g, pos);
-        const double xc = x[f];
-        const double inv_tnu = 1.0 / (tau * nu[f]);
-        const double rp = (un[f] - xc) * inv_tnu + helm_lap(g, x, f, se, pos, xc);
-        const double zp = rp / helm_diag(g, pos, inv_tnu);
-        r[p] = rp;
-        z[p] = zp;
-        l2 = fma(rp, rp, l2);
-        mx = fmax(mx, fabs(rp));
-        rz = fma(rp, zp, rz);
-        nf += isfinite(rp) ? 0u : 1u;
+    for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < 2 * plane; w += (int64_t)gridDim.x * blockDim.x) {
+        const int side = w >= plane;
+        const int64_t rem = w - side * plane;
+        const int64_t i2 = rem / g.e[a1], i1 = rem - i2 * g.e[a1];
+        us[i1 * se[a1] + i2 * se[a2] + (int64_t)side * (g.e[c] - 1) * se[c]] = 0.0;
     }
-    double acc[4] = {l2, mx, (double)nf, rz};
-    const int op[4] = {0, 1, 0, 0};
-    block_reduce_store<4>(acc, op, partials, blockIdx.x, threadIdx.x);
-    finalize_last_block(partials, gridDim.x, fin, threadIdx.x);
 }
 
-// q = d/(tau nu) - Lap_h d and the partials of d . q
-__global__ void helm_matvec_dot_kernel(HelmGeo g, int64_t n, const double* __restrict__ nu, double tau,
-                                       const double* __restrict__ d, double* __restrict__ q, double* partials,
-                                       FinSpec fin) {
-    double dq = 0.0;
-    const int64_t su[3] = {1, g.m[0], (int64_t)g.m[0] * g.m[1]};
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-        int pos[3];
-        helm_pos(g, p, pos);
-        const double dc = d[p];
-        const double qp = dc / (tau * nu[helm_face(g, pos)]) - helm_lap(g, d, p, su, pos, dc);
-        q[p] = qp;
-        dq = fma(dc, qp, dq);
-    }
-    double acc[1] = {dq};
-    const int op[1] = {0};
-    block_reduce_store<1>(acc, op, partials, blockIdx.x, threadIdx.x);
-    finalize_last_block(partials, gridDim.x, fin, threadIdx.x);
-}
-
-// x += alpha d, r -= alpha q, z = r / diag; partials as the residual kernel's
-__global__ void helm_update_kernel(HelmGeo g, int64_t n, const double* __restrict__ nu, double tau,
-                                   const Scal* __restrict__ s, const double* __restrict__ d,
-                                   const double* __restrict__ q, double* __restrict__ x, double* __restrict__ r,
-                                   double* __restrict__ z, double* partials, FinSpec fin) {
-    const double alpha = s->alpha;
-    double l2 = 0.0, mx = 0.0, rz = 0.0;
+// r = sigma (u^n - x) + Lap_h x; partials of r . r, max |r|, the non-finite
+// count, r . w r
+__global__ void __launch_bounds__(kTX* kTY, kPerSM) helm_residual_kernel(HelmGeo g, const double* __restrict__ un,
+                                                                const double* __restrict__ sig,
+                                                                const double* __restrict__ w,
+                                                                const double* __restrict__ x, double* __restrict__ r,
+                                                                double* partials, int zper, FinSpec fin) {
+    const int i = blockIdx.x * kTX + threadIdx.x, j = blockIdx.y * kTY + threadIdx.y;
+    const int tid = threadIdx.y * kTX + threadIdx.x;
+    double sums[2] = {0.0, 0.0};  // r . r and r . z
+    unsigned long long rk = 0;
     unsigned nf = 0;
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-        int pos[3];
-        helm_pos(g, p, pos);
-        const int64_t f = helm_face(g, pos);
+    if (i < g.m[0] && j < g.m[1]) {
+        const int k0 = blockIdx.z * zper, k1 = min(k0 + zper, g.m[2]);
+        const int64_t se[3] = {1, g.e[0], (int64_t)g.e[0] * g.e[1]};
+        HelmColumn col(g, x + g.off, se, i, j, k0);
+        for (int k = k0; k < k1; ++k) {
+            const int64_t p = ((int64_t)k * g.m[1] + j) * g.m[0] + i;
+            const int64_t f = g.off + i + (int64_t)g.e[0] * (j + (int64_t)g.e[1] * k);
+            double xc;
+            const double lap = col.next(k, xc);
+            const double rp = fma(g.ih2, lap, sig[p] * (un[f] - xc));
+            r[p] = rp;
+            sums[0] = fma(rp, rp, sums[0]);
+            sums[1] = fma(rp, rp * w[p], sums[1]);
+            const unsigned long long kr = abs_key(rp);
+            rk = kr > rk ? kr : rk;
+            nf += key_nonfinite(kr);
+        }
+    }
+    block_reduce_sums_kc<2>(sums, rk, nf, partials, helm_block(), tid);
+    finalize_last_block(partials, helm_blocks(), fin, tid);
+}
+
+// q = sigma d - Lap_h d and the partials of d . q
+__global__ void __launch_bounds__(kTX* kTY, kPerSM) helm_matvec_dot_kernel(HelmGeo g, const double* __restrict__ sig,
+                                                                  const double* __restrict__ d,
+                                                                  double* __restrict__ q, double* partials,
+                                                                  int zper, FinSpec fin) {
+    pdl_wait();
+    const int i = blockIdx.x * kTX + threadIdx.x, j = blockIdx.y * kTY + threadIdx.y;
+    const int tid = threadIdx.y * kTX + threadIdx.x;
+    double dq = 0.0;
+    if (i < g.m[0] && j < g.m[1]) {
+        const int k0 = blockIdx.z * zper, k1 = min(k0 + zper, g.m[2]);
+        const int64_t su[3] = {1, g.m[0], (int64_t)g.m[0] * g.m[1]};
+        HelmColumn col(g, d, su, i, j, k0);
+#pragma unroll 4
+        for (int k = k0; k < k1; ++k) {
+            const int64_t p = ((int64_t)k * g.m[1] + j) * g.m[0] + i;
+            double dc;
+            const double lap = col.next(k, dc);
+            const double qp = fma(-g.ih2, lap, sig[p] * dc);
+            q[p] = qp;
+            dq = fma(dc, qp, dq);
+        }
+    }
+    block_reduce_sum(dq, partials, helm_block(), tid);
+    finalize_last_block(partials, helm_blocks(), fin, tid);
+}
+
+// p / d for p < 2^31 by the multiplier m = floor(2^32 / d) + 1 and one
+// correction (the estimate is at most one too large)
+__device__ __forceinline__ unsigned fast_div(unsigned p, unsigned d, unsigned m) {
+    const unsigned q = d == 1 ? p : __umulhi(p, m);
+    return q * d > p ? q - 1 : q;
+}
+
+constexpr int kUU = 4;  // unknowns in flight per thread of the update
+
+// x += alpha d, r -= alpha q; partials as the residual kernel's.  A
+// grid-stride loop on resident blocks only (no last wave), four unknowns in
+// flight per thread.
+__global__ void __launch_bounds__(kRedThreads, kPerSM) helm_update_kernel(HelmGeo g, unsigned n, unsigned mul0,
+                                                                         unsigned mul1,
+                                                                         const double* __restrict__ w,
+                                                                         const Scal* __restrict__ s,
+                                                                         const double* __restrict__ d,
+                                                                         const double* __restrict__ q,
+                                                                         double* __restrict__ x,
+                                                                         double* __restrict__ r, double* partials,
+                                                                         FinSpec fin) {
+    pdl_wait();
+    const double alpha = s->alpha;
+    double sums[2] = {0.0, 0.0};
+    unsigned long long rk = 0;
+    unsigned nf = 0;
+    const unsigned m0 = (unsigned)g.m[0], m1 = (unsigned)g.m[1];
+    const bool flat = g.e[0] == g.m[0] && g.e[1] == g.m[1];  // the face array minus its offset is the vector
+    auto face = [&](unsigned p) {
+        if (flat) return g.off + (int64_t)p;
+        const unsigned row = fast_div(p, m0, mul0), k = fast_div(row, m1, mul1);
+        return g.off + (int64_t)(p - row * m0) + (int64_t)g.e[0] * ((row - k * m1) + (int64_t)g.e[1] * k);
+    };
+    const unsigned stride = gridDim.x * blockDim.x;
+    auto one = [&](double rp, double wp) {
+        sums[0] = fma(rp, rp, sums[0]);
+        sums[1] = fma(rp, rp * wp, sums[1]);
+        const unsigned long long kr = abs_key(rp);
+        rk = kr > rk ? kr : rk;
+        nf += key_nonfinite(kr);
+    };
+    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (; p + (int64_t)(kUU - 1) * stride < n; p += (int64_t)kUU * stride) {
+        double dv[kUU], qv[kUU], xv[kUU], rv[kUU], wv[kUU];
+        int64_t f[kUU];
+#pragma unroll
+        for (int u = 0; u < kUU; ++u) {
+            const int64_t c = p + (int64_t)u * stride;
+            f[u] = face((unsigned)c);
+            dv[u] = d[c];
+            qv[u] = q[c];
+            rv[u] = r[c];
+            wv[u] = w[c];
+            xv[u] = x[f[u]];
+        }
+#pragma unroll
+        for (int u = 0; u < kUU; ++u) {
+            x[f[u]] = fma(alpha, dv[u], xv[u]);
+            rv[u] = fma(-alpha, qv[u], rv[u]);
+            r[p + (int64_t)u * stride] = rv[u];
+            one(rv[u], wv[u]);
+        }
+    }
+    for (; p < n; p += stride) {
+        const int64_t f = face((unsigned)p);
         x[f] = fma(alpha, d[p], x[f]);
         const double rp = fma(-alpha, q[p], r[p]);
-        const double zp = rp / helm_diag(g, pos, 1.0 / (tau * nu[f]));
         r[p] = rp;
-        z[p] = zp;
-        l2 = fma(rp, rp, l2);
-        mx = fmax(mx, fabs(rp));
-        rz = fma(rp, zp, rz);
-        nf += isfinite(rp) ? 0u : 1u;
+        one(rp, w[p]);
     }
-    double acc[4] = {l2, mx, (double)nf, rz};
-    const int op[4] = {0, 1, 0, 0};
-    block_reduce_store<4>(acc, op, partials, blockIdx.x, threadIdx.x);
+    block_reduce_sums_kc<2>(sums, rk, nf, partials, blockIdx.x, threadIdx.x);
     finalize_last_block(partials, gridDim.x, fin, threadIdx.x);
+}
+
+// d = w r + beta d (first: d = w r)
+__global__ void helm_direction_kernel(int64_t n, const Scal* __restrict__ s, const double* __restrict__ w,
+                                      const double* __restrict__ r, double* __restrict__ d, int first) {
+    pdl_wait();
+    const double beta = s->beta;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    for (; p + 3 * stride < n; p += 4 * stride) {  // four unknowns in flight
+        double z[4], dv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            z[u] = w[p + u * stride] * r[p + u * stride];
+            dv[u] = first ? 0.0 : d[p + u * stride];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) d[p + u * stride] = first ? z[u] : fma(beta, dv[u], z[u]);
+    }
+    for (; p < n; p += stride) {
+        const double z = w[p] * r[p];
+        d[p] = first ? z : fma(beta, d[p], z);
+    }
 }
 
 // nu_f = (mu_L + mu_R) / (rho_L + rho_R) on every face of the component,
@@ -235,41 +359,61 @@ HelmGeo helm_geo(const Geo& g0, int comp, double h) {
 int64_t helm_unknowns(const HelmGeo& g) { return (int64_t)g.m[0] * g.m[1] * g.m[2]; }
 int64_t helm_faces(const HelmGeo& g) { return (int64_t)g.e[0] * g.e[1] * g.e[2]; }
 
-int64_t launch_helm_init(const HelmGeo& g, const double* un, const double* nu, double tau, double* us,
-                         double* partials, cudaStream_t st, FinSpec fin) {
-    const int64_t n = helm_unknowns(g);
-    const int nb = elementwise_blocks(n);
-    helm_init_kernel<<<nb, kRedThreads, 0, st>>>(g, n, un, nu, tau, us, partials, fin);
-    count_launch();
-    return nb;
+// grid of the marching kernels; zper: planes per block
+static dim3 helm_grid(const HelmGeo& g, int& zper) {
+    const int tx = (g.m[0] + kTX - 1) / kTX, ty = (g.m[1] + kTY - 1) / kTY;
+    zper = march_planes((int64_t)tx * ty, g.m[2], kPerSM);
+    return dim3(tx, ty, (g.m[2] + zper - 1) / zper);
 }
 
-int64_t launch_helm_residual(const HelmGeo& g, const double* un, const double* nu, double tau, const double* x,
-                             double* r, double* z, double* partials, cudaStream_t st, FinSpec fin) {
-    const int64_t n = helm_unknowns(g);
-    const int nb = elementwise_blocks(n);
-    helm_residual_kernel<<<nb, kRedThreads, 0, st>>>(g, n, un, nu, tau, x, r, z, partials, fin);
+void launch_helm_init(const HelmGeo& g, const double* un, const double* nu, double tau, double* sig, double* w,
+                      double* us, double* partials, cudaStream_t st, FinSpec fin) {
+    int zper;
+    const dim3 gr = helm_grid(g, zper);
+    helm_init_kernel<<<gr, dim3(kTX, kTY), 0, st>>>(g, un, nu, tau, sig, w, us, partials, zper, fin);
     count_launch();
-    return nb;
+    launch_helm_wall_zero(g, us, st);
 }
 
-int64_t launch_helm_matvec_dot(const HelmGeo& g, const double* nu, double tau, const double* d, double* q,
-                               double* partials, cudaStream_t st, FinSpec fin) {
-    const int64_t n = helm_unknowns(g);
-    const int nb = elementwise_blocks(n);
-    helm_matvec_dot_kernel<<<nb, kRedThreads, 0, st>>>(g, n, nu, tau, d, q, partials, fin);
+void launch_helm_wall_zero(const HelmGeo& g, double* us, cudaStream_t st) {
+    if (!g.wall) return;
+    const int c = g.comp, a1 = c == 0 ? 1 : 0, a2 = c == 2 ? 1 : 2;
+    const int64_t n = 2 * (int64_t)g.e[a1] * g.e[a2];
+    helm_wall_zero_kernel<<<elementwise_blocks(n), kRedThreads, 0, st>>>(g, us);
     count_launch();
-    return nb;
 }
 
-int64_t launch_helm_update(const HelmGeo& g, const double* nu, double tau, const Scal* s, const double* d,
-                           const double* q, double* x, double* r, double* z, double* partials, cudaStream_t st,
-                           FinSpec fin) {
-    const int64_t n = helm_unknowns(g);
-    const int nb = elementwise_blocks(n);
-    helm_update_kernel<<<nb, kRedThreads, 0, st>>>(g, n, nu, tau, s, d, q, x, r, z, partials, fin);
+void launch_helm_residual(const HelmGeo& g, const double* un, const double* sig, const double* w, const double* x,
+                          double* r, double* partials, cudaStream_t st, FinSpec fin) {
+    int zper;
+    const dim3 gr = helm_grid(g, zper);
+    helm_residual_kernel<<<gr, dim3(kTX, kTY), 0, st>>>(g, un, sig, w, x, r, partials, zper, fin);
     count_launch();
-    return nb;
+}
+
+void launch_helm_matvec_dot(const HelmGeo& g, const double* sig, const double* d, double* q, double* partials,
+                            cudaStream_t st, FinSpec fin) {
+    int zper;
+    const dim3 gr = helm_grid(g, zper);
+    launch_pdl(helm_matvec_dot_kernel, gr, dim3(kTX, kTY), 0, st, g, sig, d, q, partials, zper, fin);
+    count_launch();
+}
+
+void launch_helm_update(const HelmGeo& g, const double* w, const Scal* s, const double* d, const double* q,
+                        double* x, double* r, double* partials, cudaStream_t st, FinSpec fin) {
+    const int64_t n = helm_unknowns(g);
+    int64_t nb = (n + kRedThreads * kUU - 1) / (kRedThreads * kUU);
+    nb = std::max<int64_t>(1, std::min<int64_t>(nb, (int64_t)device_sms() * kPerSM));
+    auto mul = [](int m) { return (unsigned)(0x100000000ull / (unsigned)m + 1); };
+    launch_pdl(helm_update_kernel, (unsigned)nb, kRedThreads, 0, st, g, (unsigned)n, mul(g.m[0]), mul(g.m[1]), w, s, d,
+               q, x, r, partials, fin);
+    count_launch();
+}
+
+void launch_helm_direction(int64_t n, const Scal* s, const double* w, const double* r, double* d, bool first,
+                           cudaStream_t st) {
+    launch_pdl(helm_direction_kernel, elementwise_blocks(n), kRedThreads, 0, st, n, s, w, r, d, first ? 1 : 0);
+    count_launch();
 }
 
 void launch_helm_face_nu(const HelmGeo& g, const Geo& g0, const double* C, double mu1, double mu2, double rho1,
