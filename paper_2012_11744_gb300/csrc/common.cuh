@@ -296,77 +296,41 @@ __device__ inline double warp_max(double v) {
     return v;
 }
 
+// Block reductions.  FP64 runs at 1/64 of the FP32 rate on this GPU, and a
+// shuffle tree in every warp is 45 FP64 warp instructions a value: three
+// values took 6500 cycles of an SM's FP64 pipe at three blocks per SM.  So
+// the threads' values go through shared memory and one warp per value adds
+// the eight warps' lanes up and shuffles: 12 FP64 warp instructions.  The
+// order is fixed by the thread layout.
+
 // Reduce NV values over a block of kRedThreads threads (ops: 0 = sum,
-// 1 = max) in a fixed order and store them as this block's partials at
-// partials[NV*block + q].  Deterministic: the order depends only on the
-// thread layout.
+// 1 = max of values >= 0) and store them as this block's partials at
+// partials[NV*block + q] (written by lane 0 of warp q; the block's fence and
+// ticket follow in finalize_last_block).
 template <int NV>
 __device__ inline void block_reduce_store(double (&v)[NV], const int (&op)[NV], double* partials,
                                           int64_t block, int tid) {
-    __shared__ double sh[kRedThreads / 32][NV];
+    constexpr int kWarps = kRedThreads / 32;
+    static_assert(NV <= kWarps, "one warp per value");
+    __shared__ double sh[NV][kRedThreads];
     const int lane = tid & 31, wid = tid >> 5;
 #pragma unroll
-    for (int q = 0; q < NV; ++q) v[q] = op[q] ? warp_max(v[q]) : warp_sum(v[q]);
-    if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < NV; ++q) sh[wid][q] = v[q];
-    }
+    for (int q = 0; q < NV; ++q) sh[q][tid] = v[q];
     __syncthreads();
-    if (wid == 0) {
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            double t = lane < kRedThreads / 32 ? sh[lane][q] : (op[q] ? 0.0 : 0.0);
-            t = op[q] ? warp_max(t) : warp_sum(t);
-            if (lane == 0) partials[NV * block + q] = t;
-        }
-    }
-}
-
-// Block reduction of one sum, one magnitude key (max) and one count, stored as
-// the three partials (sum, key_value(max), count) of this block.  Keys and
-// counts are reduced with integer warp reductions and an FP32 sum with FP32
-// shuffles, so only the sum of type S uses that type's pipe; fixed order.
-template <typename S>
-__device__ inline void block_reduce_skc(S sum, unsigned long long key, unsigned cnt, double* partials,
-                                        int64_t block, int tid) {
-    __shared__ double sh_s[kRedThreads / 32];
-    __shared__ unsigned long long sh_k[kRedThreads / 32];
-    __shared__ unsigned sh_c[kRedThreads / 32];
-    const unsigned all = 0xffffffffu;
-    const int lane = tid & 31, wid = tid >> 5;
+    for (int q = 0; q < NV; ++q) {
+        if (wid != q) continue;
+        double t = sh[q][lane];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(all, sum, o);
-    const unsigned khi = __reduce_max_sync(all, (unsigned)(key >> 32));
-    const unsigned klo = __reduce_max_sync(all, (unsigned)(key >> 32) == khi ? (unsigned)key : 0u);
-    cnt = __reduce_add_sync(all, cnt);
-    if (lane == 0) {
-        sh_s[wid] = (double)sum;
-        sh_k[wid] = ((unsigned long long)khi << 32) | klo;
-        sh_c[wid] = cnt;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        double ts = 0.0;
-        unsigned long long tk = 0;
-        unsigned tc = 0;
-        for (int w = 0; w < kRedThreads / 32; ++w) {
-            ts += sh_s[w];
-            tk = sh_k[w] > tk ? sh_k[w] : tk;
-            tc += sh_c[w];
-        }
-        partials[3 * block + 0] = ts;
-        partials[3 * block + 1] = key_value(tk);
-        partials[3 * block + 2] = (double)tc;
+        for (int w = 1; w < kWarps; ++w) t = op[q] ? fmax(t, sh[q][32 * w + lane]) : t + sh[q][32 * w + lane];
+        t = op[q] ? warp_max(t) : warp_sum(t);
+        if (lane == 0) partials[NV * block + q] = t;
     }
 }
 
 // Block reduction of NS FP64 sums, one magnitude key (max) and one count,
 // stored as the NS + 2 partials (first sum, key_value(max), count, further
-// sums) of this block.  The threads' sums go through shared memory to one
-// warp, which adds the warps' lanes up and shuffles: 12 FP64 warp
-// instructions a sum instead of the 40 of a shuffle tree in every warp, which
-// on this GPU (FP64 at 1/64 of the FP32 rate) took as long as a quarter of the
-// work of a block of the viscous kernels.  Fixed order.
+// sums) of this block.
 template <int NS>
 __device__ inline void block_reduce_sums_kc(const double (&sum)[NS], unsigned long long key, unsigned cnt,
                                             double* partials, int64_t block, int tid) {
@@ -413,17 +377,46 @@ __device__ inline void block_reduce_sums_kc(const double (&sum)[NS], unsigned lo
     }
 }
 
-// Block reduction of one FP64 sum, the block's only partial (as above).
-__device__ inline void block_reduce_sum(double sum, double* partials, int64_t block, int tid) {
-    __shared__ double sh[kRedThreads];
-    sh[tid] = sum;
-    __syncthreads();
-    if (tid >= 32) return;
-    double t = sh[tid];
+// One sum of type S, one magnitude key and one count, stored as the three
+// partials (sum, key_value(max), count): an FP32 sum by FP32 shuffles within
+// the warps, an FP64 one as above.
+template <typename S>
+__device__ inline void block_reduce_skc(S sum, unsigned long long key, unsigned cnt, double* partials,
+                                        int64_t block, int tid) {
+    if constexpr (sizeof(S) == 8) {
+        const double one[1] = {sum};
+        block_reduce_sums_kc<1>(one, key, cnt, partials, block, tid);
+    } else {
+        __shared__ double sh_s[kRedThreads / 32];
+        __shared__ unsigned long long sh_k[kRedThreads / 32];
+        __shared__ unsigned sh_c[kRedThreads / 32];
+        const unsigned all = 0xffffffffu;
+        const int lane = tid & 31, wid = tid >> 5;
 #pragma unroll
-    for (int w = 1; w < kRedThreads / 32; ++w) t += sh[32 * w + tid];
-    t = warp_sum(t);
-    if (tid == 0) partials[block] = t;
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(all, sum, o);
+        const unsigned khi = __reduce_max_sync(all, (unsigned)(key >> 32));
+        const unsigned klo = __reduce_max_sync(all, (unsigned)(key >> 32) == khi ? (unsigned)key : 0u);
+        cnt = __reduce_add_sync(all, cnt);
+        if (lane == 0) {
+            sh_s[wid] = (double)sum;
+            sh_k[wid] = ((unsigned long long)khi << 32) | klo;
+            sh_c[wid] = cnt;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            double ts = 0.0;
+            unsigned long long tk = 0;
+            unsigned tc = 0;
+            for (int w = 0; w < kRedThreads / 32; ++w) {
+                ts += sh_s[w];
+                tk = sh_k[w] > tk ? sh_k[w] : tk;
+                tc += sh_c[w];
+            }
+            partials[3 * block + 0] = ts;
+            partials[3 * block + 1] = key_value(tk);
+            partials[3 * block + 2] = (double)tc;
+        }
+    }
 }
 
 }  // namespace paris

@@ -77,6 +77,14 @@ inline dim3 tile_grid(const Geo& g, int zper) {
     return dim3((g.nx + kTX - 1) / kTX, (g.ny + kTY - 1) / kTY, (g.nz + zper - 1) / zper);
 }
 
+// the same grid with march_planes' planes per block (zper)
+inline dim3 march_grid(const Geo& g, int per_sm, int& zper) {
+    dim3 gr = tile_grid(g, 1);
+    zper = march_planes((int64_t)gr.x * gr.y, g.nz, per_sm);
+    gr.z = (g.nz + zper - 1) / zper;
+    return gr;
+}
+
 inline int64_t nblocks_of(dim3 gr) { return (int64_t)gr.x * gr.y * gr.z; }
 
 __device__ inline int64_t flat_block() {
@@ -182,7 +190,9 @@ void finalize(const double* partials, int64_t nblocks, int nv, int maxmask, Scal
 
 // ------------------------------------------------------- face coefficients ---
 
-constexpr int kFSeg = 16;  // planes per thread of the face-coefficient kernel
+// resident blocks per SM of the marching kernels (their registers): the face
+// coefficients, with the forcing, the divergence, the FP64 residual, the products
+constexpr int kPerFace = 5, kPerForce = 4, kPerDiv = 6, kPerRes = 4, kPerMat = 6;
 
 // Eq. muH: rho = rho1 C + rho2 (1 - C); beta_f = 1/rho_f with rho_f the mean
 // of the two cells (the paper's "interpolation of 1/rho" read as the mean of
@@ -218,7 +228,7 @@ __global__ void __launch_bounds__(kTX* kTY) face_coeffs_kernel(Geo g, const doub
                                                               double* __restrict__ by,
                                                               double* __restrict__ bz,
                                                               float* __restrict__ rh32,
-                                                              float2* __restrict__ rh2, ForceArgs fa) {
+                                                              float2* __restrict__ rh2, ForceArgs fa, int zper) {
     __shared__ double sh[2][kTY + 1][kTX + 1];  // [plane parity][1 + row][1 + column]
     __shared__ double shc[FORCE ? 2 : 1][kTY + 1][kTX + 1];  // C (FORCE)
     __shared__ double shk[FORCE ? 2 : 1][kTY + 1][kTX + 1];  // kappa (FORCE)
@@ -227,7 +237,7 @@ __global__ void __launch_bounds__(kTX* kTY) face_coeffs_kernel(Geo g, const doub
     const int i = blockIdx.x * kTX + tx, j = blockIdx.y * kTY + ty;
     const bool in = i < nx && j < ny;
     const int ic = min(i, nx - 1), jc = min(j, ny - 1);  // idle threads shadow a cell
-    const int kb = blockIdx.z * kFSeg, ke = min(kb + kFSeg, nz);
+    const int kb = blockIdx.z * zper, ke = min(kb + zper, nz);
     const int64_t pl = (int64_t)nx * ny;
     auto rho = [&](double c) { return fma(r1h, c, r2h * (1.0 - c)); };
     auto kap = [&](int64_t c) { return fa.kappa ? fa.kappa[c] : 0.0; };
@@ -358,14 +368,14 @@ __global__ void __launch_bounds__(kTX* kTY) face_coeffs_fast_kernel(Geo g, const
                                                                    double* __restrict__ bz,
                                                                    float* __restrict__ rh32,
                                                                    float2* __restrict__ rh2,
-                                                                   __half* __restrict__ rh16) {
+                                                                   __half* __restrict__ rh16, int zper) {
     __shared__ float2 sh[2][kTY + 1][kTX + 1];  // [plane parity][1 + row][1 + column]
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int nx = g.nx, ny = g.ny, nz = g.nz;
     const int i = blockIdx.x * kTX + tx, j = blockIdx.y * kTY + ty;
     const bool in = i < nx && j < ny;
     const int ic = min(i, nx - 1), jc = min(j, ny - 1);  // idle threads shadow a cell
-    const int kb = blockIdx.z * kFSeg, ke = min(kb + kFSeg, nz);
+    const int kb = blockIdx.z * zper, ke = min(kb + zper, nz);
     const int64_t pl = (int64_t)nx * ny;
     auto pair = [&](double c) {
         const double rh = fma(d12h, c, r2h);
@@ -406,24 +416,26 @@ __global__ void __launch_bounds__(kTX* kTY) face_coeffs_fast_kernel(Geo g, const
 
 void launch_face_coeffs_fast(const Geo& g, const double* C, double rho1, double rho2, double* bx, double* by,
                              double* bz, float* rh32, float2* rh2, __half* rh16, cudaStream_t st) {
-    dim3 gr((g.nx + kTX - 1) / kTX, (g.ny + kTY - 1) / kTY, (g.nz + kFSeg - 1) / kFSeg);
+    int zper;
+    const dim3 gr = march_grid(g, kPerFace, zper);
     face_coeffs_fast_kernel<<<gr, dim3(kTX, kTY), 0, st>>>(g, C, 0.5 * rho1 - 0.5 * rho2, 0.5 * rho2, bx, by, bz,
-                                                           rh32, rh2, rh16);
+                                                           rh32, rh2, rh16, zper);
     count_launch();
 }
 
 void launch_face_coeffs(const Geo& g, const double* C, double rho1, double rho2, double* bx,
                         double* by, double* bz, float* rh32, float2* rh2, cudaStream_t st,
                         const Forcing* force) {
-    dim3 gr((g.nx + kTX - 1) / kTX, (g.ny + kTY - 1) / kTY, (g.nz + kFSeg - 1) / kFSeg);
+    int zper;
+    const dim3 gr = march_grid(g, force ? kPerForce : kPerFace, zper);
     if (force) {
         ForceArgs fa{force->kappa, force->sigma / force->h, {force->g[0], force->g[1], force->g[2]},
                      force->tau, {force->u[0], force->u[1], force->u[2]}};
         face_coeffs_kernel<true><<<gr, dim3(kTX, kTY), 0, st>>>(g, C, 0.5 * rho1, 0.5 * rho2, bx, by, bz, rh32,
-                                                                rh2, fa);
+                                                                rh2, fa, zper);
     } else {
         face_coeffs_kernel<false><<<gr, dim3(kTX, kTY), 0, st>>>(g, C, 0.5 * rho1, 0.5 * rho2, bx, by, bz, rh32,
-                                                                 rh2, ForceArgs{});
+                                                                 rh2, ForceArgs{}, zper);
     }
     count_launch();
 }
@@ -450,14 +462,14 @@ __global__ void __launch_bounds__(kTX* kTY) divergence_kernel(Geo g, const doubl
                                                               const double* __restrict__ w,
                                                               double inv_hdt,
                                                               double* __restrict__ rhs,
-                                                              double* partials, FinSpec fin) {
+                                                              double* partials, int zper, FinSpec fin) {
     const int i = blockIdx.x * kTX + threadIdx.x;
     const int j = blockIdx.y * kTY + threadIdx.y;
     double sum = 0.0;
     unsigned long long bmax_k = 0;
     unsigned nf = 0;
     if (i < g.nx && j < g.ny) {
-        const int k0 = blockIdx.z * kZ, k1 = min(k0 + kZ, g.nz);
+        const int k0 = blockIdx.z * zper, k1 = min(k0 + zper, g.nz);
         PARIS_ZLOOP(k0, k1, {
             const double b = cell_div(g, u, v, w, i, j, k) * inv_hdt;
             rhs[g.cidx(i, j, k)] = b;
@@ -473,8 +485,9 @@ __global__ void __launch_bounds__(kTX* kTY) divergence_kernel(Geo g, const doubl
 
 int64_t launch_divergence(const Geo& g, const double* u, const double* v, const double* w,
                           double inv_hdt, double* rhs, double* partials, cudaStream_t st, FinSpec fin) {
-    dim3 gr = tile_grid(g, kZ);
-    divergence_kernel<<<gr, dim3(kTX, kTY), 0, st>>>(g, u, v, w, inv_hdt, rhs, partials, fin);
+    int zper;
+    const dim3 gr = march_grid(g, kPerDiv, zper);
+    divergence_kernel<<<gr, dim3(kTX, kTY), 0, st>>>(g, u, v, w, inv_hdt, rhs, partials, zper, fin);
     count_launch();
     return nblocks_of(gr);
 }
@@ -1341,7 +1354,7 @@ __global__ void __launch_bounds__(kTX* kTY) residual64_kernel(Geo g, Coef<double
                                                               double* __restrict__ r64,
                                                               float* __restrict__ r32,
                                                               const Scal* s, double* partials,
-                                                              int zero_ok, int split, FinSpec fin) {
+                                                              int zero_ok, int split, int zper, FinSpec fin) {
     pdl_wait();
     const int i = blockIdx.x * kTX + threadIdx.x;
     const int j = blockIdx.y * kTY + threadIdx.y;
@@ -1351,7 +1364,7 @@ __global__ void __launch_bounds__(kTX* kTY) residual64_kernel(Geo g, Coef<double
     if (i < g.nx && j < g.ny) {
         const int se = r32 ? (int)s->scale_exp : 0;
         const bool zero = zero_ok && s->xmax == 0.0;
-        const int k0 = blockIdx.z * kZ, k1 = min(k0 + kZ, g.nz);
+        const int k0 = blockIdx.z * zper, k1 = min(k0 + zper, g.nz);
         PARIS_ZLOOP(k0, k1, {
             int64_t c;
             double r;
@@ -1396,11 +1409,12 @@ __global__ void __launch_bounds__(kTX* kTY) residual64_kernel(Geo g, Coef<double
 int64_t launch_residual64(const Geo& g, const Coef<double>& cf, const double* f, const double* x,
                           double* r64, float* r32, const Scal* s, double* partials, bool zero_ok,
                           cudaStream_t st, FinSpec fin, bool split) {
-    dim3 gr = tile_grid(g, kZ);
+    int zper;
+    const dim3 gr = march_grid(g, kPerRes, zper);
     auto* k = fits_i32(g) ? (cf.sig ? residual64_kernel<true, true> : residual64_kernel<true>)
                           : (cf.sig ? residual64_kernel<false, true> : residual64_kernel<false>);
     launch_pdl(k, gr, dim3(kTX, kTY), 0, st, g, cf, f, x, r64, r32, s, partials, zero_ok ? 1 : 0, split ? 1 : 0,
-               fin);
+               zper, fin);
     count_launch();
     return nblocks_of(gr);
 }
@@ -1411,12 +1425,13 @@ template <typename T, bool I32, bool SIG = false>
 __global__ void __launch_bounds__(kTX* kTY) matvec_dot_kernel(Geo g, Coef<T> cf,
                                                              const T* __restrict__ d,
                                                              T* __restrict__ q,
-                                                             double* partials, FinSpec fin) {
+                                                             double* partials, int zper, FinSpec fin) {
+    pdl_wait();
     const int i = blockIdx.x * kTX + threadIdx.x;
     const int j = blockIdx.y * kTY + threadIdx.y;
     T loc = T(0);
     if (i < g.nx && j < g.ny) {
-        const int k0 = blockIdx.z * kZ, k1 = min(k0 + kZ, g.nz);
+        const int k0 = blockIdx.z * zper, k1 = min(k0 + zper, g.nz);
         PARIS_ZLOOP(k0, k1, {
             Stencil<T> st;
             int64_t c;
@@ -1444,10 +1459,11 @@ __global__ void __launch_bounds__(kTX* kTY) matvec_dot_kernel(Geo g, Coef<T> cf,
 template <typename T>
 int64_t launch_matvec_dot(const Geo& g, const Coef<T>& cf, const T* d, T* q, double* partials,
                           cudaStream_t st, FinSpec fin) {
-    dim3 gr = tile_grid(g, kZ);
+    int zper;
+    const dim3 gr = march_grid(g, kPerMat, zper);
     auto* k = fits_i32(g) ? (cf.sig ? matvec_dot_kernel<T, true, true> : matvec_dot_kernel<T, true>)
                           : (cf.sig ? matvec_dot_kernel<T, false, true> : matvec_dot_kernel<T, false>);
-    k<<<gr, dim3(kTX, kTY), 0, st>>>(g, cf, d, q, partials, fin);
+    launch_pdl(k, gr, dim3(kTX, kTY), 0, st, g, cf, d, q, partials, zper, fin);
     count_launch();
     return nblocks_of(gr);
 }

@@ -22,7 +22,7 @@ namespace paris {
 
 namespace {
 
-constexpr int kTX = 32, kTY = 8, kZ = 16;  // 16 cells per thread along z
+constexpr int kTX = 32, kTY = 8, kPerSM = 5;  // tile, resident blocks per SM (48 registers)
 
 struct F2 {
     float hi, lo;
@@ -77,13 +77,14 @@ __device__ __forceinline__ void face_term(float2 rc, float2 rq, float ec, float 
 // r_new may be the same array (each cell reads and writes only its own r).
 // rh2 holds rho/2 per cell as (hi, lo) FP32 pairs.  The squared norm of r is
 // accumulated from the O(1)-scaled r32 in FP32 and unscaled in the finalize.
-__global__ void __launch_bounds__(kTX* kTY) refine_rho_kernel(Geo g, const float2* __restrict__ rh2,
+__global__ void __launch_bounds__(kTX* kTY, kPerSM) refine_rho_kernel(Geo g, const float2* __restrict__ rh2,
                                                             float ih2_hi, float ih2_lo,
                                                             const float* __restrict__ e,
                                                             const double* r_old, double* r_new,
                                                             double* __restrict__ x, float* __restrict__ r32,
                                                             const Scal* s, double* partials, FinSpec fin, int rev,
-                                                            int emem, const float* __restrict__ dpend) {
+                                                            int emem, const float* __restrict__ dpend,
+                                                            int zper) {
     pdl_wait();
     const int zb = rev ? (int)(gridDim.z - 1 - blockIdx.z) : (int)blockIdx.z;  // rev: descending plane chunks
     const int i = blockIdx.x * kTX + threadIdx.x;
@@ -115,7 +116,7 @@ __global__ void __launch_bounds__(kTX* kTY) refine_rho_kernel(Geo g, const float
         const int hx = nx / 2;
         const int tx = i >> 1;
         const int txm = (xlo ? nx - 1 : i - 1) >> 1, txp = (xhi ? 0 : i + 1) >> 1;
-        const int k0 = zb * kZ, k1 = min(k0 + kZ, nz);
+        const int k0 = zb * zper, k1 = min(k0 + zper, nz);
         for (int k = k0; k < k1; ++k) {
             const int c = (k * ny + j) * nx + i;
             const bool zlo = k == 0, zhi = k == nz - 1;
@@ -168,9 +169,11 @@ void launch_refine_rho(const Geo& g, const float2* rh2, double h, const float* e
     const double ih2d = 1.0 / (h * h);
     const float hi = (float)ih2d;
     const float lo = (float)(ih2d - (double)hi);
-    dim3 gr((g.nx + kTX - 1) / kTX, (g.ny + kTY - 1) / kTY, (g.nz + kZ - 1) / kZ);
+    const int tx = (g.nx + kTX - 1) / kTX, ty = (g.ny + kTY - 1) / kTY;
+    const int zper = march_planes((int64_t)tx * ty, g.nz, kPerSM);
+    const dim3 gr(tx, ty, (g.nz + zper - 1) / zper);
     launch_pdl(refine_rho_kernel, gr, dim3(kTX, kTY), 0, st, g, rh2, hi, lo, e, r_old, r_new, x, r32, s,
-        partials, FinSpec{s, 3, 2, FIN_REFINE, 0.0}, rev ? 1 : 0, emem ? 1 : 0, dpend);
+        partials, FinSpec{s, 3, 2, FIN_REFINE, 0.0}, rev ? 1 : 0, emem ? 1 : 0, dpend, zper);
     count_launch();
 }
 

@@ -1410,31 +1410,32 @@ __global__ void __launch_bounds__(kBX* VB, RESTRICT ? PARIS_OP_MINB_R * kVY / VB
     }
 }
 
-#ifndef PARIS_OP_PLANES
-#define PARIS_OP_PLANES 16
-#endif
-// planes per block of the tile product: 16 measured 98 us a launch against 102
-// with 8 and 121 with 2
-constexpr int kTileOpPlanes = PARIS_OP_PLANES;
-
 int64_t rho0_matvec_blocks(const Geo& g) {
-    // the most blocks any segment length (>= 2 planes) gives, or the plane tiles
+    // the most blocks any segment length (>= 2 planes) gives, or the plane tiles at kMinMarch planes
     const int64_t ring = (int64_t)pair_blocks_x(g) * ((g.ny + kVY - 1) / kVY) * ((g.nz + 1) / 2);
     const int64_t tiles = (int64_t)((g.nx / 2 + 2 * kBX - 1) / (2 * kBX)) * ((g.ny + kVY - 1) / kVY) *
-                          ((g.nz + kTileOpPlanes - 1) / kTileOpPlanes);
+                          ((g.nz + kMinMarch - 1) / kMinMarch);
     return ring > tiles ? ring : tiles;
 }
 
 bool rho0_product_fuses(const Geo& g, bool tiles) { return tiles && kTileOpV > 0 && (g.nx / 2) % kTileOpV == 0; }
+
+// grid of the tile product; np: planes per block
+static dim3 product_grid(int tx, const Geo& g, int& np) {
+    const int ty = (g.ny + kVY - 1) / kVY;
+    np = march_planes((int64_t)tx * ty, g.nz, PARIS_OP_MINB);
+    return dim3(tx, ty, (g.nz + np - 1) / np);
+}
 
 int64_t launch_matvec_rho_xpby(const Geo& g, const float* rh, double h, const float* z, const float* d, float* dnew,
                                float* q, const Scal* s, double* partials, cudaStream_t st, FinSpec fin, bool rev,
                                float* e, bool emem) {
     constexpr int V = kTileOpV > 0 ? kTileOpV : 2;
     const int hx = g.nx / 2;
-    dim3 gr((hx / V + kBX - 1) / kBX, (g.ny + kVY - 1) / kVY, (g.nz + kTileOpPlanes - 1) / kTileOpPlanes);
+    int np;
+    const dim3 gr = product_grid((hx / V + kBX - 1) / kBX, g, np);
     launch_pdl(op_rho_tile_kernel<false, V, true>, gr, dim3(kBX, kVY), 0, st, g, rh, (float)(1.0 / (h * h)), d,
-               (const float*)nullptr, q, g, partials, kTileOpPlanes, fin, z, s, dnew, rev ? 1 : 0, e, emem ? 1 : 0);
+               (const float*)nullptr, q, g, partials, np, fin, z, s, dnew, rev ? 1 : 0, e, emem ? 1 : 0);
     count_launch();
     return (int64_t)gr.x * gr.y * gr.z;
 }
@@ -1444,9 +1445,10 @@ int64_t launch_matvec_rho(const Geo& g, const float* rh, double h, const float* 
     const int hx = g.nx / 2;
     if (tiles && kTileOpV > 0 && hx % kTileOpV == 0) {
         constexpr int V = kTileOpV > 0 ? kTileOpV : 2;
-        dim3 gr((hx / V + kBX - 1) / kBX, (g.ny + kVY - 1) / kVY, (g.nz + kTileOpPlanes - 1) / kTileOpPlanes);
+        int np;
+        const dim3 gr = product_grid((hx / V + kBX - 1) / kBX, g, np);
         launch_pdl(op_rho_tile_kernel<false, V>, gr, dim3(kBX, kVY), 0, st, g, rh, (float)(1.0 / (h * h)), d,
-            (const float*)nullptr, q, g, partials, kTileOpPlanes, fin, (const float*)nullptr, (const Scal*)nullptr,
+            (const float*)nullptr, q, g, partials, np, fin, (const float*)nullptr, (const Scal*)nullptr,
             (float*)nullptr, rev ? 1 : 0, (float*)nullptr, 0);
         count_launch();
         return (int64_t)gr.x * gr.y * gr.z;

@@ -207,7 +207,9 @@ __global__ void __launch_bounds__(kTX* kTY, kPerSM) helm_matvec_dot_kernel(HelmG
             dq = fma(dc, qp, dq);
         }
     }
-    block_reduce_sum(dq, partials, helm_block(), tid);
+    double acc[1] = {dq};
+    const int op[1] = {0};
+    block_reduce_store<1>(acc, op, partials, helm_block(), tid);
     finalize_last_block(partials, helm_blocks(), fin, tid);
 }
 
