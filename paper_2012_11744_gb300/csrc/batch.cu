@@ -32,7 +32,11 @@
 namespace paris {
 namespace batch {
 
-constexpr int kBT = 256;     // threads per CTA
+// Threads per CTA, two CTAs per SM.  The kernel waits on memory latency, so it
+// wants warps and bytes in flight per thread, and no spills: 384 threads at
+// the 85 registers that leaves run 64 instances (20 M cells) in 17.9 ms, 256 in
+// 18.6, 512 in 19.9 (spilling); at 4 to 16 instances 256 are 6 to 8 % faster.
+constexpr int kBT = 384;
 constexpr int kMaxLev = 12;  // multigrid levels per instance
 constexpr int kMaxDense = 128;
 
@@ -42,6 +46,7 @@ struct BLevel {
     float* b[3];  // coefficients beta/h_a^2 of this level
     float* x;     // level solution (level 0: the V-cycle output)
     float* f;     // level right-hand side (level 0: the V-cycle input)
+    unsigned mx, my, mp, mq;  // fast_div multipliers of nx, ny, the pairs and the quads of a row
 };
 
 struct BInst {
@@ -56,7 +61,7 @@ struct BInst {
     float *r, *z, *d, *q, *e;
     double* cinv;  // dense inverse of the regularised coarsest operator
     int cta0, ncta;
-    unsigned* bar;  // group barrier: [0] arrivals, [1] generation
+    unsigned* bar;  // group barrier: [0] arrivals since the launch
     double* part;   // group partials: 2 buffers x ncta x 4
     double* stats;  // 8 values (see write_stats)
 };
@@ -75,74 +80,79 @@ struct Grp {
     int rank, ncta;
     int* err;
     int pb;
+    unsigned arrivals;  // of the whole group up to the last barrier (thread 0)
     long long spin;
 };
 
-__device__ inline bool group_ok(const Grp& c) { return *(volatile int*)c.err == 0; }
-
-// Barrier of the instance's CTAs (bounded spin).  Returns false once any
-// barrier of the launch has timed out, so that every CTA unwinds.
+// Barrier of the instance's CTAs: one release addition to a count that only
+// grows, then acquire polls of it by the same thread (bounded; the first ones
+// without a pause).  Returns false on every thread of a CTA whose wait gave
+// up (the error flag set), so that it unwinds; the others' waits give up in
+// turn.  About 1.5 us; with a count reset by the last arrival, a generation
+// word, fences and the error flag read by every thread after it, it took over
+// 3 (4 instances: 3.15 -> 2.92 ms).
 __device__ bool gbar(Grp& c) {
-    __syncthreads();
-    if (c.ncta > 1) {
-        if (threadIdx.x == 0) {
-            volatile unsigned* gen = c.I->bar + 1;
-            const unsigned g = *gen;
-            __threadfence();
-            const unsigned arrived = atomicAdd(c.I->bar, 1u);
-            if (arrived == (unsigned)c.ncta - 1) {
-                c.I->bar[0] = 0;
-                __threadfence();
-                atomicAdd(c.I->bar + 1, 1u);
-            } else {
-                long long it = 0;
-                while (*gen == g) {
-                    if (++it > c.spin || *(volatile int*)c.err) {
-                        atomicExch(c.err, 1);
-                        break;
-                    }
-                    __nanosleep(64);
-                }
-            }
-            __threadfence();
-        }
+    if (c.ncta == 1) {
         __syncthreads();
+        return true;
     }
-    return group_ok(c);
+    __syncthreads();
+    bool bad = false;
+    if (threadIdx.x == 0) {
+        unsigned* bar = c.I->bar;
+        c.arrivals += (unsigned)c.ncta;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        unsigned seen;
+        for (long long it = 0;; ++it) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+            if ((int)(seen - c.arrivals) >= 0) break;
+            if (it > c.spin || ((it & 1023) == 1023 && *(volatile int*)c.err)) {
+                atomicExch(c.err, 1);
+                bad = true;
+                break;
+            }
+            if (it > 64) __nanosleep(32);
+        }
+    }
+    return !__syncthreads_or(bad);
 }
 
-// Sum (op 0) or max (op 1) of NV values over the instance, identical in all
-// of its CTAs (fixed folding order).
+// Sum (op 0) or max of values >= 0 (op 1) of NV values over the instance,
+// identical in all of its CTAs (fixed folding order).  One warp per value
+// folds the CTA's threads and, after the barrier, the CTAs' partials, 32 at a
+// time (thread by thread the partials took one L2 round trip each).
 template <int NV>
 __device__ bool greduce(Grp& c, double (&v)[NV], const int (&op)[NV]) {
-    __shared__ double sh[kBT / 32][4];
-    __shared__ double res[4];
+    __shared__ double sh[NV][kBT];
+    __shared__ double res[NV];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        double t = op[q] ? warp_max(v[q]) : warp_sum(v[q]);
-        if (lane == 0) sh[wid][q] = t;
-    }
+    for (int q = 0; q < NV; ++q) sh[q][threadIdx.x] = v[q];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int q = 0; q < NV; ++q) {
-            double t = 0.0;
-            for (int w = 0; w < kBT / 32; ++w) t = op[q] ? fmax(t, sh[w][q]) : t + sh[w][q];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        if (wid != q) continue;
+        double t = sh[q][lane];
+#pragma unroll 4
+        for (int w = 1; w < kBT / 32; ++w) t = op[q] ? fmax(t, sh[q][32 * w + lane]) : t + sh[q][32 * w + lane];
+        t = op[q] ? warp_max(t) : warp_sum(t);
+        if (lane == 0) {
             res[q] = t;
             if (c.ncta > 1) c.I->part[((int64_t)c.pb * c.ncta + c.rank) * 4 + q] = t;
         }
     }
     if (c.ncta > 1) {
         if (!gbar(c)) return false;
-        if (threadIdx.x == 0) {
-            for (int q = 0; q < NV; ++q) {
-                double t = 0.0;
-                for (int r = 0; r < c.ncta; ++r) {
-                    const double x = *(volatile double*)&c.I->part[((int64_t)c.pb * c.ncta + r) * 4 + q];
-                    t = op[q] ? fmax(t, x) : t + x;
-                }
-                res[q] = t;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            if (wid != q) continue;
+            double t = 0.0;
+            for (int r = lane; r < c.ncta; r += 32) {
+                const double x = __ldcg(&c.I->part[((int64_t)c.pb * c.ncta + r) * 4 + q]);
+                t = op[q] ? fmax(t, x) : t + x;
             }
+            t = op[q] ? warp_max(t) : warp_sum(t);
+            if (lane == 0) res[q] = t;
         }
         c.pb ^= 1;
     }
@@ -150,82 +160,105 @@ __device__ bool greduce(Grp& c, double (&v)[NV], const int (&op)[NV]) {
 #pragma unroll
     for (int q = 0; q < NV; ++q) v[q] = res[q];
     __syncthreads();
-    return group_ok(c);
+    return true;
 }
 
-#define GLOOP(c_, n_)                                                          \
-    for (int64_t c_ = (int64_t)cx.rank * kBT + threadIdx.x; c_ < (int64_t)(n_); \
-         c_ += (int64_t)cx.ncta * kBT)
+#define GLOOP(c_, n_) \
+    for (int64_t c_ = (int64_t)rank * kBT + threadIdx.x; c_ < (int64_t)(n_); c_ += (int64_t)ncta * kBT)
 
-// cell index -> (i, j, k) in 32-bit arithmetic (an instance has fewer than
-// 2^31 cells and faces, checked at creation)
-__device__ inline void decomp(const Geo& g, int64_t c, int& i, int& j, int& k) {
-    const unsigned cu = (unsigned)c, nx = (unsigned)g.nx, ny = (unsigned)g.ny;
-    const unsigned t = cu / nx;
-    i = (int)(cu - t * nx);
-    k = (int)(t / ny);
-    j = (int)(t - (unsigned)k * ny);
+// cell index of a level -> (i, j, k) in 32-bit arithmetic (an instance has
+// fewer than 2^31 cells and faces, checked at creation)
+__device__ inline void decomp(const Geo& g, unsigned mx, unsigned my, int64_t c, int& i, int& j, int& k) {
+    const unsigned cu = (unsigned)c;
+    const unsigned t = fast_div(cu, (unsigned)g.nx, mx);
+    i = (int)(cu - t * (unsigned)g.nx);
+    k = (int)fast_div(t, (unsigned)g.ny, my);
+    j = (int)(t - (unsigned)k * (unsigned)g.ny);
 }
 
 // ------------------------------------------------------------ set-up ---
 
 // beta_f = 2/(rho_L + rho_R), rho = rho1 C + rho2 (1 - C) (Eq. muH), 0 on walls;
 // FP64 for the residual and the correction, FP32 beta/h^2 for the V-cycle.
-__device__ void setup_coefficients(Grp& cx) {
-    const BInst& I = *cx.I;
-    const Geo& g = I.g0;
+__device__ __noinline__ void setup_coefficients(const BInst& I, int rank, int ncta) {
+    const Geo g = I.g0;
+    const unsigned mx = I.lv[0].mx, my = I.lv[0].my;
+    const double* C = I.C;
+    double* const b64[3] = {I.b64[0], I.b64[1], I.b64[2]};
+    float* const b32[3] = {I.lv[0].b[0], I.lv[0].b[1], I.lv[0].b[2]};
     const double ih2 = 1.0 / (I.h * I.h);
-    auto rho = [&](double cc) { return fma(I.rho1, cc, I.rho2 * (1.0 - cc)); };
+    const double r1h = 0.5 * I.rho1, r2h = 0.5 * I.rho2;  // exact: beta_f = 1/(rho_L/2 + rho_R/2)
+    auto rho = [&](double cc) { return fma(r1h, cc, r2h * (1.0 - cc)); };
     GLOOP(c, g.ncell()) {
         int i, j, k;
-        decomp(g, c, i, j, k);
-        const double rc = rho(I.C[c]);
+        decomp(g, mx, my, c, i, j, k);
+        const double rc = rho(C[c]);
         AxisNb ax = axis_nb(i, g.nx, g.wx), ay = axis_nb(j, g.ny, g.wy), az = axis_nb(k, g.nz, g.wz);
         auto put = [&](int a, int64_t f, bool wall, int64_t left) {
-            const double bt = wall ? 0.0 : 2.0 / (rho(I.C[left]) + rc);
-            I.b64[a][f] = bt;
-            I.lv[0].b[a][f] = (float)(bt * ih2);
+            const double bt = wall ? 0.0 : recip64(rho(C[left]) + rc);
+            b64[a][f] = bt;
+            b32[a][f] = d2f_scaled(bt * ih2, 0);
         };
         put(0, g.fx(i, j, k), ax.wm, g.cidx(ax.m, j, k));
         put(1, g.fy(i, j, k), ay.wm, g.cidx(i, ay.m, k));
         put(2, g.fz(i, j, k), az.wm, g.cidx(i, j, az.m));
-        if (g.wx && i == g.nx - 1) { I.b64[0][g.fx(g.nx, j, k)] = 0.0; I.lv[0].b[0][g.fx(g.nx, j, k)] = 0.f; }
-        if (g.wy && j == g.ny - 1) { I.b64[1][g.fy(i, g.ny, k)] = 0.0; I.lv[0].b[1][g.fy(i, g.ny, k)] = 0.f; }
-        if (g.wz && k == g.nz - 1) { I.b64[2][g.fz(i, j, g.nz)] = 0.0; I.lv[0].b[2][g.fz(i, j, g.nz)] = 0.f; }
+        if (g.wx && i == g.nx - 1) { b64[0][g.fx(g.nx, j, k)] = 0.0; b32[0][g.fx(g.nx, j, k)] = 0.f; }
+        if (g.wy && j == g.ny - 1) { b64[1][g.fy(i, g.ny, k)] = 0.0; b32[1][g.fy(i, g.ny, k)] = 0.f; }
+        if (g.wz && k == g.nz - 1) { b64[2][g.fz(i, j, g.nz)] = 0.0; b32[2][g.fz(i, j, g.nz)] = 0.f; }
     }
 }
 
-// f = -(div u*/dt - mean) and its norms; returns false on error
-__device__ bool setup_rhs(Grp& cx, double& bnorm2, double& binf, double& nonfin) {
-    const BInst& I = *cx.I;
-    const Geo& g = I.g0;
+// out = div u*/dt; returns this thread's part of its sum
+__device__ __noinline__ double divergence(const BInst& I, int rank, int ncta) {
+    const Geo g = I.g0;
+    const unsigned mx = I.lv[0].mx, my = I.lv[0].my;
     const double ihdt = 1.0 / (I.h * I.dt);
-    double acc[1] = {0.0};
+    const double *u = I.u, *v = I.v, *w = I.w;
+    double* out = I.f64;
+    double acc = 0.0;
     GLOOP(c, g.ncell()) {
         int i, j, k;
-        decomp(g, c, i, j, k);
+        decomp(g, mx, my, c, i, j, k);
         AxisNb ax = axis_nb(i, g.nx, g.wx), ay = axis_nb(j, g.ny, g.wy), az = axis_nb(k, g.nz, g.wz);
-        const double up = ax.wp ? 0.0 : I.u[g.fx(ax.fp, j, k)], um = ax.wm ? 0.0 : I.u[g.fx(i, j, k)];
-        const double vp = ay.wp ? 0.0 : I.v[g.fy(i, ay.fp, k)], vm = ay.wm ? 0.0 : I.v[g.fy(i, j, k)];
-        const double wp = az.wp ? 0.0 : I.w[g.fz(i, j, az.fp)], wm = az.wm ? 0.0 : I.w[g.fz(i, j, k)];
+        const double up = ax.wp ? 0.0 : u[g.fx(ax.fp, j, k)], um = ax.wm ? 0.0 : u[g.fx(i, j, k)];
+        const double vp = ay.wp ? 0.0 : v[g.fy(i, ay.fp, k)], vm = ay.wm ? 0.0 : v[g.fy(i, j, k)];
+        const double wp = az.wp ? 0.0 : w[g.fz(i, j, az.fp)], wm = az.wm ? 0.0 : w[g.fz(i, j, k)];
         const double b = (((up - um) + (vp - vm)) + (wp - wm)) * ihdt;
-        I.f64[c] = b;
-        acc[0] += b;
+        out[c] = b;
+        acc += b;
     }
+    return acc;
+}
+
+// f = -(div u*/dt - mean), p = 0; this thread's |f|^2, max |f|, non-finite count
+__device__ __noinline__ void rhs_norms(const BInst& I, int rank, int ncta, double mean, double (&n3)[3]) {
+    const int64_t n = I.g0.ncell();
+    double *f = I.f64, *p = I.p;
+    double l2 = 0.0;
+    unsigned nf = 0;
+    unsigned long long mk = 0;  // max |f| as an integer key: no FP64 instruction
+    GLOOP(c, n) {
+        const double t = -(f[c] - mean);
+        f[c] = t;
+        p[c] = 0.0;
+        l2 = fma(t, t, l2);
+        const unsigned long long kt = abs_key(t);
+        mk = kt > mk ? kt : mk;
+        nf += key_nonfinite(kt);
+    }
+    n3[0] = l2;
+    n3[1] = key_value(mk);
+    n3[2] = (double)nf;
+}
+
+// the right-hand side and its norms; returns false on error
+__device__ bool setup_rhs(Grp& cx, double& bnorm2, double& binf, double& nonfin) {
+    const BInst& I = *cx.I;
+    double acc[1] = {divergence(I, cx.rank, cx.ncta)};
     const int op1[1] = {0};
     if (!greduce<1>(cx, acc, op1)) return false;
-    const double mean = acc[0] / (double)g.ncell();
-    double n3[3] = {0.0, 0.0, 0.0};
-    unsigned nf = 0;
-    GLOOP(c, g.ncell()) {
-        const double t = -(I.f64[c] - mean);
-        I.f64[c] = t;
-        I.p[c] = 0.0;
-        n3[0] = fma(t, t, n3[0]);
-        n3[1] = fmax(n3[1], fabs(t));
-        nf += isfinite(t) ? 0u : 1u;
-    }
-    n3[2] = (double)nf;
+    double n3[3];
+    rhs_norms(I, cx.rank, cx.ncta, acc[0] / (double)I.g0.ncell(), n3);
     const int op3[3] = {0, 1, 0};
     if (!greduce<3>(cx, n3, op3)) return false;
     bnorm2 = n3[0];
@@ -235,30 +268,32 @@ __device__ bool setup_rhs(Grp& cx, double& bnorm2, double& binf, double& nonfin)
 }
 
 // coarse coefficients: mean of the covering fine faces times (h_f/h_c)^2
+__device__ __noinline__ void coarse_coefficients(const BLevel& F, const BLevel& L, int rank, int ncta) {
+    for (int a = 0; a < 3; ++a) {
+        const int n0 = L.g.nx + (a == 0 ? L.g.wx : 0), n1 = L.g.ny + (a == 1 ? L.g.wy : 0);
+        const int fn0 = F.g.nx + (a == 0 ? F.g.wx : 0), fn1 = F.g.ny + (a == 1 ? F.g.wy : 0);
+        const float ratio = 1.0f / (float)(L.fac[a] * L.fac[a]);
+        GLOOP(t, L.g.nface(a)) {
+            const int C3[3] = {(int)(t % n0), (int)((t / n0) % n1), (int)(t / ((int64_t)n0 * n1))};
+            int lo[3], cnt[3];
+            for (int b = 0; b < 3; ++b) {
+                lo[b] = C3[b] * L.fac[b];
+                cnt[b] = b == a ? 1 : L.fac[b];
+            }
+            float s = 0.f;
+            for (int dk = 0; dk < cnt[2]; ++dk)
+                for (int dj = 0; dj < cnt[1]; ++dj)
+                    for (int di = 0; di < cnt[0]; ++di)
+                        s += F.b[a][((int64_t)(lo[2] + dk) * fn1 + (lo[1] + dj)) * fn0 + (lo[0] + di)];
+            L.b[a][t] = s / (float)(cnt[0] * cnt[1] * cnt[2]) * ratio;
+        }
+    }
+}
+
 __device__ bool setup_levels(Grp& cx) {
     const BInst& I = *cx.I;
     for (int l = 1; l < I.nlev; ++l) {
-        const BLevel& F = I.lv[l - 1];
-        const BLevel& L = I.lv[l];
-        for (int a = 0; a < 3; ++a) {
-            const int n0 = L.g.nx + (a == 0 ? L.g.wx : 0), n1 = L.g.ny + (a == 1 ? L.g.wy : 0);
-            const int fn0 = F.g.nx + (a == 0 ? F.g.wx : 0), fn1 = F.g.ny + (a == 1 ? F.g.wy : 0);
-            const float ratio = 1.0f / (float)(L.fac[a] * L.fac[a]);
-            GLOOP(t, L.g.nface(a)) {
-                const int C3[3] = {(int)(t % n0), (int)((t / n0) % n1), (int)(t / ((int64_t)n0 * n1))};
-                int lo[3], cnt[3];
-                for (int b = 0; b < 3; ++b) {
-                    lo[b] = C3[b] * L.fac[b];
-                    cnt[b] = b == a ? 1 : L.fac[b];
-                }
-                float s = 0.f;
-                for (int dk = 0; dk < cnt[2]; ++dk)
-                    for (int dj = 0; dj < cnt[1]; ++dj)
-                        for (int di = 0; di < cnt[0]; ++di)
-                            s += F.b[a][((int64_t)(lo[2] + dk) * fn1 + (lo[1] + dj)) * fn0 + (lo[0] + di)];
-                L.b[a][t] = s / (float)(cnt[0] * cnt[1] * cnt[2]) * ratio;
-            }
-        }
+        coarse_coefficients(I.lv[l - 1], I.lv[l], cx.rank, cx.ncta);
         if (!gbar(cx)) return false;
     }
     // dense inverse of the coarsest operator (FP64 Gauss-Jordan by the first CTA)
@@ -316,11 +351,11 @@ __device__ bool setup_levels(Grp& cx) {
 struct PassCell {
     int i, j, k, io;
 };
-__device__ inline PassCell pass_cell(const Geo& g, unsigned pp, unsigned npair, int color) {
-    const unsigned ny = (unsigned)g.ny, row = pp / npair;
+__device__ inline PassCell pass_cell(const Geo& g, unsigned pp, unsigned npair, unsigned mp, unsigned my, int color) {
+    const unsigned ny = (unsigned)g.ny, row = fast_div(pp, npair, mp);
     PassCell p;
     const int tp = (int)(pp - row * npair);
-    p.k = (int)(row / ny);
+    p.k = (int)fast_div(row, ny, my);
     p.j = (int)(row - (unsigned)p.k * ny);
     const int i0 = 2 * tp;
     p.i = i0 + ((i0 + p.j + p.k + color) & 1);
@@ -336,12 +371,13 @@ struct PassLoad {
     float f, x, nb[6];
     bool on;
 };
-__device__ __forceinline__ void pass_load(PassLoad& d, const BLevel& L, const float* f, const float* x,
-                                          const PassCell& p, bool zero) {
-    d.on = p.i < L.g.nx;
+__device__ __forceinline__ void pass_load(PassLoad& d, const Geo& g, const float* bx, const float* by,
+                                          const float* bz, const float* f, const float* x, const PassCell& p,
+                                          bool zero) {
+    d.on = p.i < g.nx;
     if (!d.on) return;
     Stencil<float> s;
-    load_stencil_fast(L.g, L.b[0], L.b[1], L.b[2], p.i, p.j, p.k, s, d.c);
+    load_stencil_fast(g, bx, by, bz, p.i, p.j, p.k, s, d.c);
 #pragma unroll
     for (int q = 0; q < 6; ++q) d.b[q] = s.b[q];
     d.f = f[d.c];
@@ -367,136 +403,543 @@ __device__ __forceinline__ void pass_store(const PassLoad& d, const Geo& g, floa
     }
 }
 
+// The colour pass with a thread per four cells of a row marching through
+// up to kQuadPlanes planes: every array read as 16-byte vectors, the quad's x and
+// z-faces carried from plane to plane (the neighbours read are of the other
+// colour, which this pass leaves alone).  Per two updated cells 8 vector and
+// 3 scalar loads where the pairs take 28 scalar ones; the pairs' pass was bound
+// by the latency of its loads (200 us over 64 instances of 20 M cells, 2.5 TB/s
+// of algorithmic bytes; 115 us in quads).  Needs nx % 4 == 0, no walls along x (the face rows are the cell
+// rows; arrays start on 256 bytes, so quads are aligned) and enough quads to
+// give every thread of the group a column.  Same update as pass_store.
+constexpr int kQuadPlanes = 8;
+
+__device__ __forceinline__ void ldq(float (&d)[4], const float* p) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    d[0] = v.x;
+    d[1] = v.y;
+    d[2] = v.z;
+    d[3] = v.w;
+}
+
+__device__ __noinline__ void rb_quads(int rank, int ncta, const BLevel& L, const float* __restrict__ f, float* x,
+                                         int color, float omega, bool zero, int planes) {
+    const Geo g = L.g;
+    const float *__restrict__ bx = L.b[0], *__restrict__ by = L.b[1], *__restrict__ bz = L.b[2];
+    const int nx = g.nx, ny = g.ny, nz = g.nz, pl = nx * ny, nq = nx / 4;
+    const unsigned mq = L.mq, my = L.my;
+    const int nzc = (nz + planes - 1) / planes;
+    const unsigned total = (unsigned)(nq * ny) * (unsigned)nzc;
+    for (unsigned t = (unsigned)(rank * kBT) + threadIdx.x; t < total; t += (unsigned)(ncta * kBT)) {
+        const unsigned row = fast_div(t, (unsigned)nq, mq), kc = fast_div(row, (unsigned)ny, my);
+        const int i0 = 4 * (int)(t - row * (unsigned)nq), j = (int)(row - kc * (unsigned)ny);
+        const int k0 = (int)kc * planes, k1 = min(k0 + planes, nz);
+        const bool ylo = j == 0, yhi = j == ny - 1;
+        const int oym = !ylo ? -nx : (g.wy ? 0 : (ny - 1) * nx), oyp = !yhi ? nx : (g.wy ? 0 : -(ny - 1) * nx);
+        const int ofy = (!yhi || g.wy) ? nx : -(ny - 1) * nx;  // the + y-face from the - one
+        const int ol = i0 > 0 ? -1 : nx - 1, orr = i0 + 4 < nx ? 4 : 4 - nx;  // cells next to the quad
+        int c = (k0 * ny + j) * nx + i0;
+        // carried from plane to plane: this plane's quad, and of the plane below
+        // (the z-faces below) the two entries that the updated cells need
+        float XC[4] = {0.f, 0.f, 0.f, 0.f}, xm[2] = {0.f, 0.f}, z0[2];
+        float XP[4] = {0.f, 0.f, 0.f, 0.f}, YM[4] = {0.f, 0.f, 0.f, 0.f}, YP[4] = {0.f, 0.f, 0.f, 0.f};
+        float Z1[4], BX[4], Y0[4], Y1[4], F[4];
+        float xl = 0.f, xr = 0.f;
+        bool m = (j + k0 + color) & 1;  // the updated member of both pairs
+        if (!zero) {
+            ldq(XP, x + (k0 > 0 ? c - pl : (g.wz ? c : c + (nz - 1) * pl)));
+            ldq(XC, x + c);
+        }
+        ldq(Z1, bz + c);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            xm[u] = m ? XP[2 * u + 1] : XP[2 * u];
+            z0[u] = m ? Z1[2 * u + 1] : Z1[2 * u];
+        }
+        for (int k = k0; k < k1; ++k, c += pl) {
+            const bool zlo = k == 0, zhi = k == nz - 1;
+            const int fy = (k * (ny + g.wy) + j) * nx + i0;
+            if (!zero) {
+                ldq(XP, x + (!zhi ? c + pl : (g.wz ? c : c - (nz - 1) * pl)));
+                ldq(YM, x + c + oym);
+                ldq(YP, x + c + oyp);
+                xl = x[c + ol];
+                xr = x[c + orr];
+            }
+            ldq(Z1, bz + ((!zhi || g.wz) ? c + pl : c - (nz - 1) * pl));
+            ldq(BX, bx + c);
+            ldq(Y0, by + fy);
+            ldq(Y1, by + fy + ofy);
+            ldq(F, f + c);
+            const float bxr = bx[c + orr];
+            float xn[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                auto sel = [&](const float (&a)[4]) { return m ? a[2 * u + 1] : a[2 * u]; };
+                const float b0 = sel(BX), b1 = m ? (u == 0 ? BX[2] : bxr) : BX[2 * u + 1];
+                const float b2 = (g.wy && ylo) ? 0.f : sel(Y0), b3 = (g.wy && yhi) ? 0.f : sel(Y1);
+                const float b4 = (g.wz && zlo) ? 0.f : z0[u], b5 = (g.wz && zhi) ? 0.f : sel(Z1);
+                const float sum = ((b0 + b1) + (b2 + b3)) + (b4 + b5);
+                const float wv = sum > 0.f ? rcp_rn(sum) : 0.f;
+                if (zero) {
+                    xn[u] = omega * wv * sel(F);
+                } else {
+                    float acc = sel(F);
+                    acc = fmaf(b0, m ? XC[2 * u] : (u == 0 ? xl : XC[1]), acc);
+                    acc = fmaf(b1, m ? (u == 0 ? XC[2] : xr) : XC[2 * u + 1], acc);
+                    acc = fmaf(b2, sel(YM), acc);
+                    acc = fmaf(b3, sel(YP), acc);
+                    acc = fmaf(b4, xm[u], acc);
+                    acc = fmaf(b5, sel(XP), acc);
+                    const float xc = sel(XC);
+                    xn[u] = fmaf(omega, fmaf(wv, acc, -xc), xc);
+                }
+            }
+            if (zero) {  // the other colour zeroed
+                *reinterpret_cast<float4*>(x + c) =
+                    make_float4(m ? 0.f : xn[0], m ? xn[0] : 0.f, m ? 0.f : xn[1], m ? xn[1] : 0.f);
+            } else {
+                x[c + (m ? 1 : 0)] = xn[0];
+                x[c + (m ? 3 : 2)] = xn[1];
+            }
+            m = !m;  // the next plane updates the other members
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                xm[u] = m ? XC[2 * u + 1] : XC[2 * u];
+                z0[u] = m ? Z1[2 * u + 1] : Z1[2 * u];
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v) XC[v] = XP[v];
+        }
+    }
+}
+
 // One red-black colour pass in place on level L (zero: x taken as 0 and the
 // other colour zeroed).  x_c <- x_c + omega (w (f + sum beta x_nb) - x_c).
 // A thread takes two pairs per iteration and loads both stencils before it
 // updates either: cells of the updated colour are never neighbours of one
 // another, so the two updates are independent.
-__device__ __noinline__ void rb_pass(Grp& cx, const BLevel& L, const float* f, float* x, int color, float omega,
-                        bool zero) {
-    const Geo& g = L.g;
-    const unsigned npair = (unsigned)(g.nx + 1) / 2;
+__device__ __noinline__ void rb_pairs(int rank, int ncta, const BLevel& L, const float* f, float* x, int color,
+                                      float omega, bool zero) {
+    const Geo g = L.g;  // in registers: the stores below could alias the descriptor
+    const float *bx = L.b[0], *by = L.b[1], *bz = L.b[2];
+    const unsigned npair = (unsigned)(g.nx + 1) / 2, mp = L.mp, my = L.my;
     const int64_t total = (int64_t)npair * g.ny * g.nz;
-    const int64_t stride = (int64_t)cx.ncta * kBT;
-    for (int64_t p0 = (int64_t)cx.rank * kBT + threadIdx.x; p0 < total; p0 += 2 * stride) {
+    const int64_t stride = (int64_t)ncta * kBT;
+    for (int64_t p0 = (int64_t)rank * kBT + threadIdx.x; p0 < total; p0 += 2 * stride) {
         const int64_t p1 = p0 + stride;
-        const PassCell a = pass_cell(g, (unsigned)p0, npair, color);
-        const PassCell b = p1 < total ? pass_cell(g, (unsigned)p1, npair, color) : PassCell{g.nx, 0, 0, g.nx};
+        const PassCell a = pass_cell(g, (unsigned)p0, npair, mp, my, color);
+        const PassCell b = p1 < total ? pass_cell(g, (unsigned)p1, npair, mp, my, color) : PassCell{g.nx, 0, 0, g.nx};
         PassLoad da, db;
-        pass_load(da, L, f, x, a, zero);
-        pass_load(db, L, f, x, b, zero);
+        pass_load(da, g, bx, by, bz, f, x, a, zero);
+        pass_load(db, g, bx, by, bz, f, x, b, zero);
         pass_store(da, g, x, a, omega, zero);
         pass_store(db, g, x, b, omega, zero);
     }
 }
 
-__device__ bool vcycle(Grp& cx, const BParams& P, const float* f0, float* x0) {
-    const BInst& I = *cx.I;
-    const int nl = I.nlev;
-    for (int l = 0; l < nl - 1; ++l) {
-        const BLevel& L = I.lv[l];
-        const float* f = l == 0 ? f0 : L.f;
-        float* x = l == 0 ? x0 : L.x;
-        for (int s = 0; s < P.nu1; ++s) {
-            rb_pass(cx, L, f, x, 0, P.omega, s == 0);
-            if (!gbar(cx)) return false;
-            rb_pass(cx, L, f, x, 1, P.omega, false);
-            if (!gbar(cx)) return false;
+// One colour pass on a level: quads where every thread of the group gets at
+// least two planes of one, pairs otherwise.
+__device__ __forceinline__ void rb_pass(int rank, int ncta, const BLevel& L, const float* f, float* x, int color,
+                                        float omega, bool zero) {
+    const int nx = L.g.nx, per = nx / 4 * L.g.ny * L.g.nz / (ncta * kBT);
+    if (nx % 4 == 0 && !L.g.wx && per >= 2)
+        rb_quads(rank, ncta, L, f, x, color, omega, zero, per < kQuadPlanes ? per : kQuadPlanes);
+    else
+        rb_pairs(rank, ncta, L, f, x, color, omega, zero);
+}
+
+// q = A d on the finest level; returns this thread's part of d . q.  Quads
+// marching through planes as in rb_quads, cell by cell otherwise.
+__device__ __noinline__ float product(int rank, int ncta, const BLevel& L, const float* __restrict__ d,
+                                      float* __restrict__ q) {
+    const Geo g = L.g;
+    const float *__restrict__ bx = L.b[0], *__restrict__ by = L.b[1], *__restrict__ bz = L.b[2];
+    const int nx = g.nx, ny = g.ny, nz = g.nz, pl = nx * ny, nq = nx / 4;
+    const unsigned mx = L.mx, my = L.my, mq = L.mq;
+    float loc = 0.f;
+    const int per = nq * ny * nz / (ncta * kBT);
+    if (nx % 4 != 0 || g.wx || per < 2) {
+        for (int64_t c = (int64_t)rank * kBT + threadIdx.x; c < g.ncell(); c += (int64_t)ncta * kBT) {
+            int i, j, k, c32;
+            decomp(g, mx, my, c, i, j, k);
+            Stencil<float> s;
+            load_stencil_fast(g, bx, by, bz, i, j, k, s, c32);
+            const float dc = d[c], qc = apply_A(s, d, dc, 1.0f);
+            q[c] = qc;
+            loc = fmaf(dc, qc, loc);
         }
-        if (P.nu1 == 0) {
-            GLOOP(c, L.g.ncell()) x[c] = 0.f;
-            if (!gbar(cx)) return false;
-        }
-        const BLevel& Cl = I.lv[l + 1];
-        Coef<float> cf{L.b[0], L.b[1], L.b[2], 1.0f};
-        GLOOP(cc, Cl.g.ncell()) {
-            int I0, J0, K0;
-            decomp(Cl.g, cc, I0, J0, K0);
-            float sum = 0.f;
-            for (int dk = 0; dk < Cl.fac[2]; ++dk)
-                for (int dj = 0; dj < Cl.fac[1]; ++dj)
-                    for (int di = 0; di < Cl.fac[0]; ++di) {
-                        const int i = I0 * Cl.fac[0] + di, j = J0 * Cl.fac[1] + dj, k = K0 * Cl.fac[2] + dk;
-                        const int64_t c = L.g.cidx(i, j, k);
-                        Stencil<float> s;
-                        int c32_;
-                        load_stencil_fast(L.g, cf.bx, cf.by, cf.bz, i, j, k, s, c32_);
-                        sum += f[c] - apply_A(s, x, x[c], 1.0f);
-                    }
-            Cl.f[cc] = sum / (float)(Cl.fac[0] * Cl.fac[1] * Cl.fac[2]);
-        }
-        if (!gbar(cx)) return false;
+        return loc;
     }
-    {
-        const BLevel& Cl = I.lv[nl - 1];
-        const float* f = nl == 1 ? f0 : Cl.f;
-        float* x = nl == 1 ? x0 : Cl.x;
-        if (I.dense) {
-            if (cx.rank == 0) {
-                const int n = I.ncoarse;
-                __shared__ double fs[kMaxDense];
-                __shared__ double mean;
-                for (int c = threadIdx.x; c < n; c += kBT) fs[c] = (double)f[c];
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    double t = 0.0;
-                    for (int c = 0; c < n; ++c) t += fs[c];
-                    mean = t / n;
-                }
-                __syncthreads();
-                for (int r = threadIdx.x; r < n; r += kBT) {
-                    double acc = 0.0;
-                    for (int c = 0; c < n; ++c) acc = fma(I.cinv[(int64_t)r * n + c], fs[c] - mean, acc);
-                    x[r] = (float)acc;
-                }
+    const int planes = per < kQuadPlanes ? per : kQuadPlanes;
+    const unsigned total = (unsigned)(nq * ny) * (unsigned)((nz + planes - 1) / planes);
+    for (unsigned t = (unsigned)(rank * kBT) + threadIdx.x; t < total; t += (unsigned)(ncta * kBT)) {
+        const unsigned row = fast_div(t, (unsigned)nq, mq), kc = fast_div(row, (unsigned)ny, my);
+        const int i0 = 4 * (int)(t - row * (unsigned)nq), j = (int)(row - kc * (unsigned)ny);
+        const int k0 = (int)kc * planes, k1 = min(k0 + planes, nz);
+        const bool ylo = j == 0, yhi = j == ny - 1;
+        const int oym = !ylo ? -nx : (g.wy ? 0 : (ny - 1) * nx), oyp = !yhi ? nx : (g.wy ? 0 : -(ny - 1) * nx);
+        const int ofy = (!yhi || g.wy) ? nx : -(ny - 1) * nx;
+        const int ol = i0 > 0 ? -1 : nx - 1, orr = i0 + 4 < nx ? 4 : 4 - nx;
+        int c = (k0 * ny + j) * nx + i0;
+        float XM[4], XC[4], XP[4], YM[4], YP[4], Z0[4], Z1[4], BX[4], Y0[4], Y1[4];
+        ldq(XM, d + (k0 > 0 ? c - pl : (g.wz ? c : c + (nz - 1) * pl)));
+        ldq(XC, d + c);
+        ldq(Z0, bz + c);
+        for (int k = k0; k < k1; ++k, c += pl) {
+            const bool zlo = k == 0, zhi = k == nz - 1;
+            const int fy = (k * (ny + g.wy) + j) * nx + i0;
+            ldq(XP, d + (!zhi ? c + pl : (g.wz ? c : c - (nz - 1) * pl)));
+            ldq(YM, d + c + oym);
+            ldq(YP, d + c + oyp);
+            ldq(Z1, bz + ((!zhi || g.wz) ? c + pl : c - (nz - 1) * pl));
+            ldq(BX, bx + c);
+            ldq(Y0, by + fy);
+            ldq(Y1, by + fy + ofy);
+            const float xl = d[c + ol], xr = d[c + orr], bxr = bx[c + orr];
+            float Q[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const float xc = XC[v];
+                float a = BX[v] * (xc - (v > 0 ? XC[v - 1] : xl));
+                a = fmaf(v < 3 ? BX[v + 1] : bxr, xc - (v < 3 ? XC[v + 1] : xr), a);
+                a = fmaf((g.wy && ylo) ? 0.f : Y0[v], xc - YM[v], a);
+                a = fmaf((g.wy && yhi) ? 0.f : Y1[v], xc - YP[v], a);
+                a = fmaf((g.wz && zlo) ? 0.f : Z0[v], xc - XM[v], a);
+                a = fmaf((g.wz && zhi) ? 0.f : Z1[v], xc - XP[v], a);
+                Q[v] = a;
+                loc = fmaf(xc, a, loc);
             }
-            if (!gbar(cx)) return false;
-        } else {
-            for (int s = 0; s < 8; ++s) {
-                rb_pass(cx, Cl, f, x, 0, P.omega, s == 0);
-                if (!gbar(cx)) return false;
-                rb_pass(cx, Cl, f, x, 1, P.omega, false);
-                if (!gbar(cx)) return false;
-            }
-            for (int s = 0; s < 8; ++s) {
-                rb_pass(cx, Cl, f, x, 1, P.omega, false);
-                if (!gbar(cx)) return false;
-                rb_pass(cx, Cl, f, x, 0, P.omega, false);
-                if (!gbar(cx)) return false;
+            *reinterpret_cast<float4*>(q + c) = make_float4(Q[0], Q[1], Q[2], Q[3]);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                XM[v] = XC[v];
+                XC[v] = XP[v];
+                Z0[v] = Z1[v];
             }
         }
     }
-    for (int l = nl - 2; l >= 0; --l) {
-        const BLevel& L = I.lv[l];
-        const BLevel& Cl = I.lv[l + 1];
-        const float* f = l == 0 ? f0 : L.f;
-        float* x = l == 0 ? x0 : L.x;
-        GLOOP(c, L.g.ncell()) {
-            int i, j, k;
-            decomp(L.g, c, i, j, k);
-            // coarsening factors are 1 or 2: halving is a shift
-            x[c] += Cl.x[Cl.g.cidx(i >> (Cl.fac[0] - 1), j >> (Cl.fac[1] - 1), k >> (Cl.fac[2] - 1))];
+    return loc;
+}
+
+// Coarse right-hand side: the children's mean of f - A x, A x on the coarse
+// cell's surface faces only (apply_A_faces).
+__device__ __noinline__ void restrict_level(int rank, int ncta, const BLevel& L, const BLevel& Cl, const float* f,
+                                            const float* x) {
+    const Geo g = L.g, cg = Cl.g;
+    const float *bx = L.b[0], *by = L.b[1], *bz = L.b[2];
+    const int f0 = Cl.fac[0], f1 = Cl.fac[1], f2 = Cl.fac[2];
+    const unsigned mx = Cl.mx, my = Cl.my;
+    float* out = Cl.f;
+    const float inv = 1.0f / (float)(f0 * f1 * f2);
+    auto child = [&](int I0, int J0, int K0, int di, int dj, int dk, unsigned mask) {
+        Stencil<float> s;
+        int c;
+        load_stencil_fast(g, bx, by, bz, I0 * f0 + di, J0 * f1 + dj, K0 * f2 + dk, s, c);
+        return f[c] - apply_A_faces(s, x, x[c], 1.0f, mask);
+    };
+    for (int64_t cc = (int64_t)rank * kBT + threadIdx.x; cc < cg.ncell(); cc += (int64_t)ncta * kBT) {
+        int I0, J0, K0;
+        decomp(cg, mx, my, cc, I0, J0, K0);
+        float sum = 0.f;
+        for (int dk = 0; dk < f2; ++dk) {
+            if (f0 == 2 && f1 == 2) {  // four children at a time in flight
+#pragma unroll
+                for (int dj = 0; dj < 2; ++dj)
+#pragma unroll
+                    for (int di = 0; di < 2; ++di)
+                        sum += child(I0, J0, K0, di, dj, dk, surface_faces(di, dj, dk, 2, 2, f2));
+            } else {
+                for (int dj = 0; dj < f1; ++dj)
+                    for (int di = 0; di < f0; ++di)
+                        sum += child(I0, J0, K0, di, dj, dk, surface_faces(di, dj, dk, f0, f1, f2));
+            }
         }
-        if (!gbar(cx)) return false;
-        for (int s = 0; s < P.nu2; ++s) {
-            rb_pass(cx, L, f, x, 1, P.omega, false);
-            if (!gbar(cx)) return false;
-            rb_pass(cx, L, f, x, 0, P.omega, false);
-            if (!gbar(cx)) return false;
+        out[cc] = sum * inv;
+    }
+}
+
+__device__ __noinline__ void prolong_level(int rank, int ncta, const BLevel& L, const BLevel& Cl, float* x) {
+    const Geo g = L.g, cg = Cl.g;
+    const int s0 = Cl.fac[0] - 1, s1 = Cl.fac[1] - 1, s2 = Cl.fac[2] - 1;  // factors are 1 or 2: halving is a shift
+    const unsigned mx = L.mx, my = L.my;
+    const float* xc = Cl.x;
+    const int64_t n = g.ncell(), stride = (int64_t)ncta * kBT;
+    if (s0 && g.nx % 4 == 0) {  // four cells and their two parents along x at a time
+        const unsigned nq = (unsigned)(g.nx / 4), mq = L.mq, ny = (unsigned)g.ny;
+        for (int64_t t = (int64_t)rank * kBT + threadIdx.x; t < n / 4; t += stride) {
+            const unsigned row = fast_div((unsigned)t, nq, mq), k = fast_div(row, ny, my);
+            const int q = (int)((unsigned)t - row * nq), j = (int)(row - k * ny);
+            const float* e = xc + cg.cidx(2 * q, j >> s1, (int)k >> s2);
+            float4* px = reinterpret_cast<float4*>(x) + t;
+            const float e0 = e[0], e1 = e[1];
+            float4 v = *px;
+            v.x += e0;
+            v.y += e0;
+            v.z += e1;
+            v.w += e1;
+            *px = v;
         }
+        return;
+    }
+    for (int64_t c = (int64_t)rank * kBT + threadIdx.x; c < n; c += stride) {
+        int i, j, k;
+        decomp(g, mx, my, c, i, j, k);
+        x[c] += xc[cg.cidx(i >> s0, j >> s1, k >> s2)];
+    }
+}
+
+// One group of CTAs, or (solo) one CTA alone: the barrier between the steps.
+__device__ __forceinline__ bool step_sync(Grp& cx, bool solo) {
+    if (solo) {
+        __syncthreads();
+        return true;
+    }
+    return gbar(cx);
+}
+
+// First level of the V-cycle that one CTA runs alone: below kSoloCells cells
+// a step is shorter than the barrier of the group after it.
+constexpr int64_t kSoloCells = 4096;
+
+__device__ bool smooth_level(Grp& cx, const BParams& P, const BLevel& L, const float* f, float* x, int sweeps,
+                             bool first_zero, bool reverse, bool solo) {
+    const int rank = solo ? 0 : cx.rank, ncta = solo ? 1 : cx.ncta, c0 = reverse ? 1 : 0;
+    for (int s = 0; s < sweeps; ++s) {
+        rb_pass(rank, ncta, L, f, x, c0, P.omega, first_zero && s == 0);
+        if (!step_sync(cx, solo)) return false;
+        rb_pass(rank, ncta, L, f, x, 1 - c0, P.omega, false);
+        if (!step_sync(cx, solo)) return false;
     }
     return true;
 }
 
+// The V-cycle from level l down to the coarsest and back, on all CTAs of the
+// group or (solo) on this one alone; stop: the level where the descent ends
+// (nl - 1: the coarsest, solved; less: left to one CTA, see vcycle).
+__device__ bool vcycle_down(Grp& cx, const BParams& P, const float* f0, float* x0, int l, int stop, bool solo) {
+    const BInst& I = *cx.I;
+    const int rank = solo ? 0 : cx.rank, ncta = solo ? 1 : cx.ncta;
+    for (; l < stop; ++l) {
+        const BLevel& L = I.lv[l];
+        const float* f = l == 0 ? f0 : L.f;
+        float* x = l == 0 ? x0 : L.x;
+        if (P.nu1 == 0) {
+            for (int64_t c = (int64_t)rank * kBT + threadIdx.x; c < L.g.ncell(); c += (int64_t)ncta * kBT) x[c] = 0.f;
+            if (!step_sync(cx, solo)) return false;
+        }
+        if (!smooth_level(cx, P, L, f, x, P.nu1, true, false, solo)) return false;
+        restrict_level(rank, ncta, L, I.lv[l + 1], f, x);
+        if (!step_sync(cx, solo)) return false;
+    }
+    return true;
+}
+
+__device__ bool vcycle_up(Grp& cx, const BParams& P, const float* f0, float* x0, int from, int to, bool solo) {
+    const BInst& I = *cx.I;
+    const int rank = solo ? 0 : cx.rank, ncta = solo ? 1 : cx.ncta;
+    for (int l = from; l >= to; --l) {
+        const BLevel& L = I.lv[l];
+        float* x = l == 0 ? x0 : L.x;
+        prolong_level(rank, ncta, L, I.lv[l + 1], x);
+        if (!step_sync(cx, solo)) return false;
+        if (!smooth_level(cx, P, L, l == 0 ? f0 : L.f, x, P.nu2, false, true, solo)) return false;
+    }
+    return true;
+}
+
+// the dense coarsest solve x = M (f - mean f), by one CTA
+__device__ void coarse_dense(const BInst& I, const float* f, float* x) {
+    const int n = I.ncoarse;
+    __shared__ double fs[kMaxDense];
+    __shared__ double mean;
+    for (int c = threadIdx.x; c < n; c += kBT) fs[c] = (double)f[c];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int c = 0; c < n; ++c) t += fs[c];
+        mean = t / n;
+    }
+    __syncthreads();
+    for (int r = threadIdx.x; r < n; r += kBT) {
+        double acc = 0.0;
+        for (int c = 0; c < n; ++c) acc = fma(I.cinv[(int64_t)r * n + c], fs[c] - mean, acc);
+        x[r] = (float)acc;
+    }
+    __syncthreads();
+}
+
+__device__ bool vcycle(Grp& cx, const BParams& P, const float* f0, float* x0) {
+    const BInst& I = *cx.I;
+    const int nl = I.nlev;
+    // levels [solo, nl) on the group's first CTA alone; the others wait at one barrier
+    int solo = nl;
+    if (I.dense) {
+        solo = nl - 1;
+        while (solo > 0 && I.lv[solo - 1].g.ncell() <= kSoloCells) --solo;
+    }
+    const int stop = solo < nl ? solo : nl - 1;
+    if (!vcycle_down(cx, P, f0, x0, 0, stop, false)) return false;
+    if (solo < nl) {
+        if (cx.rank == 0) {
+            vcycle_down(cx, P, f0, x0, solo, nl - 1, true);
+            coarse_dense(I, nl == 1 ? f0 : I.lv[nl - 1].f, nl == 1 ? x0 : I.lv[nl - 1].x);
+            vcycle_up(cx, P, f0, x0, nl - 2, solo, true);
+        }
+        if (!gbar(cx)) return false;
+    } else {  // a coarsest level too large for the dense solve: 8 + 8 sweeps
+        const BLevel& Cl = I.lv[nl - 1];
+        const float* f = nl == 1 ? f0 : Cl.f;
+        float* x = nl == 1 ? x0 : Cl.x;
+        if (!smooth_level(cx, P, Cl, f, x, 8, true, false, false)) return false;
+        if (!smooth_level(cx, P, Cl, f, x, 8, false, true, false)) return false;
+    }
+    return vcycle_up(cx, P, f0, x0, stop - 1, 0, false);
+}
+
 // ------------------------------------------------------------ solve ---
+
+// The solve's passes over its vectors, each a function of its own: inlined
+// into the kernel they spilled (its registers are bounded for two CTAs per
+// SM).  The vectors start on 256 bytes: four elements at a time, then the rest.
+#define VLOOP(t_, n_) for (int64_t t_ = (int64_t)rank * kBT + threadIdx.x; t_ < (n_) / 4; t_ += (int64_t)ncta * kBT)
+#define VTAIL(c_, n_) for (int64_t c_ = (n_) / 4 * 4 + (int64_t)rank * kBT + threadIdx.x; c_ < (n_); c_ += (int64_t)ncta * kBT)
+
+// r = (float)(scale f): the first residual (p = 0)
+__device__ __noinline__ void first_residual(const BInst& I, int rank, int ncta, double scale) {
+    const double* f = I.f64;
+    float* r = I.r;
+    const int64_t n = I.g0.ncell();
+    GLOOP(c, n) r[c] = d2f_scaled(f[c] * scale, 0);
+}
+
+// r = (float)(scale (f - A p)) and this thread's |r|^2, max |r|, non-finite count of the FP64 residual
+__device__ __noinline__ void true_residual(const BInst& I, int rank, int ncta, double scale, double (&n3)[3]) {
+    const Geo g = I.g0;
+    const unsigned mx = I.lv[0].mx, my = I.lv[0].my;
+    const double *bx = I.b64[0], *by = I.b64[1], *bz = I.b64[2], *f = I.f64, *p = I.p;
+    const double ih2 = 1.0 / (I.h * I.h);
+    float* r = I.r;
+    double l2 = 0.0;
+    unsigned nf = 0;
+    unsigned long long mk = 0;
+    GLOOP(c, g.ncell()) {
+        int i, j, k, c32;
+        decomp(g, mx, my, c, i, j, k);
+        Stencil<double> s;
+        load_stencil_fast(g, bx, by, bz, i, j, k, s, c32);
+        const double rc = f[c] - apply_A(s, p, p[c], ih2);
+        r[c] = d2f_scaled(rc * scale, 0);
+        l2 = fma(rc, rc, l2);
+        const unsigned long long kr = abs_key(rc);
+        mk = kr > mk ? kr : mk;
+        nf += key_nonfinite(kr);
+    }
+    n3[0] = l2;
+    n3[1] = key_value(mk);
+    n3[2] = (double)nf;
+}
+
+// d = z; returns this thread's part of r . z
+__device__ __noinline__ float dot_copy(const BInst& I, int rank, int ncta) {
+    const int64_t n = I.g0.ncell();
+    const float *r = I.r, *z = I.z;
+    float* d = I.d;
+    float a = 0.f;
+    VLOOP(t, n) {
+        const float4 rv = reinterpret_cast<const float4*>(r)[t], zv = reinterpret_cast<const float4*>(z)[t];
+        reinterpret_cast<float4*>(d)[t] = zv;
+        a = fmaf(rv.x, zv.x, fmaf(rv.y, zv.y, fmaf(rv.z, zv.z, fmaf(rv.w, zv.w, a))));
+    }
+    VTAIL(c, n) {
+        d[c] = z[c];
+        a = fmaf(r[c], z[c], a);
+    }
+    return a;
+}
+
+// e += alpha d (first: e = alpha d), r -= alpha q; this thread's |r|^2 and non-finite count
+__device__ __noinline__ float update(const BInst& I, int rank, int ncta, float al, bool first, unsigned& nonfin) {
+    const int64_t n = I.g0.ncell();
+    const float *d = I.d, *q = I.q;
+    float *e = I.e, *r = I.r;
+    float l2 = 0.f;
+    unsigned nf = 0;
+    VLOOP(t, n) {
+        const float4 dv = reinterpret_cast<const float4*>(d)[t], qv = reinterpret_cast<const float4*>(q)[t];
+        float4 rv = reinterpret_cast<float4*>(r)[t];
+        float4 evv = first ? make_float4(0.f, 0.f, 0.f, 0.f) : reinterpret_cast<float4*>(e)[t];
+        auto one = [&](float dc, float qc, float& ec, float& rc) {
+            ec = fmaf(al, dc, ec);
+            rc = fmaf(-al, qc, rc);
+            l2 = fmaf(rc, rc, l2);
+            nf += isfinite(rc) ? 0u : 1u;
+        };
+        one(dv.x, qv.x, evv.x, rv.x);
+        one(dv.y, qv.y, evv.y, rv.y);
+        one(dv.z, qv.z, evv.z, rv.z);
+        one(dv.w, qv.w, evv.w, rv.w);
+        reinterpret_cast<float4*>(e)[t] = evv;
+        reinterpret_cast<float4*>(r)[t] = rv;
+    }
+    VTAIL(c, n) {
+        e[c] = fmaf(al, d[c], first ? 0.f : e[c]);
+        const float rc = fmaf(-al, q[c], r[c]);
+        r[c] = rc;
+        l2 = fmaf(rc, rc, l2);
+        nf += isfinite(rc) ? 0u : 1u;
+    }
+    nonfin = nf;
+    return l2;
+}
+
+// this thread's parts of z . r and z . q
+__device__ __noinline__ float2 dots(const BInst& I, int rank, int ncta) {
+    const int64_t n = I.g0.ncell();
+    const float *z = I.z, *r = I.r, *q = I.q;
+    float a = 0.f, b = 0.f;
+    VLOOP(t, n) {
+        const float4 zv = reinterpret_cast<const float4*>(z)[t], rv = reinterpret_cast<const float4*>(r)[t];
+        const float4 qv = reinterpret_cast<const float4*>(q)[t];
+        a = fmaf(zv.x, rv.x, fmaf(zv.y, rv.y, fmaf(zv.z, rv.z, fmaf(zv.w, rv.w, a))));
+        b = fmaf(zv.x, qv.x, fmaf(zv.y, qv.y, fmaf(zv.z, qv.z, fmaf(zv.w, qv.w, b))));
+    }
+    VTAIL(c, n) {
+        a = fmaf(z[c], r[c], a);
+        b = fmaf(z[c], q[c], b);
+    }
+    return make_float2(a, b);
+}
+
+// d = z + beta d
+__device__ __noinline__ void direction(const BInst& I, int rank, int ncta, float be) {
+    const int64_t n = I.g0.ncell();
+    const float* z = I.z;
+    float* d = I.d;
+    VLOOP(t, n) {
+        const float4 zv = reinterpret_cast<const float4*>(z)[t];
+        float4 dv = reinterpret_cast<float4*>(d)[t];
+        dv.x = fmaf(be, dv.x, zv.x);
+        dv.y = fmaf(be, dv.y, zv.y);
+        dv.z = fmaf(be, dv.z, zv.z);
+        dv.w = fmaf(be, dv.w, zv.w);
+        reinterpret_cast<float4*>(d)[t] = dv;
+    }
+    VTAIL(c, n) d[c] = fmaf(be, d[c], z[c]);
+}
+
+// p += e / scale
+__device__ __noinline__ void accumulate(const BInst& I, int rank, int ncta, double inv) {
+    const int64_t n = I.g0.ncell();
+    const float* e = I.e;
+    double* p = I.p;
+    GLOOP(c, n) p[c] = fma(f2d_scaled(e[c], 0), inv, p[c]);
+}
 
 __device__ bool solve(Grp& cx, const BParams& P, double bnorm2, double binf, int& iters, int& outer,
                       double& rr, double& rinf, int& converged) {
     const BInst& I = *cx.I;
-    const Geo& g = I.g0;
-    const int64_t N = g.ncell();
-    Coef<double> c64{I.b64[0], I.b64[1], I.b64[2], 1.0 / (I.h * I.h)};
-    Coef<float> c32{I.lv[0].b[0], I.lv[0].b[1], I.lv[0].b[2], 1.0f};
+    const int rank = cx.rank, ncta = cx.ncta;
     const double tol = P.tol;
     double rinf_prev = binf, prev_rr = INFINITY;
     int stalls = 0;
@@ -507,26 +950,20 @@ __device__ bool solve(Grp& cx, const BParams& P, double bnorm2, double binf, int
         converged = 1;
         return true;
     }
-    for (;;) {
+    for (bool first = true;; first = false) {
         // FP64 true residual, scaled FP32 copy for the inner solve
         const double scale = 1.0 / (rinf_prev > 1e-300 ? rinf_prev : 1.0);
         double n3[3] = {0.0, 0.0, 0.0};
-        unsigned nonfin = 0;
-        GLOOP(c, N) {
-            int i, j, k;
-            decomp(g, c, i, j, k);
-            Stencil<double> s;
-            int c32_;
-            load_stencil_fast(g, c64.bx, c64.by, c64.bz, i, j, k, s, c32_);
-            const double r = I.f64[c] - apply_A(s, I.p, I.p[c], c64.scale);
-            I.r[c] = (float)(r * scale);
-            n3[0] = fma(r, r, n3[0]);
-            n3[1] = fmax(n3[1], fabs(r));
-            nonfin += isfinite(r) ? 0u : 1u;
+        if (first) {  // p = 0: r = f, whose norms the set-up took
+            first_residual(I, rank, ncta, scale);
+            if (!gbar(cx)) return false;
+            n3[0] = bnorm2;
+            n3[1] = binf;
+        } else {
+            true_residual(I, rank, ncta, scale, n3);
+            const int op3[3] = {0, 1, 0};
+            if (!greduce<3>(cx, n3, op3)) return false;
         }
-        n3[2] = (double)nonfin;
-        const int op3[3] = {0, 1, 0};
-        if (!greduce<3>(cx, n3, op3)) return false;
         rr = n3[0];
         rinf = n3[1];
         if (n3[2] > 0) return true;
@@ -546,67 +983,76 @@ __device__ bool solve(Grp& cx, const BParams& P, double bnorm2, double binf, int
         double need2 = (tol * tol * bnorm2) / fmax(rr, 1e-300) * 1e-2;
         const double target = rr32 * fmax(P.inner_tol * P.inner_tol, fmin(need2, 1.0));
         // inner flexible CG on A e = r (FP32 vectors, FP64 group sums)
-        GLOOP(c, N) I.e[c] = 0.f;
         if (!vcycle(cx, P, I.r, I.z)) return false;
         // per-thread sums in FP32 (the element-wise products' precision),
         // across threads and CTAs in FP64
-        float a0 = 0.f;
-        GLOOP(c, N) {
-            a0 = fmaf(I.r[c], I.z[c], a0);
-            I.d[c] = I.z[c];
-        }
+        const float a0 = dot_copy(I, rank, ncta);
         double d2[2] = {(double)a0, 0.0};
         const int op2[2] = {0, 0};
         if (!greduce<2>(cx, d2, op2)) return false;
         double rho = d2[0];
         for (int jj = 0; jj < 50 && iters < P.max_iter; ++jj) {
-            float aq = 0.f;
-            GLOOP(c, N) {
-                int i, j, k;
-                decomp(g, c, i, j, k);
-                Stencil<float> s;
-                int c32_;
-                load_stencil_fast(g, c32.bx, c32.by, c32.bz, i, j, k, s, c32_);
-                const float qc = apply_A(s, I.d, I.d[c], 1.0f);
-                I.q[c] = qc;
-                aq = fmaf(I.d[c], qc, aq);
-            }
+            const float aq = product(rank, ncta, I.lv[0], I.d, I.q);
             double dq[1] = {(double)aq};
             const int op1[1] = {0};
             if (!greduce<1>(cx, dq, op1)) return false;
             const double alpha = dq[0] > 0.0 ? rho / dq[0] : 0.0;
-            const float af = (float)alpha;
-            float ar = 0.f;
-            unsigned nonfin = 0;
-            GLOOP(c, N) {
-                I.e[c] = fmaf(af, I.d[c], I.e[c]);
-                const float rc = fmaf(-af, I.q[c], I.r[c]);
-                I.r[c] = rc;
-                ar = fmaf(rc, rc, ar);
-                nonfin += isfinite(rc) ? 0u : 1u;
-            }
+            unsigned nonfin;
+            const float ar = update(I, rank, ncta, (float)alpha, jj == 0, nonfin);
             double rn[2] = {(double)ar, (double)nonfin};
             if (!greduce<2>(cx, rn, op2)) return false;
             ++iters;
             if (rn[1] > 0 || rn[0] <= target || rn[0] > 1e6 * rr32) break;
             if (!vcycle(cx, P, I.r, I.z)) return false;
-            float z0 = 0.f, z1 = 0.f;
-            GLOOP(c, N) {
-                z0 = fmaf(I.z[c], I.r[c], z0);
-                z1 = fmaf(I.z[c], I.q[c], z1);
-            }
-            double zz[2] = {(double)z0, (double)z1};
+            const float2 zs = dots(I, rank, ncta);
+            double zz[2] = {(double)zs.x, (double)zs.y};
             if (!greduce<2>(cx, zz, op2)) return false;
             const double beta = rho != 0.0 ? -alpha * zz[1] / rho : 0.0;
             rho = zz[0];
-            const float bf = (float)beta;
-            GLOOP(c, N) I.d[c] = fmaf(bf, I.d[c], I.z[c]);
+            direction(I, rank, ncta, (float)beta);
             if (!gbar(cx)) return false;
         }
-        const double inv = 1.0 / scale;
-        GLOOP(c, N) I.p[c] = fma((double)I.e[c], inv, I.p[c]);
+        accumulate(I, rank, ncta, 1.0 / scale);
         if (!gbar(cx)) return false;
         rinf_prev = rinf;
+    }
+}
+
+__device__ __noinline__ double sum_p(const BInst& I, int rank, int ncta) {
+    const double* p = I.p;
+    const int64_t n = I.g0.ncell();
+    double m = 0.0;
+    GLOOP(c, n) m += p[c];
+    return m;
+}
+
+__device__ __noinline__ void subtract_mean(const BInst& I, int rank, int ncta, double mean) {
+    double* p = I.p;
+    const int64_t n = I.g0.ncell();
+    GLOOP(c, n) p[c] -= mean;
+}
+
+// u = u* - dt beta grad p, walls blocked
+__device__ __noinline__ void correct_velocity(const BInst& I, int rank, int ncta) {
+    const Geo g = I.g0;
+    const unsigned mx = I.lv[0].mx, my = I.lv[0].my;
+    const double dth = I.dt / I.h;
+    const double *bx = I.b64[0], *by = I.b64[1], *bz = I.b64[2], *p = I.p;
+    double *u = I.u, *v = I.v, *w = I.w;
+    GLOOP(c, g.ncell()) {
+        int i, j, k;
+        decomp(g, mx, my, c, i, j, k);
+        const double pc = p[c];
+        AxisNb ax = axis_nb(i, g.nx, g.wx), ay = axis_nb(j, g.ny, g.wy), az = axis_nb(k, g.nz, g.wz);
+        int64_t f = g.fx(i, j, k);
+        u[f] = ax.wm ? 0.0 : u[f] - dth * bx[f] * (pc - p[g.cidx(ax.m, j, k)]);
+        f = g.fy(i, j, k);
+        v[f] = ay.wm ? 0.0 : v[f] - dth * by[f] * (pc - p[g.cidx(i, ay.m, k)]);
+        f = g.fz(i, j, k);
+        w[f] = az.wm ? 0.0 : w[f] - dth * bz[f] * (pc - p[g.cidx(i, j, az.m)]);
+        if (g.wx && i == g.nx - 1) u[g.fx(g.nx, j, k)] = 0.0;
+        if (g.wy && j == g.ny - 1) v[g.fy(i, g.ny, k)] = 0.0;
+        if (g.wz && k == g.nz - 1) w[g.fz(i, j, g.nz)] = 0.0;
     }
 }
 
@@ -621,11 +1067,13 @@ __global__ void __launch_bounds__(kBT, 2) persistent_kernel(const BInst* __restr
     cx.ncta = cx.I->ncta;
     cx.err = err;
     cx.pb = 0;
+    cx.arrivals = 0;
     cx.spin = P.spin_limit;
     const BInst& I = *cx.I;
     double bnorm2 = 0, binf = 0, nonfin = 0, rr = 0, rinf = 0;
     int iters = 0, outer = 0, converged = 0;
-    setup_coefficients(cx);
+    const int rank = cx.rank, ncta = cx.ncta;
+    setup_coefficients(I, rank, ncta);
     if (!gbar(cx)) return;
     if (!setup_rhs(cx, bnorm2, binf, nonfin)) return;
     if (!setup_levels(cx)) return;
@@ -633,30 +1081,12 @@ __global__ void __launch_bounds__(kBT, 2) persistent_kernel(const BInst* __restr
         if (!solve(cx, P, bnorm2, binf, iters, outer, rr, rinf, converged)) return;
     }
     // mean-free p, then u = u* - dt beta grad p (walls blocked)
-    double m[1] = {0.0};
-    GLOOP(c, I.g0.ncell()) m[0] += I.p[c];
+    double m[1] = {sum_p(I, rank, ncta)};
     const int op1[1] = {0};
     if (!greduce<1>(cx, m, op1)) return;
-    const double mean = m[0] / (double)I.g0.ncell();
-    GLOOP(c, I.g0.ncell()) I.p[c] -= mean;
+    subtract_mean(I, rank, ncta, m[0] / (double)I.g0.ncell());
     if (!gbar(cx)) return;
-    const Geo& g = I.g0;
-    const double dth = I.dt / I.h;
-    GLOOP(c, g.ncell()) {
-        int i, j, k;
-        decomp(g, c, i, j, k);
-        const double pc = I.p[c];
-        AxisNb ax = axis_nb(i, g.nx, g.wx), ay = axis_nb(j, g.ny, g.wy), az = axis_nb(k, g.nz, g.wz);
-        int64_t f = g.fx(i, j, k);
-        I.u[f] = ax.wm ? 0.0 : I.u[f] - dth * I.b64[0][f] * (pc - I.p[g.cidx(ax.m, j, k)]);
-        f = g.fy(i, j, k);
-        I.v[f] = ay.wm ? 0.0 : I.v[f] - dth * I.b64[1][f] * (pc - I.p[g.cidx(i, ay.m, k)]);
-        f = g.fz(i, j, k);
-        I.w[f] = az.wm ? 0.0 : I.w[f] - dth * I.b64[2][f] * (pc - I.p[g.cidx(i, j, az.m)]);
-        if (g.wx && i == g.nx - 1) I.u[g.fx(g.nx, j, k)] = 0.0;
-        if (g.wy && j == g.ny - 1) I.v[g.fy(i, g.ny, k)] = 0.0;
-        if (g.wz && k == g.nz - 1) I.w[g.fz(i, j, g.nz)] = 0.0;
-    }
+    correct_velocity(I, rank, ncta);
     if (cx.rank == 0 && threadIdx.x == 0) {
         I.stats[0] = iters;
         I.stats[1] = outer;
@@ -767,7 +1197,7 @@ std::vector<int> allot(const std::vector<int64_t>& work, int R) {
         int best = -1;
         double bw = 0;
         for (int i = 0; i < n; ++i) {
-            const int64_t cap = std::max<int64_t>(1, work[i] / (kBT * 4));
+            const int64_t cap = std::max<int64_t>(1, work[i] / 1024);
             if (k[i] >= cap) continue;
             const double w = (double)work[i] / k[i];
             if (w > bw) { bw = w; best = i; }
@@ -822,7 +1252,7 @@ void set_params(paris_batch* b) {
     b->prm.nu1 = b->opts.nu1;
     b->prm.nu2 = b->opts.nu2;
     b->prm.omega = (float)b->opts.omega;
-    b->prm.spin_limit = 1ll << 24;  // ~2 s at 64 ns per spin
+    b->prm.spin_limit = 1ll << 22;  // a few seconds at about 0.7 us a poll
 }
 
 }  // namespace
@@ -898,6 +1328,10 @@ paris_status paris_batch_create(paris_batch** out, int n, const paris_grid* grid
                 L.fac[a] = lv[l].second[a];
                 L.b[a] = balloc<float>(b, L.g.nface(a), e);
             }
+            L.mx = fast_div_mul(L.g.nx);
+            L.my = fast_div_mul(L.g.ny);
+            L.mp = fast_div_mul((L.g.nx + 1) / 2);
+            L.mq = fast_div_mul(std::max(1, L.g.nx / 4));
             L.x = l == 0 ? nullptr : balloc<float>(b, L.g.ncell(), e);
             L.f = l == 0 ? nullptr : balloc<float>(b, L.g.ncell(), e);
         }

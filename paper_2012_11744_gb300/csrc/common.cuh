@@ -275,6 +275,14 @@ __device__ inline double recip64(double s) {
     return fma(y0, fma(e, e, e), y0);
 }
 
+// p / d for p < 2^31 by the multiplier m = floor(2^32 / d) + 1 of
+// fast_div_mul and one correction (the estimate is at most one too large)
+inline unsigned fast_div_mul(int d) { return (unsigned)(0x100000000ull / (unsigned)d + 1); }
+__device__ __forceinline__ unsigned fast_div(unsigned p, unsigned d, unsigned m) {
+    const unsigned q = d == 1 ? p : __umulhi(p, m);
+    return q * d > p ? q - 1 : q;
+}
+
 // Programmatic dependent launch: a kernel launched with launch_pdl may start
 // while the kernel before it on the stream is finishing; it waits here for
 // that kernel's completion (and its memory) before touching anything the

@@ -213,13 +213,6 @@ __global__ void __launch_bounds__(kTX* kTY, kPerSM) helm_matvec_dot_kernel(HelmG
     finalize_last_block(partials, helm_blocks(), fin, tid);
 }
 
-// p / d for p < 2^31 by the multiplier m = floor(2^32 / d) + 1 and one
-// correction (the estimate is at most one too large)
-__device__ __forceinline__ unsigned fast_div(unsigned p, unsigned d, unsigned m) {
-    const unsigned q = d == 1 ? p : __umulhi(p, m);
-    return q * d > p ? q - 1 : q;
-}
-
 constexpr int kUU = 4;  // unknowns in flight per thread of the update
 
 // x += alpha d, r -= alpha q; partials as the residual kernel's.  A
@@ -406,8 +399,7 @@ void launch_helm_update(const HelmGeo& g, const double* w, const Scal* s, const 
     const int64_t n = helm_unknowns(g);
     int64_t nb = (n + kRedThreads * kUU - 1) / (kRedThreads * kUU);
     nb = std::max<int64_t>(1, std::min<int64_t>(nb, (int64_t)device_sms() * kPerSM));
-    auto mul = [](int m) { return (unsigned)(0x100000000ull / (unsigned)m + 1); };
-    launch_pdl(helm_update_kernel, (unsigned)nb, kRedThreads, 0, st, g, (unsigned)n, mul(g.m[0]), mul(g.m[1]), w, s, d,
+    launch_pdl(helm_update_kernel, (unsigned)nb, kRedThreads, 0, st, g, (unsigned)n, fast_div_mul(g.m[0]), fast_div_mul(g.m[1]), w, s, d,
                q, x, r, partials, fin);
     count_launch();
 }

@@ -141,3 +141,20 @@ def test_batch_autotune_and_cache(paris, tmp_path):
                     u, v, w, cache_path=cache)
         assert b2.tuning() == (nu, om, bps)
         assert len(open(cache).read().strip().splitlines()) == 1
+
+
+def test_batch_quad_passes_with_walls(paris):
+    """With few CTAs per instance the finest level's passes run in quads
+    marching through planes: walls in y and z, plane counts that are no
+    multiple of the march, rows of 4, 5 and 8 quads; 60 copies of each grid
+    leave one or two CTAs per instance."""
+    grids = [pi.Grid(32, 16, 22, 1 / 32, (P, W, W)), pi.Grid(16, 20, 28, 1 / 28, (P, P, W)),
+             pi.Grid(20, 12, 30, 1 / 30, (P, W, P))]
+    probs = [pi.random_problem(g, seed=110 + i, rho1=[1000.0, 30.0, 300.0][i]) for i, g in enumerate(grids)]
+    out, st, ctas = run_batch(paris, probs * 60)
+    assert ctas < 3 * len(out)
+    for i, pr in enumerate(probs):
+        ref = oracle.projection_step(pr.grid, pr.C, pr.rho1, pr.rho2, pr.dt, pr.u, pr.v, pr.w)
+        for q in (i, i + 177):  # the first and the last copy
+            assert st[q]["converged"] == 1, st[q]
+            check_instance(pr, *out[q], ref=ref)
