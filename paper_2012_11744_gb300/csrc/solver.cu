@@ -1863,7 +1863,6 @@ paris_status paris_viscous_solve_mg(paris_ctx* c, int comp, const double* nu, do
     // the SPD form decides convergence; each refinement step solves A e = r
     // in FP32 with r scaled by a power of two (exact in both directions) to a
     // relative reduction inner_tol (or what the outer tolerance still needs)
-    double* r = c->r;
     float *r32 = c->r32, *z32 = c->z32, *d32 = c->d32, *q32 = c->q32, *e32 = c->e32;
     launch_hmg_setup(g, un, nu, tau, c->hmg.sig64, c->hmg.sig[0], us, c->partials, c->st,
                      FinSpec{c->scal, 3, 2, FIN_BNORMS, 0.0});
@@ -1872,7 +1871,9 @@ paris_status paris_viscous_solve_mg(paris_ctx* c, int comp, const double* nu, do
     bool converged = false, nonfinite = false;
     double prev_rr = INFINITY;
     for (;;) {
-        launch_hmg_residual64(g, un, c->hmg.sig64, us, r, c->partials, c->st, rnorms);
+        // the scale from the residual before (|b| at first), as in the Poisson solve
+        finalize(c->partials, 0, 1, 0, c->scal, FIN_SCALE, 0.0, c->st);
+        launch_hmg_residual64(g, un, c->hmg.sig64, us, c->scal, r32, c->partials, c->st, rnorms);
         CK(cudaGetLastError());
         s = read_scal(c);
         if (s != PARIS_OK) return s;
@@ -1883,33 +1884,42 @@ paris_status paris_viscous_solve_mg(paris_ctx* c, int comp, const double* nu, do
         if (h.rr > 0.25 * prev_rr) { if (++stalls >= 2) break; } else stalls = 0;
         prev_rr = h.rr;
         ++outer;
-        finalize(c->partials, 0, 1, 0, c->scal, FIN_SCALE, 0.0, c->st);  // scale from max |r|
-        launch_hmg_scale_d2f(n, r, c->scal, r32, c->partials, c->st, FinSpec{c->scal, 2, 2, FIN_STORE, 0.0});
         CK(cudaMemsetAsync(e32, 0, sizeof(float) * n, c->st));
-        s = read_scal(c);
-        if (s != PARIS_OK) return s;
-        const double rr32 = c->scal_h->red[0];
+        const double rr32 = h.rr * h.scale * h.scale;
         const double need2 = (tol * tol * h.bnorm2) / std::max(h.rr, 1e-300) * 1e-2;
         const double it2 = o.inner_tol * o.inner_tol;
         const double target = rr32 * std::max(it2, std::min(need2, 1.0));
         launch_hmg_vcycle32(P, c->hmg, r32, z32, nu1, nu2, 8, omega, c->st);
         launch_dot2<float>(n, r32, z32, nullptr, c->partials, c->st, FinSpec{c->scal, 2, 0, FIN_RHO_INIT, 0.0});
         std::swap(d32, z32);  // first direction d = z
+        double prev_in_rr = rr32;  // ||r32||^2 before the last iteration
         for (int j = 0; j < 50 && iters < max_iter; ++j) {
             launch_hmg_matvec32(P, c->hmg.sig[0], d32, q32, c->partials, c->st, FinSpec{c->scal, 1, 0, FIN_ALPHA, 0.0});
             launch_update_xr<float>(n, c->scal, d32, q32, e32, r32, c->partials, c->st,
                                     FinSpec{c->scal, 3, 2, FIN_STORE, 0.0});
+            s = read_scal_async(c);
+            if (s != PARIS_OK) return s;
+            // the next V-cycle and direction go in behind the norms' copy while
+            // even a reduction of ||r||^2 by 1000 in this iteration would leave
+            // it above the target (as in the Poisson solve); if the iteration
+            // converges all the same, they go unused
+            auto next_direction = [&]() {
+                launch_hmg_vcycle32(P, c->hmg, r32, z32, nu1, nu2, 8, omega, c->st);
+                // flexible CG(1): beta = -(z . q) / (d . q) with the new z
+                launch_dot2<float>(n, z32, r32, q32, c->partials, c->st, FinSpec{c->scal, 2, 0, FIN_FCG_BETA, 0.0});
+                launch_xpby<float>(n, c->scal, z32, d32, c->st);
+            };
+            const bool ahead = prev_in_rr * 1e-3 > target;
+            if (ahead) next_direction();
             CK(cudaGetLastError());
-            s = read_scal(c);
+            s = read_scal_wait(c);
             if (s != PARIS_OK) return s;
             ++iters;
             const double in_rr = c->scal_h->red[0];
             if (!(in_rr == in_rr) || c->scal_h->red[2] > 0) break;  // non-finite: the FP64 residual decides
             if (in_rr <= target || in_rr > 1e6 * rr32) break;
-            launch_hmg_vcycle32(P, c->hmg, r32, z32, nu1, nu2, 8, omega, c->st);
-            // flexible CG(1): beta = -(z . q) / (d . q) with the new z
-            launch_dot2<float>(n, z32, r32, q32, c->partials, c->st, FinSpec{c->scal, 2, 0, FIN_FCG_BETA, 0.0});
-            launch_xpby<float>(n, c->scal, z32, d32, c->st);
+            prev_in_rr = in_rr;
+            if (!ahead) next_direction();
         }
         launch_hmg_accumulate(g, e32, c->scal, us, c->st);  // u* += e / scale
         CK(cudaGetLastError());

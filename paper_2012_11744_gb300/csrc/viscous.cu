@@ -30,7 +30,7 @@
 // divisions), the column's values carried from plane to plane.
 #include <algorithm>
 
-#include "kernels.cuh"
+#include "helm.cuh"
 
 namespace paris {
 
@@ -38,64 +38,6 @@ namespace {
 
 constexpr int kTX = 32, kTY = 8;  // tile of the marching kernels
 constexpr int kPerSM = 4;         // their resident blocks per SM (at most 64 registers)
-
-// The column (i, j) of unknowns over planes [k0, k1) of an array x with
-// strides st: base points at (i, j, 0).  next(k) returns Lap_h x / ih2 at
-// plane k: the neighbours present (or wrapped) summed, minus the diagonal
-// count times the value: 2 an axis, one more at a no-slip end (ghost value
-// minus the end value), 0 along a periodic axis of one point.
-struct HelmColumn {
-    const double* base;
-    int64_t sz, oxm, oxp, oym, oyp;  // plane stride; offsets of the x and y neighbours
-    bool hxm, hxp, hym, hyp;         // which of them exist
-    int m2, kz;                      // planes and the kind of the z axis
-    double dxy;                      // diagonal count of the x and y axes
-    double zm, zc;
-
-    __device__ __forceinline__ HelmColumn(const HelmGeo& g, const double* x, const int64_t (&st)[3], int i, int j,
-                                          int k0) {
-        base = x + i * st[0] + j * st[1];
-        sz = st[2];
-        auto axis = [&](int a, int p, bool& hm, bool& hp, int64_t& om, int64_t& op) {
-            const int m = g.m[a];
-            const bool per = g.kind[a] == HELM_PERIODIC;
-            hm = per ? m > 1 : p > 0;
-            hp = per ? m > 1 : p < m - 1;
-            om = p > 0 ? -st[a] : (int64_t)(m - 1) * st[a];
-            op = p < m - 1 ? st[a] : -(int64_t)(m - 1) * st[a];
-            return (double)count(g.kind[a], m, p);
-        };
-        dxy = axis(0, i, hxm, hxp, oxm, oxp) + axis(1, j, hym, hyp, oym, oyp);
-        m2 = g.m[2];
-        kz = g.kind[2];
-        zc = base[k0 * sz];
-        zm = below(k0);
-    }
-    __device__ __forceinline__ static int count(int kind, int m, int p) {
-        if (kind == HELM_PERIODIC) return m > 1 ? 2 : 0;
-        return 2 + (kind == HELM_NOSLIP ? (p == 0) + (p == m - 1) : 0);
-    }
-    __device__ __forceinline__ double below(int k) const {
-        if (k > 0) return base[(k - 1) * sz];
-        return kz == HELM_PERIODIC && m2 > 1 ? base[(m2 - 1) * sz] : 0.0;
-    }
-    __device__ __forceinline__ double above(int k) const {
-        if (k < m2 - 1) return base[(k + 1) * sz];
-        return kz == HELM_PERIODIC && m2 > 1 ? base[0] : 0.0;
-    }
-    __device__ __forceinline__ double next(int k, double& xc) {
-        const double* c = base + k * sz;
-        const double xm = hxm ? c[oxm] : 0.0, xp = hxp ? c[oxp] : 0.0;
-        const double ym = hym ? c[oym] : 0.0, yp = hyp ? c[oyp] : 0.0;
-        const double zp = above(k);
-        xc = zc;
-        const double dg = dxy + (double)count(kz, m2, k);
-        const double s = ((xm + xp) + (ym + yp)) + (zm + zp);
-        zm = zc;
-        zc = zp;
-        return fma(-dg, xc, s);
-    }
-};
 
 __device__ __forceinline__ int64_t helm_block() {
     return ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
@@ -303,32 +245,70 @@ __global__ void helm_direction_kernel(int64_t n, const Scal* __restrict__ s, con
     }
 }
 
+// a / b for positive a and b, correctly rounded: y = 1/b to one ulp (recip64),
+// q = a y, and one step with the exact remainder, q + (a - b q) y (Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000", 1990).
+// 6 FP64 instructions; outside the window in which no intermediate over- or
+// underflows, the division.
+__device__ __forceinline__ double div_pos(double a, double b) {
+    const int ha = __double2hiint(a), hb = __double2hiint(b);
+    if (ha < (700 << 20) || ha >= (1300 << 20) || hb < (900 << 20) || hb >= (1140 << 20)) return a / b;
+    const double y = recip64(b), q = a * y;
+    return fma(fma(-b, q, a), y, q);
+}
+
 // nu_f = (mu_L + mu_R) / (rho_L + rho_R) on every face of the component,
 // mu and rho from Eq. muH in the two cells sharing the face; 0 on its wall
 // faces.  Rounded products and sums (no contraction), in the order written.
-__global__ void helm_face_nu_kernel(HelmGeo g, int64_t nfull, int nx, int ny, const double* __restrict__ C,
-                                    double mu1, double mu2, double rho1, double rho2, double* __restrict__ nu) {
-    const int c = g.comp;
-    for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < nfull; f += (int64_t)gridDim.x * blockDim.x) {
-        int pos[3];
-        const int64_t t = f / g.e[0];
-        pos[0] = (int)(f - t * g.e[0]);
-        pos[1] = (int)(t % g.e[1]);
-        pos[2] = (int)(t / g.e[1]);
-        if (g.wall && (pos[c] == 0 || pos[c] == g.e[c] - 1)) {
-            nu[f] = 0.0;
-            continue;
+// Bound by the FP64 pipe: a cell's mu and rho (7 instructions) are formed once
+// and reach its other face through the plane before (z), the warp (x) or the
+// tile (y), where every face formed both cells' (788 -> 572 us at 256^3).
+__global__ void __launch_bounds__(kTX* kTY, kPerSM) helm_face_nu_kernel(HelmGeo g, int nx, int ny, int nz,
+                                                                       const double* __restrict__ C, double mu1,
+                                                                       double mu2, double rho1, double rho2,
+                                                                       double* __restrict__ nu, int zper) {
+    __shared__ double2 sh[2][kTY][kTX];  // (mu, rho) of the tile's cells, by plane parity
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    const int i = blockIdx.x * kTX + tx, j = blockIdx.y * kTY + ty, comp = g.comp;
+    const int ic = min(i, nx - 1), jc = min(j, ny - 1);  // idle threads shadow a cell
+    const int k0 = blockIdx.z * zper, k1 = min(k0 + zper, nz);
+    const bool in = i < nx && j < ny;
+    auto cell = [&](int ci, int cj, int ck) {
+        const double c = C[((int64_t)ck * ny + cj) * nx + ci], d = __dsub_rn(1.0, c);
+        return make_double2(__dadd_rn(__dmul_rn(mu1, c), __dmul_rn(mu2, d)),
+                            __dadd_rn(__dmul_rn(rho1, c), __dmul_rn(rho2, d)));
+    };
+    // the cell below the face along the component's axis: wrapped, or not read on a wall
+    const int im = ic > 0 ? ic - 1 : nx - 1, jm = jc > 0 ? jc - 1 : ny - 1;
+    const int pos0 = comp == 0 ? i : j;
+    double2 below = make_double2(0.0, 0.0);
+    if (comp == 2) below = cell(ic, jc, k0 > 0 ? k0 - 1 : nz - 1);
+    for (int k = k0; k < k1; ++k) {
+        const double2 here = cell(ic, jc, k);
+        double2 lo = below;
+        if (comp == 0) {
+            lo = make_double2(__shfl_up_sync(0xffffffffu, here.x, 1), __shfl_up_sync(0xffffffffu, here.y, 1));
+            if (tx == 0) lo = cell(im, jc, k);
+        } else if (comp == 1) {
+            sh[k & 1][ty][tx] = here;
+            __syncthreads();
+            lo = ty > 0 ? sh[k & 1][ty - 1][tx] : cell(ic, jm, k);
         }
-        // face pos[c] lies between cells pos[c]-1 (wrapped along a periodic axis) and pos[c]
-        int lo[3] = {pos[0], pos[1], pos[2]};
-        lo[c] = pos[c] > 0 ? pos[c] - 1 : g.e[c] - 1;
-        const double cl = C[((int64_t)lo[2] * ny + lo[1]) * nx + lo[0]];
-        const double cr = C[((int64_t)pos[2] * ny + pos[1]) * nx + pos[0]];
-        const double mul = __dadd_rn(__dmul_rn(mu1, cl), __dmul_rn(mu2, __dsub_rn(1.0, cl)));
-        const double mur = __dadd_rn(__dmul_rn(mu1, cr), __dmul_rn(mu2, __dsub_rn(1.0, cr)));
-        const double rhol = __dadd_rn(__dmul_rn(rho1, cl), __dmul_rn(rho2, __dsub_rn(1.0, cl)));
-        const double rhor = __dadd_rn(__dmul_rn(rho1, cr), __dmul_rn(rho2, __dsub_rn(1.0, cr)));
-        nu[f] = __dadd_rn(mul, mur) / __dadd_rn(rhol, rhor);
+        below = here;
+        const int pos = comp == 2 ? k : pos0;
+        if (in) {
+            const int64_t f = i + (int64_t)g.e[0] * (j + (int64_t)g.e[1] * k);
+            nu[f] = g.wall && pos == 0 ? 0.0 : div_pos(__dadd_rn(lo.x, here.x), __dadd_rn(lo.y, here.y));
+        }
+    }
+    // the far wall face of the component's axis
+    if (g.wall && in) {
+        const int64_t se[3] = {1, g.e[0], (int64_t)g.e[0] * g.e[1]};
+        if (comp == 2) {
+            if (k1 == nz) nu[i + se[1] * j + se[2] * nz] = 0.0;
+        } else if (pos0 == (comp == 0 ? nx : ny) - 1) {
+            for (int k = k0; k < k1; ++k) nu[i + se[1] * j + se[2] * k + se[comp]] = 0.0;
+        }
     }
 }
 
@@ -412,9 +392,10 @@ void launch_helm_direction(int64_t n, const Scal* s, const double* w, const doub
 
 void launch_helm_face_nu(const HelmGeo& g, const Geo& g0, const double* C, double mu1, double mu2, double rho1,
                          double rho2, double* nu, cudaStream_t st) {
-    const int64_t nfull = helm_faces(g);
-    helm_face_nu_kernel<<<elementwise_blocks(nfull), kRedThreads, 0, st>>>(g, nfull, g0.nx, g0.ny, C, mu1, mu2,
-                                                                           rho1, rho2, nu);
+    const int tx = (g0.nx + kTX - 1) / kTX, ty = (g0.ny + kTY - 1) / kTY;
+    const int zper = march_planes((int64_t)tx * ty, g0.nz, kPerSM);
+    helm_face_nu_kernel<<<dim3(tx, ty, (g0.nz + zper - 1) / zper), dim3(kTX, kTY), 0, st>>>(
+        g, g0.nx, g0.ny, g0.nz, C, mu1, mu2, rho1, rho2, nu, zper);
     count_launch();
 }
 
