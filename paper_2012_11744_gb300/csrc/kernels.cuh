@@ -526,16 +526,18 @@ struct TailLevel {
     const T* by;
     const T* bz;
     const T* w;
+    const T* sig;  // diagonal excess, or null
     T* x;
     T* f;
 };
 constexpr int kMaxTail = 16;         // levels in one tail launch
 constexpr int kMaxDenseCells = 128;  // cells of a dense coarsest level
 // The V-cycle from levels[0] (its f already restricted from above) down to
-// the dense coarsest levels[n-1] (inverse Minv) and back: one block.
+// the dense coarsest levels[n-1] (inverse Minv) and back: one block.  term:
+// scratch of a value per cell of levels[0].
 template <typename T>
 void launch_tail_vcycle(const TailLevel<T>* levels, int n, const double* Minv, double omega, int nu1,
-                        int nu2, bool use_w, cudaStream_t st);
+                        int nu2, T* term, bool keep_mean, cudaStream_t st);
 
 // ------------------------------------------------------------ Krylov ------
 // r = f - A x (FP64), optional r32 = scale * r; partials (||r||^2, max|r|, nonfinite).

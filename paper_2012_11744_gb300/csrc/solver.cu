@@ -45,7 +45,7 @@ struct Level {
     double* t64 = nullptr;
     double* sig64 = nullptr;  // diagonal excess of a Dirichlet-coupled operator (levels >= 1, on first use)
     float* sig32 = nullptr;   // its FP32 copy for the mixed form's V-cycle
-    __half* b16[3] = {nullptr, nullptr, nullptr};  // level 1 of the mixed step: FP16 coefficients (see half1)
+    __half* b16[3] = {nullptr, nullptr, nullptr};  // level 1 of the mixed step: FP16 coefficients
     float scale16 = 1.f;                           // their scale (the coefficient is b16 * scale16)
 };
 
@@ -146,8 +146,8 @@ struct paris_ctx {
     // CUDA graphs of the coarse part of the V-cycle (index 0: FP32, 1: FP64)
     cudaStream_t cap_stream = nullptr;
     bool cap_stream_broken = false;
-    cudaGraphExec_t cg_exec[3] = {nullptr, nullptr, nullptr};
-    int cg_kernels[3] = {0, 0, 0};
+    cudaGraphExec_t cg_exec[5] = {};
+    int cg_kernels[5] = {};
 };
 
 namespace {
@@ -380,8 +380,14 @@ Coef<T> level_coef(paris_ctx* c, int l, const Coef<T>& c0) {
     return cf;
 }
 
-int tail_start(const paris_ctx* c);
+// Levels with at most this many cells, down to the dense coarsest level, run
+// as one single-block launch (launch_tail_vcycle).  8^3 cells: a pass on 16^3
+// takes one SM longer than its launch on the whole chip (FP64: 5 us on the SM's
+// two instructions a clock; the general kernel took 97 us a V-cycle from 16^3
+// and 26 from 8^3, FP32 37 and 17).
+constexpr int64_t kTailCells = 512;
 
+int tail_start(const paris_ctx* c);
 // Per-solve set-up of the hierarchy in precision T: coarse coefficients,
 // inverse diagonals, dense coarsest inverse.
 template <typename T>
@@ -631,22 +637,12 @@ void vup(paris_ctx* c, const Coef<T>& c0, const T* f0, T* x0, int l) {
     if (o.nu2 > 0) smooth<T>(c, l, cf, f, x, o.nu2, false, true);
 }
 
-// Levels with at most this many cells, down to the dense coarsest level,
-// run as one single-block launch (launch_tail_vcycle).
-#ifndef PARIS_TAIL_CELLS
-#define PARIS_TAIL_CELLS 4096
-#endif
-constexpr int64_t kTailCells = PARIS_TAIL_CELLS;
-
-// First level of that tail, or -1 (the tail needs the two-pass red-black
-// smoother and at least one level above the dense coarsest).
+// First level of that launch, or -1 (it needs the two-pass red-black smoother
+// and at least one level above the dense coarsest).
 int tail_start(const paris_ctx* c) {
     const int nl = (int)c->lv.size();
-    if (c->opts.coarse_tail == 0 || c->opts.smoother != PARIS_SMOOTH_RBGS_2PASS || nl < 3 ||
-        c->dirichlet)
-        return -1;
-    // level 1 with FP16 coefficients (the mixed step's FP16 rho/2) keeps its own kernels
-    const int lo = (c->rho0 && c->half_rho) ? 2 : 1;
+    if (c->opts.coarse_tail == 0 || c->opts.smoother != PARIS_SMOOTH_RBGS_2PASS || nl < 3) return -1;
+    const int lo = (c->rho0 && c->half_rho) ? 2 : 1;  // level 1 with FP16 coefficients keeps its own kernels
     int t = nl - 1;
     while (t - 1 >= lo && c->lv[t - 1].g.ncell() <= kTailCells) --t;
     if (t >= nl - 1 || nl - t > kMaxTail) return -1;
@@ -672,10 +668,12 @@ void launch_tail(paris_ctx* c, int t) {
         d.by = Prec<T>::b(L, 1);
         d.bz = Prec<T>::b(L, 2);
         d.w = Prec<T>::w(L);  // the inverse diagonals (set up with the hierarchy)
+        d.sig = c->dirichlet ? Prec<T>::sig(L) : nullptr;
         d.x = Prec<T>::x(L);
         d.f = Prec<T>::f(L);
     }
-    launch_tail_vcycle<T>(tl, nl - t, c->coarse_inv, c->opts.omega, c->opts.nu1, c->opts.nu2, true, c->st);
+    launch_tail_vcycle<T>(tl, nl - t, c->coarse_inv, c->opts.omega, c->opts.nu1, c->opts.nu2,
+                          Prec<T>::t(c->lv[t]), c->dirichlet, c->st);
 }
 
 // Levels 1 .. L-1 of the V-cycle (level 0's restriction already done).
@@ -703,8 +701,9 @@ void coarse_part(paris_ctx* c, const Coef<T>& c0) {
 template <typename T>
 bool coarse_graph_launch(paris_ctx* c, const Coef<T>& c0) {
     const int nl = (int)c->lv.size();
-    // FP32 graphs with level 1 from the FP32 or from the FP16 coefficients, FP64
-    const int slot = sizeof(T) == 8 ? 1 : ((c->rho0 && c->half_rho) ? 2 : 0);
+    // FP32 graphs with level 1 from the FP32 or from the FP16 coefficients, FP64;
+    // the two precisions with a diagonal excess
+    const int slot = c->dirichlet ? (sizeof(T) == 8 ? 4 : 3) : (sizeof(T) == 8 ? 1 : ((c->rho0 && c->half_rho) ? 2 : 0));
     if (nl < 3 || !c->cap_stream) return false;
     if (!c->cg_exec[slot]) {
         cudaStream_t user = c->st;
@@ -737,7 +736,7 @@ bool coarse_graph_launch(paris_ctx* c, const Coef<T>& c0) {
 template <typename T>
 void vcycle(paris_ctx* c, const Coef<T>& c0, const T* f0, T* x0) {
     const int nl = (int)c->lv.size();
-    if (nl >= 3 && !c->cap_stream_broken && !c->dirichlet) {
+    if (nl >= 3 && !c->cap_stream_broken) {
         vdown<T>(c, c0, f0, x0, 0);
         {
             ProfScope ps(c, PARIS_K_COARSE, 0.0);
@@ -1137,6 +1136,9 @@ paris_status paris_set_opts(paris_ctx* c, const paris_opts* o) {
         if (c->scal_h) cudaFreeHost(c->scal_h);
         c->scal_h = nullptr;
         c->hC = c->hu = c->hv = c->hw = c->hp = nullptr;
+        c->sig0 = nullptr;  // the free-surface arrays went with the rest: allocated anew on their next use
+        c->sig32_0 = nullptr;
+        c->fs_cls = c->fs_tmp = nullptr;
         c->opts = *o;
         return alloc_ctx(c);
     }

@@ -193,3 +193,26 @@ def test_free_surface_rejects_invalid_arguments(paris):
         with pytest.raises(paris.ParisError):
             ctx.phantom_projection(C, *u)
         ctx.set_solid(None)
+
+
+@pytest.mark.parametrize("precision", ["FP64", "MIXED"])
+@pytest.mark.parametrize("grid", [pi.Grid(32, 32, 32, 1 / 32, (P, W, P)), pi.Grid(24, 20, 16, 1 / 24, (P, W, W)),
+                                  pi.Grid(33, 12, 14, 1 / 33, (W, W, W))],
+                         ids=lambda g: f"{g.nx}x{g.ny}x{g.nz}")
+def test_free_surface_tail_bit_identical(paris, grid, precision):
+    """The smallest levels with a diagonal excess in one launch and by their
+    own kernels: the same arithmetic in the same order (periodic axes even on
+    every smoothed level)."""
+    pr, theta, kappa, p_gas = bubbles(grid, seed=83)
+    out = []
+    for tail in (0, 1):
+        opts = paris.default_opts(precision=getattr(paris, precision), coarse_tail=tail)
+        with paris.Context(grid, opts=opts) as ctx:
+            u = [dev(x) for x in (pr.u, pr.v, pr.w)]
+            p = torch.zeros(grid.shape, dtype=torch.float64, device="cuda")
+            st = ctx.free_surface_step(dev(pr.C), 1000.0, 1e-3, *u, p, p_gas=dev(p_gas),
+                                       theta=[dev(t) for t in theta], kappa=dev(kappa), sigma=0.07)
+            assert st["converged"] == 1, (tail, st)
+            out.append([host(p)] + [host(x) for x in u])
+    for a, b in zip(*out):
+        np.testing.assert_array_equal(a, b)
