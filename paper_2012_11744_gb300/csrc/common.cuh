@@ -289,6 +289,10 @@ __device__ __forceinline__ unsigned fast_div(unsigned p, unsigned d, unsigned m)
 // earlier kernel writes.  Without the launch attribute the wait returns at
 // once.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the kernel after this one start while this one still runs, as far as
+// its pdl_wait(): for grids that leave most of the chip idle, followed by
+// kernels with work of their own before the wait.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ------------------------------------------------------------ reductions ---
 

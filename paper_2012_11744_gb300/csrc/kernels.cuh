@@ -539,6 +539,19 @@ template <typename T>
 void launch_tail_vcycle(const TailLevel<T>* levels, int n, const double* Minv, double omega, int nu1,
                         int nu2, T* term, bool keep_mean, cudaStream_t st);
 
+// ------------------------------------------- a small level in one launch ----
+// The launches below serve a level of at most 32^3 cells (FP64: 8192) whose periodic
+// axes are even and whose smoothing phases are one or two sweeps (boxes.cu).
+bool box_level_fits(const Geo& g, int nu1, int nu2, bool fp64);
+// Level g with coefficients b (times scale), inverse diagonals w (null: from b)
+// and diagonal excess sig (or null), coarsened by fac to cg.  Down (up false):
+// x = the pre-smoothed zero, fc = the restricted residual.  Up: x = xin plus the
+// parents' xc, post-smoothed; x must not be xin.
+template <typename T, typename TB>
+void launch_box_level(const Geo& g, const TB* const b[3], T scale, const T* w, const T* sig, const T* f, const Geo& cg,
+                      const int fac[3], bool up, const T* xin, T* x, T* fc, const T* xc, double omega, int sweeps,
+                      cudaStream_t st);
+
 // ------------------------------------------------------------ Krylov ------
 // r = f - A x (FP64), optional r32 = scale * r; partials (||r||^2, max|r|, nonfinite).
 // zero_ok: x is the initial guess whose max |x| the prologue stored in s->xmax;

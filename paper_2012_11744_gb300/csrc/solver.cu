@@ -676,20 +676,51 @@ void launch_tail(paris_ctx* c, int t) {
                           Prec<T>::t(c->lv[t]), c->dirichlet, c->st);
 }
 
+// Whether level l (above the tail) runs as one launch down and one up: the
+// levels of box_level_fits, with the tail's smoother and switch.
+bool box_level(const paris_ctx* c, int l, bool fp64) {
+    return c->opts.coarse_tail != 0 && c->opts.smoother == PARIS_SMOOTH_RBGS_2PASS && l >= 1 &&
+           l + 1 < (int)c->lv.size() && box_level_fits(c->lv[l].g, c->opts.nu1, c->opts.nu2, fp64);
+}
+
+// Level l's half of the V-cycle as one launch; the pre-smoothed x waits in the
+// level's second buffer (neighbouring blocks read it while x is written).
+template <typename T>
+void box_pass(paris_ctx* c, int l, bool up) {
+    Level& L = c->lv[l];
+    Level& C = c->lv[l + 1];
+    T* t = Prec<T>::t(L);
+    T* out = up ? Prec<T>::x(L) : t;
+    const int sweeps = up ? c->opts.nu2 : c->opts.nu1;
+    if constexpr (sizeof(T) == 4) {
+        if (l == 1 && c->rho0 && c->half_rho) {
+            launch_box_level<float, __half>(L.g, L.b16, L.scale16, nullptr, nullptr, L.f32, C.g, C.fac, up, t, out, C.f32,
+                                            C.x32, c->opts.omega, sweeps, c->st);
+            return;
+        }
+    }
+    const T* const b[3] = {Prec<T>::b(L, 0), Prec<T>::b(L, 1), Prec<T>::b(L, 2)};
+    // as the colour passes: 1/D read in FP64 and with a diagonal excess, else from the coefficients
+    const T* w = sizeof(T) == 8 || c->dirichlet ? Prec<T>::w(L) : nullptr;
+    launch_box_level<T, T>(L.g, b, T(1), w, c->dirichlet ? Prec<T>::sig(L) : nullptr, Prec<T>::f(L), C.g, C.fac, up, t, out,
+                           Prec<T>::f(C), Prec<T>::x(C), c->opts.omega, sweeps, c->st);
+}
+
 // Levels 1 .. L-1 of the V-cycle (level 0's restriction already done).
 template <typename T>
 void coarse_part(paris_ctx* c, const Coef<T>& c0) {
     const int nl = (int)c->lv.size();
-    const int t = tail_start(c);
-    if (t > 0) {
-        for (int l = 1; l < t; ++l) vdown<T>(c, c0, nullptr, nullptr, l);
-        launch_tail<T>(c, t);
-        for (int l = t - 1; l >= 1; --l) vup<T>(c, c0, nullptr, nullptr, l);
-        return;
+    const int t = tail_start(c), end = t > 0 ? t : nl - 1;
+    for (int l = 1; l < end; ++l) {
+        if (box_level(c, l, sizeof(T) == 8)) box_pass<T>(c, l, false);
+        else vdown<T>(c, c0, nullptr, nullptr, l);
     }
-    for (int l = 1; l < nl - 1; ++l) vdown<T>(c, c0, nullptr, nullptr, l);
-    vcoarse<T>(c, nullptr, nullptr);
-    for (int l = nl - 2; l >= 1; --l) vup<T>(c, c0, nullptr, nullptr, l);
+    if (t > 0) launch_tail<T>(c, t);
+    else vcoarse<T>(c, nullptr, nullptr);
+    for (int l = end - 1; l >= 1; --l) {
+        if (box_level(c, l, sizeof(T) == 8)) box_pass<T>(c, l, true);
+        else vup<T>(c, c0, nullptr, nullptr, l);
+    }
 }
 
 // The part of the V-cycle below level 0 (levels 1 .. L-1) only reads and

@@ -323,7 +323,7 @@ struct Pair {
 };
 
 template <typename T>
-__device__ __forceinline__ void pair_load(Pair<T>& o, const TailLevel<T>& L, const TailLevel<T>& C, bool with_f) {
+__device__ __forceinline__ void pair_load(Pair<T>& o, const TailLevel<T>& L, const TailLevel<T>& C) {
     const Geo g = L.g, cg = C.g;
     const unsigned npair = (unsigned)(g.nx + 1) / 2, t = threadIdx.x;
     o.c = -1;
@@ -368,7 +368,7 @@ __device__ __forceinline__ void pair_load(Pair<T>& o, const TailLevel<T>& L, con
                 o.bz[m][0] = s.b[4];
                 o.bz[m][1] = s.b[5];
                 o.w[m] = L.w[c];
-                o.f[m] = with_f ? L.f[c] : T(0);
+                o.f[m] = T(0);
                 o.sig[m] = L.sig ? L.sig[c] : T(0);
                 o.mask[m] = (unsigned char)mask;
                 o.par[m] = (short)((K * cg.ny + J) * cg.nx + I);
@@ -494,7 +494,7 @@ __device__ __forceinline__ void small_restrict(const Geo& fg, const TailLevel<T>
 // NH: smoothed levels (1 or 2) above the dense one.
 template <typename T, int NH>
 __global__ void __launch_bounds__(kSmallThreads) tail_small_kernel(const __grid_constant__ TailArgs<T> a) {
-    pdl_wait();
+    pdl_trigger();
     constexpr int kMax = 2 * kSmallThreads;  // cells of 256 pairs
     __shared__ T x[NH][kMax], term[kMax], f1[kMax], fc[kMaxDenseCells], xc[kMaxDenseCells];
     __shared__ double fs[kMaxDenseCells], mean;
@@ -505,12 +505,15 @@ __global__ void __launch_bounds__(kSmallThreads) tail_small_kernel(const __grid_
     if (small)
         for (int e = threadIdx.x; e < nd * nd; e += kSmallThreads) async_copy(Ms + e, a.Minv + e);
     Pair<T> o0, o1;
-    pair_load(o0, a.L[0], a.L[1], true);
-    if (NH == 2) pair_load(o1, a.L[1], a.L[2], false);
+    pair_load(o0, a.L[0], a.L[1]);
+    if (NH == 2) pair_load(o1, a.L[1], a.L[2]);
     for (int t = threadIdx.x; t < kMax; t += kSmallThreads)
         for (int l = 0; l < NH; ++l) x[l][t] = T(0);
     const double rn = 1.0 / (double)nd;  // exact when nd is a power of two
     asm volatile("cp.async.wait_all;" ::: "memory");
+    pdl_wait();  // the first level's right-hand side: what the preceding launch wrote
+    pair_rhs<0>(o0, a.L[0].f);
+    pair_rhs<1>(o0, a.L[0].f);
     __syncthreads();
     const bool sig = a.L[0].sig != nullptr;
     pair_smooth(o0, x[0], a.nu1, true, false, a.omega);
