@@ -78,7 +78,7 @@ template <typename T, typename TB>
 struct BoxArgs {
     Geo g, cg;
     int fac[3], tc[3];  // coarsening factors; coarse cells of a box along each axis
-    const TB* b[3];
+    const TB* b[3];  // coefficients, or rho/2 in b[0]
     const T* w;    // inverse diagonals (null: from the coefficients)
     const T* sig;  // diagonal excess, or null
     const T* f;
@@ -86,9 +86,23 @@ struct BoxArgs {
     T* x;
     T* fc;         // down: the coarse right-hand side
     const T* xc;   // up: the coarse solution
-    T scale, omega;
+    T hs, rs;      // the right-hand side's factor in a pass; the operator's in the residual
+    T omega;
     int sweeps;    // 1 or 2
 };
+
+__device__ __forceinline__ float2 ld_pair(const float* p) { return __ldg(reinterpret_cast<const float2*>(p)); }
+__device__ __forceinline__ float2 ld_pair(const __half* p) {
+    return __half22float2(__ldg(reinterpret_cast<const __half2*>(p)));
+}
+__device__ __forceinline__ float2 ld_pair(const double*) { return {}; }  // FP64 levels have face arrays
+
+__device__ __forceinline__ float box_rcp(float v) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(v));
+    return y;
+}
+__device__ __forceinline__ double box_rcp(double v) { return v; }
 
 // index i of an axis of n, wrapped around if it is periodic; -1: beyond a wall
 __device__ __forceinline__ int box_wrap(int i, int n, int wall) {
@@ -111,15 +125,21 @@ struct BoxPair {
     bool black;  // the left cell is black
 };
 
-// Colour pass M over the cells at most D steps from the box.
-template <typename T, typename B, int M, int D>
+// Colour pass M over the cells at most D steps from the box (RHO: the pass of
+// tile_update, which takes a cell's x-face outside its pair first).
+template <typename T, typename B, int M, int D, bool RHO>
 __device__ __forceinline__ void box_pass(const BoxPair<T>& o, T* x, T hs, bool scaled, T omega) {
     if (o.d[M] <= D) {
         const bool right = o.black == (M == 0);
         const int c = o.c + (right ? 1 : 0);
         T acc = scaled ? o.f[M] * hs : o.f[M];
-        acc = fma(right ? o.bx[1] : o.bx[0], x[c - 1], acc);
-        acc = fma(right ? o.bx[2] : o.bx[1], x[c + 1], acc);
+        if (RHO) {
+            acc = fma(right ? o.bx[2] : o.bx[0], x[right ? c + 1 : c - 1], acc);
+            acc = fma(o.bx[1], x[right ? c - 1 : c + 1], acc);
+        } else {
+            acc = fma(right ? o.bx[1] : o.bx[0], x[c - 1], acc);
+            acc = fma(right ? o.bx[2] : o.bx[1], x[c + 1], acc);
+        }
         acc = fma(o.by[M][0], x[c - B::bx], acc);
         acc = fma(o.by[M][1], x[c + B::bx], acc);
         acc = fma(o.bz[M][0], x[c - B::bx * B::by], acc);
@@ -131,11 +151,14 @@ __device__ __forceinline__ void box_pass(const BoxPair<T>& o, T* x, T hs, bool s
 }
 
 // UP: prolongation and post-smoothing; else pre-smoothing and restriction.
-template <typename T, typename TB, int TX, int TY, int TZ, bool UP>
+// RHO: the finest level of the mixed step, coefficients 1/(rh_L + rh_R) from
+// rho/2 and vectors in the colour-split layout, with the arithmetic of
+// tile_update and op_rho_tile_kernel.
+template <typename T, typename TB, int TX, int TY, int TZ, bool UP, bool RHO>
 __global__ void __launch_bounds__(Box<TX, TY, TZ>::threads, Box<TX, TY, TZ>::threads <= 512 ? 2 : 1)
     box_kernel(const __grid_constant__ BoxArgs<T, TB> a) {
     using B = Box<TX, TY, TZ>;
-    constexpr bool kScaled = sizeof(TB) == 2;
+    constexpr bool kScaled = RHO || sizeof(TB) == 2;
     __shared__ T x[B::cells];
     __shared__ T term[UP ? 1 : TX * TY * TZ];
     const int tid = threadIdx.x;
@@ -165,7 +188,31 @@ __global__ void __launch_bounds__(Box<TX, TY, TZ>::threads, Box<TX, TY, TZ>::thr
     T bl = T(0), bm = T(0), br = T(0);
     T byl[2] = {T(0), T(0)}, byr[2] = {T(0), T(0)}, bzl[2] = {T(0), T(0)}, bzr[2] = {T(0), T(0)};
     T fl = T(0), fr = T(0), wl = T(0), wr = T(0), xl = T(0), xr = T(0);
-    if (inl) {
+    if constexpr (RHO) {
+        if (inl) {  // even axes: the pair is whole
+            const TB* p = a.b[0] + c;
+            const int jm = j > 0 ? -g.nx : (g.ny - 1) * g.nx, jp = j + 1 < g.ny ? g.nx : -(g.ny - 1) * g.nx;
+            const int pl = g.nx * g.ny;
+            const int km = k > 0 ? -pl : (g.nz - 1) * pl, kp = k + 1 < g.nz ? pl : -(g.nz - 1) * pl;
+            const float2 r = ld_pair(p), rym = ld_pair(p + jm), ryp = ld_pair(p + jp), rzm = ld_pair(p + km);
+            const float2 rzp = ld_pair(p + kp);
+            const float rl = (float)ldc(p + (i > 0 ? -1 : g.nx - 1)), rr = (float)ldc(p + (i + 2 < g.nx ? 2 : 2 - g.nx));
+            const bool y0 = g.wy && j == 0, y1 = g.wy && j == g.ny - 1, z0 = g.wz && k == 0, z1 = g.wz && k == g.nz - 1;
+            bl = g.wx && i == 0 ? T(0) : (T)box_rcp(r.x + rl);
+            bm = (T)box_rcp(r.x + r.y);
+            br = g.wx && i + 2 == g.nx ? T(0) : (T)box_rcp(r.y + rr);
+            byl[0] = y0 ? T(0) : (T)box_rcp(r.x + rym.x);
+            byr[0] = y0 ? T(0) : (T)box_rcp(r.y + rym.y);
+            byl[1] = y1 ? T(0) : (T)box_rcp(r.x + ryp.x);
+            byr[1] = y1 ? T(0) : (T)box_rcp(r.y + ryp.y);
+            bzl[0] = z0 ? T(0) : (T)box_rcp(r.x + rzm.x);
+            bzr[0] = z0 ? T(0) : (T)box_rcp(r.y + rzm.y);
+            bzl[1] = z1 ? T(0) : (T)box_rcp(r.x + rzp.x);
+            bzr[1] = z1 ? T(0) : (T)box_rcp(r.y + rzp.y);
+            wl = box_rcp(((bl + bm) + (byl[0] + byl[1])) + (bzl[0] + bzl[1]));
+            wr = box_rcp(((br + bm) + (byr[0] + byr[1])) + (bzr[0] + bzr[1]));
+        }
+    } else if (inl) {
         const TB* p = a.b[0] + row * (g.nx + g.wx) + i;
         if (!(g.wx && i == 0)) bl = (T)ldc(p);
         if (inr) bm = (T)ldc(p + 1);
@@ -193,12 +240,15 @@ __global__ void __launch_bounds__(Box<TX, TY, TZ>::threads, Box<TX, TY, TZ>::thr
     }
     // what the preceding launches of the V-cycle wrote
     pdl_wait();
+    // the pair's entries in the vectors: side by side, or one in each half of a split row
+    const int hx = g.nx / 2, cl = RHO ? row * g.nx + i / 2 + (o.black ? hx : 0) : c;
+    const int cr = RHO ? row * g.nx + i / 2 + (o.black ? 0 : hx) : c + 1;
     if (inl) {
-        fl = a.f[c];
-        if (UP) xl = a.xin[c];
+        fl = a.f[cl];
+        if (UP) xl = a.xin[cl];
         if (inr) {
-            fr = a.f[c + 1];
-            if (UP) xr = a.xin[c + 1];
+            fr = a.f[cr];
+            if (UP) xr = a.xin[cr];
         }
         if (UP) {
             const int pr = (parent_of(k, cg.nz, a.fac[2]) * cg.ny + parent_of(j, cg.ny, a.fac[1])) * cg.nx;
@@ -233,8 +283,8 @@ __global__ void __launch_bounds__(Box<TX, TY, TZ>::threads, Box<TX, TY, TZ>::thr
             inv = (a.fac[0] == 2 ? T(0.5) : T(1)) * (a.fac[1] == 2 ? T(0.5) : T(1)) * (a.fac[2] == 2 ? T(0.5) : T(1));
         }
     }
-    const T hs = kScaled ? T(1) / a.scale : T(1);
-    if (!a.w) {
+    const T hs = a.hs;
+    if (!RHO && !a.w) {
         const T s[6] = {bl, bm, byl[0], byl[1], bzl[0], bzl[1]}, t[6] = {bm, br, byr[0], byr[1], bzr[0], bzr[1]};
         wl = inv_sum6(s);
         wr = inv_sum6(t);
@@ -264,22 +314,22 @@ __global__ void __launch_bounds__(Box<TX, TY, TZ>::threads, Box<TX, TY, TZ>::thr
         }
     }
     __syncthreads();
-    box_pass<T, B, 1, 3>(o, x, hs, kScaled, a.omega);
+    box_pass<T, B, 1, 3, RHO>(o, x, hs, kScaled, a.omega);
     if (!UP) {
         if (a.sweeps == 2) {
-            box_pass<T, B, 0, 2>(o, x, hs, kScaled, a.omega);
-            box_pass<T, B, 1, 1>(o, x, hs, kScaled, a.omega);
+            box_pass<T, B, 0, 2, RHO>(o, x, hs, kScaled, a.omega);
+            box_pass<T, B, 1, 1, RHO>(o, x, hs, kScaled, a.omega);
         }
     } else {
-        box_pass<T, B, 0, 2>(o, x, hs, kScaled, a.omega);
+        box_pass<T, B, 0, 2, RHO>(o, x, hs, kScaled, a.omega);
         if (a.sweeps == 2) {
-            box_pass<T, B, 1, 1>(o, x, hs, kScaled, a.omega);
-            box_pass<T, B, 0, 0>(o, x, hs, kScaled, a.omega);
+            box_pass<T, B, 1, 1, RHO>(o, x, hs, kScaled, a.omega);
+            box_pass<T, B, 0, 0, RHO>(o, x, hs, kScaled, a.omega);
         }
     }
     if (core) {
-        a.x[c] = x[o.c];
-        if (inr) a.x[c + 1] = x[o.c + 1];
+        a.x[cl] = x[o.c];
+        if (inr) a.x[cr] = x[o.c + 1];
         if (!UP) {  // each cell's term of its parent's sum
             auto residual = [&](int M, int cl, T b0, T b1, unsigned mask) {
                 const T xc = x[cl];
@@ -291,7 +341,7 @@ __global__ void __launch_bounds__(Box<TX, TY, TZ>::threads, Box<TX, TY, TZ>::thr
                 if (mask & 16u) acc = fma(M ? o.bz[1][0] : o.bz[0][0], xc - x[cl - B::bx * B::by], acc);
                 if (mask & 32u) acc = fma(M ? o.bz[1][1] : o.bz[0][1], xc - x[cl + B::bx * B::by], acc);
                 const T f = M ? o.f[1] : o.f[0];
-                if (kScaled) return fma(-a.scale, acc, f);  // never with a diagonal excess
+                if (kScaled) return fma(-a.rs, acc, f);  // never with a diagonal excess
                 if (a.sig) acc = fma(a.sig[c + cl - o.c], xc, acc);
                 return f - acc;
             };
@@ -304,15 +354,21 @@ __global__ void __launch_bounds__(Box<TX, TY, TZ>::threads, Box<TX, TY, TZ>::thr
         __syncthreads();
         if (tc >= 0) {
             T sum = T(0);
-            for (int dk = 0; dk < tn2; ++dk)
-                for (int dj = 0; dj < tn1; ++dj)
-                    for (int di = 0; di < tn0; ++di) sum += term[tp + (dk * TY + dj) * TX + di];
+            if (RHO) {  // rows of both planes, then the two rows
+                const T* p = term + tp;
+                sum = ((p[0] + p[1]) + (p[TY * TX] + p[TY * TX + 1])) +
+                      ((p[TX] + p[TX + 1]) + (p[TY * TX + TX] + p[TY * TX + TX + 1]));
+            } else {
+                for (int dk = 0; dk < tn2; ++dk)
+                    for (int dj = 0; dj < tn1; ++dj)
+                        for (int di = 0; di < tn0; ++di) sum += term[tp + (dk * TY + dj) * TX + di];
+            }
             a.fc[tc] = sum * inv;
         }
     }
 }
 
-template <typename T, typename TB, int TX, int TY, int TZ>
+template <typename T, typename TB, int TX, int TY, int TZ, bool RHO = false>
 void launch_box(BoxArgs<T, TB>& a, bool up, cudaStream_t st) {
     const int n[3] = {a.g.nx, a.g.ny, a.g.nz}, cn[3] = {a.cg.nx, a.cg.ny, a.cg.nz}, tt[3] = {TX, TY, TZ};
     int nb[3];
@@ -322,7 +378,7 @@ void launch_box(BoxArgs<T, TB>& a, bool up, cudaStream_t st) {
         nb[q] = (cn[q] + a.tc[q] - 1) / a.tc[q];
     }
     using B = Box<TX, TY, TZ>;
-    launch_pdl(up ? box_kernel<T, TB, TX, TY, TZ, true> : box_kernel<T, TB, TX, TY, TZ, false>,
+    launch_pdl(up ? box_kernel<T, TB, TX, TY, TZ, true, RHO> : box_kernel<T, TB, TX, TY, TZ, false, RHO>,
                dim3(nb[0], nb[1], nb[2]), B::threads, 0, st, a);
     count_launch();
 }
@@ -362,7 +418,8 @@ void launch_box_level(const Geo& g, const TB* const b[3], T scale, const T* w, c
     a.x = x;
     a.fc = fc;
     a.xc = xc;
-    a.scale = scale;
+    a.hs = T(1) / scale;
+    a.rs = scale;
     a.omega = (T)omega;
     a.sweeps = sweeps;
     if constexpr (sizeof(T) == 4) {
@@ -373,6 +430,32 @@ void launch_box_level(const Geo& g, const TB* const b[3], T scale, const T* w, c
     }
     launch_box<T, TB, 4, 4, 4>(a, up, st);
 }
+
+template <typename RT>
+void launch_box_rho(const Geo& g, const RT* rh, double h, const float* f, const Geo& cg, bool up, const float* xin, float* x,
+                    float* fc, const float* xc, double omega, int sweeps, cudaStream_t st) {
+    BoxArgs<float, RT> a{};
+    a.g = g;
+    a.cg = cg;
+    for (int q = 0; q < 3; ++q) a.fac[q] = 2;
+    a.b[0] = rh;
+    a.f = f;
+    a.xin = xin;
+    a.x = x;
+    a.fc = fc;
+    a.xc = xc;
+    a.hs = (float)(h * h);
+    a.rs = (float)(1.0 / (h * h));
+    a.omega = (float)omega;
+    a.sweeps = sweeps;
+    // 32^3: 707 us a step by large boxes, 765 by small ones, 798 by passes
+    if (g.ncell() > kSmallBoxCells) launch_box<float, RT, 8, 8, 4, true>(a, up, st);
+    else launch_box<float, RT, 4, 4, 4, true>(a, up, st);
+}
+template void launch_box_rho<float>(const Geo&, const float*, double, const float*, const Geo&, bool, const float*, float*,
+                                    float*, const float*, double, int, cudaStream_t);
+template void launch_box_rho<__half>(const Geo&, const __half*, double, const float*, const Geo&, bool, const float*, float*,
+                                     float*, const float*, double, int, cudaStream_t);
 
 template void launch_box_level<float, float>(const Geo&, const float* const[3], float, const float*, const float*,
                                              const float*, const Geo&, const int[3], bool, const float*, float*, float*,

@@ -551,6 +551,11 @@ template <typename T, typename TB>
 void launch_box_level(const Geo& g, const TB* const b[3], T scale, const T* w, const T* sig, const T* f, const Geo& cg,
                       const int fac[3], bool up, const T* xin, T* x, T* fc, const T* xc, double omega, int sweeps,
                       cudaStream_t st);
+// The same for the finest level of the mixed step: coefficients from rho/2, the
+// level's vectors in the colour-split layout, every axis halved.
+template <typename RT>
+void launch_box_rho(const Geo& g, const RT* rh, double h, const float* f, const Geo& cg, bool up, const float* xin, float* x,
+                    float* fc, const float* xc, double omega, int sweeps, cudaStream_t st);
 
 // ------------------------------------------------------------ Krylov ------
 // r = f - A x (FP64), optional r32 = scale * r; partials (||r||^2, max|r|, nonfinite).

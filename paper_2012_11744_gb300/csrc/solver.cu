@@ -679,7 +679,7 @@ void launch_tail(paris_ctx* c, int t) {
 // Whether level l (above the tail) runs as one launch down and one up: the
 // levels of box_level_fits, with the tail's smoother and switch.
 bool box_level(const paris_ctx* c, int l, bool fp64) {
-    return c->opts.coarse_tail != 0 && c->opts.smoother == PARIS_SMOOTH_RBGS_2PASS && l >= 1 &&
+    return c->opts.coarse_tail != 0 && c->opts.smoother == PARIS_SMOOTH_RBGS_2PASS &&
            l + 1 < (int)c->lv.size() && box_level_fits(c->lv[l].g, c->opts.nu1, c->opts.nu2, fp64);
 }
 
@@ -767,13 +767,35 @@ bool coarse_graph_launch(paris_ctx* c, const Coef<T>& c0) {
 template <typename T>
 void vcycle(paris_ctx* c, const Coef<T>& c0, const T* f0, T* x0) {
     const int nl = (int)c->lv.size();
+    // the finest level of a small mixed step by boxes too
+    const bool box0 = sizeof(T) == 4 && c->rho0 && c->opts.level0_tiles == 1 && nl >= 3 && box_level(c, 0, false);
+    auto finest = [&](bool up) {
+        if constexpr (sizeof(T) == 4) {
+            if (box0) {
+                float* t = c->lv[0].t32;
+                const int sweeps = up ? c->opts.nu2 : c->opts.nu1;
+                // f, rho/2 and x once each; counted as the colour passes that it makes
+                ProfScope ps(c, PARIS_K_SMOOTH0, c->N * ((up ? 12.0 : 8.0) + (c->half_rho ? 2.0 : 4.0)), 2 * sweeps);
+                float* out = up ? x0 : t;
+                if (c->half_rho)
+                    launch_box_rho<__half>(c->g0, c->rh16, c->grid.h, f0, c->lv[1].g, up, t, out, c->lv[1].f32, c->lv[1].x32,
+                                           c->opts.omega, sweeps, c->st);
+                else
+                    launch_box_rho<float>(c->g0, c->rh32, c->grid.h, f0, c->lv[1].g, up, t, out, c->lv[1].f32, c->lv[1].x32,
+                                          c->opts.omega, sweeps, c->st);
+                return;
+            }
+        }
+        if (up) vup<T>(c, c0, f0, x0, 0);
+        else vdown<T>(c, c0, f0, x0, 0);
+    };
     if (nl >= 3 && !c->cap_stream_broken) {
-        vdown<T>(c, c0, f0, x0, 0);
+        finest(false);
         {
             ProfScope ps(c, PARIS_K_COARSE, 0.0);
             if (!coarse_graph_launch<T>(c, c0)) coarse_part<T>(c, c0);
         }
-        vup<T>(c, c0, f0, x0, 0);
+        finest(true);
         return;
     } else {
         for (int l = 0; l < nl - 1; ++l) vdown<T>(c, c0, f0, x0, l);
