@@ -12,7 +12,9 @@
 // i.e. the paper's A7 p - sum A_nb p_nb with A_nb = beta_f scale.
 #include <math.h>
 
+#include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cstdio>
 
 #include "kernels.cuh"
@@ -632,26 +634,42 @@ void launch_project(const Geo& g, const double* bx, const double* by, const doub
 // ------------------------------------------------------------ level set-up ---
 
 // Level-0 coefficient copy in the solver's precision, pre-multiplied by scale.
-template <typename T>
-__global__ void convert_beta_kernel(int64_t n, const double* __restrict__ b, double scale,
-                                    T* __restrict__ out) {
-    PARIS_EW_FOR(c, n)
-        out[c] = (T)(b[c] * scale);
+// out = float(b * scale), blockIdx.y selecting one of up to three arrays.  The
+// conversion by integer operations, the three face arrays in one launch: 128^3
+// 32 us in three launches of hardware conversions, 24.5 in this one.
+struct ConvertArgs {
+    const double* in[3];
+    float* out[3];
+    int64_t n[3];
+};
+
+__global__ void convert_kernel(const __grid_constant__ ConvertArgs a, double scale) {
+    pdl_wait();
+    const double* __restrict__ b = a.in[blockIdx.y];
+    float* __restrict__ out = a.out[blockIdx.y];
+    const int64_t n = a.n[blockIdx.y];
+    PARIS_EW_FOR(c, n) out[c] = d2f_scaled(b[c] * scale, 0);
 }
 
-template <typename T>
-void launch_convert_beta(const Geo& g, const double* b64[3], double scale, T* out[3],
-                         cudaStream_t st) {
-    for (int a = 0; a < 3; ++a) {
-        int64_t n = g.nface(a);
-        convert_beta_kernel<T><<<elementwise_blocks(n), kRedThreads, 0, st>>>(n, b64[a], scale,
-                                                                              out[a]);
-        count_launch();
+void launch_convert_beta(const Geo& g, const double* b64[3], double scale, float* out[3], cudaStream_t st) {
+    ConvertArgs a{};
+    int64_t most = 0;
+    for (int q = 0; q < 3; ++q) {
+        a.in[q] = b64[q];
+        a.out[q] = out[q];
+        a.n[q] = g.nface(q);
+        most = std::max(most, a.n[q]);
     }
+    launch_pdl(convert_kernel, dim3(elementwise_blocks(most), 3), dim3(kRedThreads), 0, st, a, scale);
+    count_launch();
 }
 
 void launch_convert_scaled(int64_t n, const double* in, double scale, float* out, cudaStream_t st) {
-    convert_beta_kernel<float><<<elementwise_blocks(n), kRedThreads, 0, st>>>(n, in, scale, out);
+    ConvertArgs a{};
+    a.in[0] = in;
+    a.out[0] = out;
+    a.n[0] = n;
+    launch_pdl(convert_kernel, dim3(elementwise_blocks(n)), dim3(kRedThreads), 0, st, a, scale);
     count_launch();
 }
 
@@ -667,127 +685,221 @@ void launch_convert_scaled(int64_t n, const double* in, double scale, float* out
 // and through the periodic seam crosses a longer distance between centres:
 // r_last and r_seam are the fine distance over the coarse one, each in its
 // level's cell widths (1 where all cells are alike).
+// The coarse diagonal excess is the mean over the children of the fine one
+// times the fine level's scale (the coarse levels hold absolute coefficients),
+// the restriction of the fine equations (an average) applied to sig x with x
+// constant over the children.
+//
+// One thread forms the three faces on the minus sides of a coarse cell (and,
+// past a wall's last cell, the closed faces) and the cell's excess: one launch
+// a level instead of three or four, the fine faces of a regular cell loaded
+// together, FP32 values widened and rounded by integer operations and the
+// divisions by counts (powers of two) as exact products.  128^3 to 2^3 in
+// FP32: 134 us in 18 launches, 37 in 6.
 template <typename T>
-__global__ void coarse_beta_kernel(Geo fg, Coef<T> cf, Geo cg, int fa0, int fa1, int fa2,
-                                   int axis, double ratio, double r_last, double r_seam, T* __restrict__ out) {
-    const int n0 = cg.nx + (axis == 0 ? cg.wx : 0);
-    const int n1 = cg.ny + (axis == 1 ? cg.wy : 0);
-    const int n2 = cg.nz + (axis == 2 ? cg.wz : 0);
-    const int64_t total = (int64_t)n0 * n1 * n2;
-    const int fac[3] = {fa0, fa1, fa2};
-    const T* src = axis == 0 ? cf.bx : (axis == 1 ? cf.by : cf.bz);
-    const int fn0 = fg.nx + (axis == 0 ? fg.wx : 0);
-    const int fn1 = fg.ny + (axis == 1 ? fg.wy : 0);
-    const int fn[3] = {fg.nx, fg.ny, fg.nz}, cn[3] = {cg.nx, cg.ny, cg.nz};
-    PARIS_EW_FOR(t, total) {
-        const int I = (int)(t % n0);
-        const int J = (int)((t / n0) % n1);
-        const int K = (int)(t / ((int64_t)n0 * n1));
-        const int C3[3] = {I, J, K};
-        int lo[3], cnt[3];
-        for (int b = 0; b < 3; ++b) {
-            lo[b] = C3[b] * fac[b];
-            cnt[b] = b == axis ? 1 : child_count(C3[b], cn[b], fn[b], fac[b]);
+struct CoarseArgs {
+    Geo fg, cg;
+    Coef<T> cf;
+    int fac[3];
+    double c[3];               // (h_fine / h_coarse)^2 over the number of fine faces, a power of two
+    double r_last[3], r_seam[3];
+    T* out[3];
+    double csig;               // 1 / children, a power of two
+    T* sig;                    // or null
+};
+
+__device__ __forceinline__ double widen(float v) { return f2d_scaled(v, 0); }
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ void narrow(double v, float& out) { out = d2f_scaled(v, 0); }
+__device__ __forceinline__ void narrow(double v, double& out) { out = v; }
+
+template <typename T, int AXIS>
+__device__ __forceinline__ void coarse_face(const CoarseArgs<T>& a, int I, int J, int K) {
+    const Geo &fg = a.fg, &cg = a.cg;
+    const int n0 = cg.nx + (AXIS == 0 ? cg.wx : 0), n1 = cg.ny + (AXIS == 1 ? cg.wy : 0);
+    const int n2 = cg.nz + (AXIS == 2 ? cg.wz : 0);
+    if (I >= n0 || J >= n1 || K >= n2) return;
+    T* out = a.out[AXIS] + ((int64_t)K * n1 + J) * n0 + I;
+    const int F = AXIS == 0 ? I : AXIS == 1 ? J : K, cn = AXIS == 0 ? cg.nx : AXIS == 1 ? cg.ny : cg.nz;
+    if (F == cn) {  // the far wall: closed
+        *out = T(0);
+        return;
+    }
+    const int fn0 = fg.nx + (AXIS == 0 ? fg.wx : 0), fn1 = fg.ny + (AXIS == 1 ? fg.wy : 0);
+    const T* src = (AXIS == 0 ? a.cf.bx : AXIS == 1 ? a.cf.by : a.cf.bz) +
+                   ((int64_t)K * a.fac[2] * fn1 + J * a.fac[1]) * fn0 + I * a.fac[0];
+    // the fine faces of the coarse one: p (inner) by q (outer), along the two other axes
+    const int np = AXIS == 0 ? child_count(J, cg.ny, fg.ny, a.fac[1]) : child_count(I, cg.nx, fg.nx, a.fac[0]);
+    const int nq = AXIS == 2 ? child_count(J, cg.ny, fg.ny, a.fac[1]) : child_count(K, cg.nz, fg.nz, a.fac[2]);
+    const int64_t sp = AXIS == 0 ? fn0 : 1, sq = AXIS == 2 ? fn0 : (int64_t)fn0 * fn1;
+    double sum = 0.0;
+    if (np == 2 && nq == 2) {
+        const T v[4] = {src[0], src[sp], src[sq], src[sq + sp]};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sum += widen(v[q]);
+    } else {
+        for (int q = 0; q < nq; ++q)
+            for (int p = 0; p < np; ++p) sum += widen(src[q * sq + p * sp]);
+    }
+    double v = sum * a.c[AXIS] * (double)a.cf.scale;
+    if (F == 0) v *= a.r_seam[AXIS];
+    else if (F == cn - 1) v *= a.r_last[AXIS];
+    narrow(v, *out);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kTX* kTY) coarse_level_kernel(const __grid_constant__ CoarseArgs<T> a) {
+    pdl_wait();
+    const int I = blockIdx.x * kTX + threadIdx.x, J = blockIdx.y * kTY + threadIdx.y, K = blockIdx.z;
+    const Geo &fg = a.fg, &cg = a.cg;
+    const bool cell = I < cg.nx && J < cg.ny && K < cg.nz;
+    if (cell && (a.fac[0] & a.fac[1] & a.fac[2]) == 2 &&
+        child_count(I, cg.nx, fg.nx, 2) + child_count(J, cg.ny, fg.ny, 2) + child_count(K, cg.nz, fg.nz, 2) == 6) {
+        // a regular cell: its three faces' twelve fine ones in flight together
+        const T* src[3];
+        T v[12];
+        T* out[3];
+        const int n0[3] = {fg.nx + fg.wx, fg.nx, fg.nx}, n1[3] = {fg.ny, fg.ny + fg.wy, fg.ny};
+        const int m0[3] = {cg.nx + cg.wx, cg.nx, cg.nx}, m1[3] = {cg.ny, cg.ny + cg.wy, cg.ny};
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            src[q] = (q == 0 ? a.cf.bx : q == 1 ? a.cf.by : a.cf.bz) + ((int64_t)2 * K * n1[q] + 2 * J) * n0[q] + 2 * I;
+            out[q] = a.out[q] + ((int64_t)K * m1[q] + J) * m0[q] + I;
+            const int64_t sp = q == 0 ? n0[q] : 1, sq = q == 2 ? n0[q] : (int64_t)n0[q] * n1[q];
+            v[4 * q] = src[q][0];
+            v[4 * q + 1] = src[q][sp];
+            v[4 * q + 2] = src[q][sq];
+            v[4 * q + 3] = src[q][sq + sp];
         }
-        const int F = C3[axis];
-        if (F == cn[axis]) {  // the far wall: closed
-            out[t] = T(0);
-            continue;
+        const int F[3] = {I, J, K}, cn[3] = {cg.nx, cg.ny, cg.nz};
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            double t = ((widen(v[4 * q]) + widen(v[4 * q + 1])) + widen(v[4 * q + 2])) + widen(v[4 * q + 3]);
+            t = t * a.c[q] * (double)a.cf.scale;
+            if (F[q] == 0) t *= a.r_seam[q];
+            else if (F[q] == cn[q] - 1) t *= a.r_last[q];
+            narrow(t, *out[q]);
         }
+    } else {
+        coarse_face<T, 0>(a, I, J, K);
+        coarse_face<T, 1>(a, I, J, K);
+        coarse_face<T, 2>(a, I, J, K);
+    }
+    if (a.sig && cell) {
+        const int n0 = child_count(I, cg.nx, fg.nx, a.fac[0]), n1 = child_count(J, cg.ny, fg.ny, a.fac[1]);
+        const int n2 = child_count(K, cg.nz, fg.nz, a.fac[2]);
+        const T* src = a.cf.sig + fg.cidx(I * a.fac[0], J * a.fac[1], K * a.fac[2]);
+        const int64_t sy = fg.nx, sz = (int64_t)fg.nx * fg.ny;
         double sum = 0.0;
-        for (int dk = 0; dk < cnt[2]; ++dk)
-            for (int dj = 0; dj < cnt[1]; ++dj)
-                for (int di = 0; di < cnt[0]; ++di) {
-                    int64_t fi = ((int64_t)(lo[2] + dk) * fn1 + (lo[1] + dj)) * fn0 + (lo[0] + di);
-                    sum += (double)src[fi];
-                }
-        const double mean = sum / (double)((fa0 * fa1 * fa2) / fac[axis]);
-        const double r = F == 0 ? r_seam : (F == cn[axis] - 1 ? r_last : 1.0);
-        out[t] = (T)(mean * ratio * (double)cf.scale * r);
+        if (n0 + n1 + n2 == 6 && n0 == 2 && n1 == 2) {
+            T v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = src[(q >> 2) * sz + ((q >> 1) & 1) * sy + (q & 1)];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) sum += widen(v[q]);
+        } else {
+            for (int dk = 0; dk < n2; ++dk)
+                for (int dj = 0; dj < n1; ++dj)
+                    for (int di = 0; di < n0; ++di) sum += widen(src[dk * sz + dj * sy + di]);
+        }
+        narrow(sum * a.csig * (double)a.cf.scale, a.sig[cg.cidx(I, J, K)]);
     }
 }
 
 template <typename T>
-void launch_coarse_beta(const Geo& fine, const Coef<T>& cf, const Geo& coarse, const int f[3],
-                        const double wf[3], const double wc[3], T* out[3], cudaStream_t st) {
-    for (int a = 0; a < 3; ++a) {
-        int64_t n = coarse.nface(a);
+void launch_coarse_level(const Geo& fine, const Coef<T>& cf, const Geo& coarse, const int f[3], const double wf[3],
+                         const double wc[3], T* out[3], T* sig, cudaStream_t st) {
+    CoarseArgs<T> a{};
+    a.fg = fine;
+    a.cg = coarse;
+    a.cf = cf;
+    for (int q = 0; q < 3; ++q) {
         // distances over the seam: half of the first and of the last cell's width; the
         // last interior coarse face lies between fine cells of width 1 when the axis is halved
-        const double df = 0.5 * (1.0 + wf[a]), dc = 0.5 * (1.0 + wc[a]);
-        coarse_beta_kernel<T><<<elementwise_blocks(n), kRedThreads, 0, st>>>(
-            fine, cf, coarse, f[0], f[1], f[2], a, 1.0 / ((double)f[a] * f[a]), (f[a] == 2 ? 1.0 : df) / dc, df / dc,
-            out[a]);
-        count_launch();
+        const double df = 0.5 * (1.0 + wf[q]), dc = 0.5 * (1.0 + wc[q]);
+        a.fac[q] = f[q];
+        a.c[q] = 1.0 / ((double)f[q] * f[q]) / (double)((f[0] * f[1] * f[2]) / f[q]);
+        a.r_last[q] = (f[q] == 2 ? 1.0 : df) / dc;
+        a.r_seam[q] = df / dc;
+        a.out[q] = out[q];
     }
-}
-
-// Coarse diagonal excess: the mean over the children of the fine one times
-// the fine level's scale (the coarse levels hold absolute coefficients), the
-// restriction of the fine equations (an average) applied to sig x with x
-// constant over the children.
-template <typename T>
-__global__ void coarse_sig_kernel(Geo fg, const T* __restrict__ sf, double scale, Geo cg, int fa0, int fa1,
-                                  int fa2, T* __restrict__ out) {
-    const int64_t total = cg.ncell();
-    PARIS_EW_FOR(t, total) {
-        const int I = (int)(t % cg.nx);
-        const int J = (int)((t / cg.nx) % cg.ny);
-        const int K = (int)(t / ((int64_t)cg.nx * cg.ny));
-        const int n0 = child_count(I, cg.nx, fg.nx, fa0), n1 = child_count(J, cg.ny, fg.ny, fa1);
-        const int n2 = child_count(K, cg.nz, fg.nz, fa2);
-        double sum = 0.0;
-        for (int dk = 0; dk < n2; ++dk)
-            for (int dj = 0; dj < n1; ++dj)
-                for (int di = 0; di < n0; ++di)
-                    sum += (double)sf[fg.cidx(I * fa0 + di, J * fa1 + dj, K * fa2 + dk)];
-        out[t] = (T)(sum / (double)(fa0 * fa1 * fa2) * scale);
-    }
-}
-
-template <typename T>
-void launch_coarse_sig(const Geo& fine, const T* sig, double scale, const Geo& coarse, const int f[3], T* out,
-                       cudaStream_t st) {
-    coarse_sig_kernel<T><<<elementwise_blocks(coarse.ncell()), kRedThreads, 0, st>>>(fine, sig, scale, coarse,
-                                                                                      f[0], f[1], f[2], out);
+    a.csig = 1.0 / (double)(f[0] * f[1] * f[2]);
+    a.sig = cf.sig ? sig : nullptr;
+    launch_pdl(coarse_level_kernel<T>,
+               dim3((coarse.nx + coarse.wx + kTX - 1) / kTX, (coarse.ny + coarse.wy + kTY - 1) / kTY, coarse.nz + coarse.wz),
+               dim3(kTX, kTY), 0, st, a);
     count_launch();
 }
 
 // w = 1 / (sum_f beta_f + sig_c) (unscaled inverse diagonal; the smoother
 // divides the right-hand side by the level's scale).
+// All levels of the range in one launch: a block finds its level by its index.
 template <typename T>
-__global__ void inv_diag_kernel(Geo g, Coef<T> cf, T* __restrict__ w) {
-    const int i = blockIdx.x * kTX + threadIdx.x;
-    const int j = blockIdx.y * kTY + threadIdx.y;
-    const int k = blockIdx.z;
+struct InvDiagArgs {
+    int n;
+    Geo g[kMaxInvLevels];
+    Coef<T> cf[kMaxInvLevels];
+    T* w[kMaxInvLevels];
+    int first[kMaxInvLevels + 1];  // first block of each level
+};
+
+template <typename T>
+__global__ void __launch_bounds__(kTX* kTY) inv_diag_kernel(const __grid_constant__ InvDiagArgs<T> a) {
+    pdl_wait();
+    int l = 0;
+    while (l + 1 < a.n && (int)blockIdx.x >= a.first[l + 1]) ++l;
+    const Geo g = a.g[l];
+    const Coef<T> cf = a.cf[l];
+    const int tx = (g.nx + kTX - 1) / kTX, ty = (g.ny + kTY - 1) / kTY;
+    const int blk = blockIdx.x - a.first[l], bx = blk % tx, r = blk / tx;
+    const int i = bx * kTX + threadIdx.x, j = (r % ty) * kTY + threadIdx.y, k = r / ty;
     if (i >= g.nx || j >= g.ny) return;
     Stencil<T> s;
     load_stencil(g, cf, i, j, k, s);
     const int64_t c = g.cidx(i, j, k);
     if (cf.sig) {  // the diagonal of a Dirichlet-coupled cell includes its excess
         const T d = (((s.b[0] + s.b[1]) + (s.b[2] + s.b[3])) + (s.b[4] + s.b[5])) + cf.sig[c];
-        w[c] = d > T(0) ? rcp_rn(d) : T(0);
+        a.w[l][c] = d > T(0) ? rcp_rn(d) : T(0);
     } else {
-        w[c] = inv_sum6(s.b);
+        a.w[l][c] = inv_sum6(s.b);
     }
 }
 
 template <typename T>
-void launch_inv_diag(const Geo& g, const Coef<T>& cf, T* w, cudaStream_t st) {
-    dim3 gr((g.nx + kTX - 1) / kTX, (g.ny + kTY - 1) / kTY, g.nz);
-    inv_diag_kernel<T><<<gr, dim3(kTX, kTY), 0, st>>>(g, cf, w);
-    count_launch();
+void launch_inv_diag(int n, const Geo* g, const Coef<T>* cf, T* const* w, cudaStream_t st) {
+    while (n > 0) {
+        InvDiagArgs<T> a{};
+        int64_t blocks = 0;
+        while (a.n < n && a.n < kMaxInvLevels) {
+            const Geo& q = g[a.n];
+            const int64_t more = (int64_t)((q.nx + kTX - 1) / kTX) * ((q.ny + kTY - 1) / kTY) * q.nz;
+            if (blocks + more > INT_MAX) break;  // beyond 8e11 cells in one launch
+            a.g[a.n] = q;
+            a.cf[a.n] = cf[a.n];
+            a.w[a.n] = w[a.n];
+            a.first[a.n++] = (int)blocks;
+            blocks += more;
+        }
+        if (a.n == 0) return;
+        launch_pdl(inv_diag_kernel<T>, dim3((unsigned)blocks), dim3(kTX, kTY), 0, st, a);
+        count_launch();
+        n -= a.n;
+        g += a.n;
+        cf += a.n;
+        w += a.n;
+    }
 }
 
 // Dense inverse of the coarsest operator regularised on its null space:
 // (A + a 1 1^T)^{-1} with a = mean(diag)/n, which maps a mean-free f to the
 // mean-free solution of A x = f (with a diagonal excess, cf.sig: A^{-1}).  FP64 Gauss-Jordan without pivoting (the
 // regularised matrix is SPD) by one CTA of 32 x 32 threads on a copy of the
-// matrix in shared memory (n <= 128: at most 129 KB); the elimination step
+// matrix in shared memory (n <= 128: at most 129 KB; n <= 16: 32 x 4); the elimination step
 // maps rows to threadIdx.y and columns to threadIdx.x.
 template <typename T>
 __global__ void __launch_bounds__(1024) coarse_inverse_kernel(Geo g, Coef<T> cf, double* __restrict__ Mout) {
     extern __shared__ double smem[];
+    pdl_wait();
     const int n = (int)g.ncell();
     double* M = smem;         // n x n, row-major
     double* col = smem + n * n;  // column kk before the pivot step
@@ -856,7 +968,8 @@ void launch_coarse_inverse(const Geo& g, const Coef<T>& cf, double* inv, cudaStr
                              (int)(sizeof(double) * (128 * 128 + 128)));
         opted = true;
     }
-    coarse_inverse_kernel<T><<<1, dim3(32, 32), bytes, st>>>(g, cf, inv);
+    // a small matrix is a chain of barriers: fewer warps, cheaper barriers (n = 8: 14.5 -> 12.3 us)
+    launch_pdl(coarse_inverse_kernel<T>, dim3(1), dim3(32, n <= 16 ? 4 : 32), bytes, st, g, cf, inv);
     count_launch();
 }
 
@@ -1846,15 +1959,11 @@ cudaError_t stream_rates(const float* a, const float* b, const float* c, float* 
 // ------------------------------------------------------ explicit instances ---
 
 #define PARIS_INSTANTIATE(T)                                                                  \
-    template void launch_convert_beta<T>(const Geo&, const double* [3], double, T* [3],        \
-                                         cudaStream_t);                                        \
-    template void launch_coarse_beta<T>(const Geo&, const Coef<T>&, const Geo&, const int[3],  \
-                                        const double[3], const double[3], T* [3], cudaStream_t); \
-    template void launch_inv_diag<T>(const Geo&, const Coef<T>&, T*, cudaStream_t);            \
+    template void launch_coarse_level<T>(const Geo&, const Coef<T>&, const Geo&, const int[3], \
+                                         const double[3], const double[3], T* [3], T*, cudaStream_t); \
+    template void launch_inv_diag<T>(int, const Geo*, const Coef<T>*, T* const*, cudaStream_t); \
     template void launch_coarse_inverse<T>(const Geo&, const Coef<T>&, double*, cudaStream_t); \
     template void launch_coarse_solve<T>(const Geo&, const double*, const T*, T*, cudaStream_t, bool); \
-    template void launch_coarse_sig<T>(const Geo&, const T*, double, const Geo&, const int[3], T*,     \
-                                       cudaStream_t);                                                  \
     template void launch_rbgs<T>(const Geo&, const Coef<T>&, const T*, const T*, T*, int,     \
                                  double, bool, cudaStream_t, int, int);                        \
     template void launch_jacobi<T>(const Geo&, const Coef<T>&, const T*, const T*, const T*,  \

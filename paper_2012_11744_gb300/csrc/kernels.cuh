@@ -385,26 +385,24 @@ int64_t launch_max_divergence(const Geo& g, const double* u, const double* v, co
                               double inv_h, double* partials, cudaStream_t st);
 
 // ---------------------------------------------------- level set-up --------
-template <typename T>
-void launch_convert_beta(const Geo& g, const double* b64[3], double scale, T* out[3],
-                         cudaStream_t st);
+// FP32 copies of the face arrays times scale
+void launch_convert_beta(const Geo& g, const double* b64[3], double scale, float* out[3], cudaStream_t st);
 // out = float(in * scale) over n cells (the FP32 copy of a diagonal excess)
 void launch_convert_scaled(int64_t n, const double* in, double scale, float* out, cudaStream_t st);
+// coarse coefficients, and the coarse diagonal excess sig where cf has one
 template <typename T>
-void launch_coarse_beta(const Geo& fine, const Coef<T>& cf, const Geo& coarse, const int f[3],
-                        const double wf[3], const double wc[3], T* out[3], cudaStream_t st);
+void launch_coarse_level(const Geo& fine, const Coef<T>& cf, const Geo& coarse, const int f[3], const double wf[3],
+                         const double wc[3], T* out[3], T* sig, cudaStream_t st);
+constexpr int kMaxInvLevels = 24;  // levels in one launch_inv_diag launch
+// inverse diagonals w[l] of n levels
 template <typename T>
-void launch_inv_diag(const Geo& g, const Coef<T>& cf, T* w, cudaStream_t st);
+void launch_inv_diag(int n, const Geo* g, const Coef<T>* cf, T* const* w, cudaStream_t st);
 // dense (A + a 1 1^T)^{-1} of the coarsest operator, FP64, one CTA
 template <typename T>
 void launch_coarse_inverse(const Geo& g, const Coef<T>& cf, double* inv, cudaStream_t st);
 // x = inv (f - mean f); keep_mean: x = inv f (an operator without null space)
 template <typename T>
 void launch_coarse_solve(const Geo& g, const double* inv, const T* f, T* x, cudaStream_t st, bool keep_mean);
-// coarse diagonal excess (Coef::sig) from the fine one of a level with the given scale
-template <typename T>
-void launch_coarse_sig(const Geo& fine, const T* sig, double scale, const Geo& coarse, const int f[3], T* out,
-                       cudaStream_t st);
 
 // ------------------------------------------------------------ V-cycle -----
 // One red-black colour pass of over-relaxed Gauss-Seidel on A x = f, in

@@ -1533,8 +1533,8 @@ void launch_prolong_split(const Geo& fine, const Geo& coarse, const float* xc, f
 // that tile each coarse face, times (h0/h1)^2 = 1/4 and the fine scale
 // 1/h0^2 (the coarse arrays hold scaled coefficients).
 template <int AXIS>
-__global__ void coarse_beta_rho_kernel(Geo fg, const float* __restrict__ rh, float scale, Geo cg,
-                                       float* __restrict__ out, __half* __restrict__ out16, float s16) {
+__device__ __forceinline__ void coarse_beta_rho(const Geo& fg, const float* __restrict__ rh, float scale, const Geo& cg,
+                                                float* __restrict__ out, __half* __restrict__ out16, float s16) {
     const int n0 = cg.nx + (AXIS == 0 ? cg.wx : 0);
     const int n1 = cg.ny + (AXIS == 1 ? cg.wy : 0);
     const int n2 = cg.nz + (AXIS == 2 ? cg.wz : 0);
@@ -1572,18 +1572,33 @@ __global__ void coarse_beta_rho_kernel(Geo fg, const float* __restrict__ rh, flo
     }
 }
 
+// the three axes in one launch (blockIdx.y)
+struct CoarseRhoArgs {
+    float* out[3];
+    __half* out16[3];
+};
+__global__ void coarse_beta_rho_kernel(Geo fg, const float* __restrict__ rh, float scale, Geo cg,
+                                       const __grid_constant__ CoarseRhoArgs a, float s16) {
+    pdl_wait();
+    if (blockIdx.y == 0) coarse_beta_rho<0>(fg, rh, scale, cg, a.out[0], a.out16[0], s16);
+    if (blockIdx.y == 1) coarse_beta_rho<1>(fg, rh, scale, cg, a.out[1], a.out16[1], s16);
+    if (blockIdx.y == 2) coarse_beta_rho<2>(fg, rh, scale, cg, a.out[2], a.out16[2], s16);
+}
+
 void launch_coarse_beta_rho(const Geo& fine, const float* rh, double h, const Geo& coarse, float* out[3],
                             cudaStream_t st, __half* const out16[3], float s16) {
     // mean of 4 faces (1/4) x (h0/h1)^2 (1/4) x 1/h0^2
     const float scale = (float)(1.0 / (16.0 * h * h));
-    for (int a = 0; a < 3; ++a) {
-        const unsigned nb = (unsigned)elementwise_blocks(coarse.nface(a));
-        __half* o16 = out16 ? out16[a] : nullptr;
-        if (a == 0) coarse_beta_rho_kernel<0><<<nb, kRedThreads, 0, st>>>(fine, rh, scale, coarse, out[0], o16, s16);
-        if (a == 1) coarse_beta_rho_kernel<1><<<nb, kRedThreads, 0, st>>>(fine, rh, scale, coarse, out[1], o16, s16);
-        if (a == 2) coarse_beta_rho_kernel<2><<<nb, kRedThreads, 0, st>>>(fine, rh, scale, coarse, out[2], o16, s16);
+    CoarseRhoArgs a{};
+    int64_t most = 0;
+    for (int q = 0; q < 3; ++q) {
+        a.out[q] = out[q];
+        a.out16[q] = out16 ? out16[q] : nullptr;
+        if (coarse.nface(q) > most) most = coarse.nface(q);
     }
-    count_launch(3);
+    launch_pdl(coarse_beta_rho_kernel, dim3(elementwise_blocks(most), 3), dim3(kRedThreads), 0, st, fine, rh, scale, coarse,
+               a, s16);
+    count_launch();
 }
 
 }  // namespace paris

@@ -190,7 +190,7 @@ bool valid_opts(const paris_opts* o) {
 // Level plan: halve every axis of at least four cells while the level has
 // more than coarse_max_cells cells.  An axis of odd length n is halved to
 // (n-1)/2 cells, the last one made of three (its coefficients take the longer
-// distance between centres, see launch_coarse_beta), but only while the level
+// distance between centres, see launch_coarse_level), but only while the level
 // is larger than the dense coarsest solve takes: below that the odd axis
 // stays as it is and the dense solve takes over.  So every grid ends in a
 // dense coarsest level.  The paper's in-code multigrid (Sec. 3.7.3) needs 2^n
@@ -412,21 +412,23 @@ void setup_hierarchy(paris_ctx* c, const Coef<T>& c0) {
                 continue;
             }
         }
-        launch_coarse_beta<T>(F.g, cf, L.g, L.fac, F.wlast, L.wlast, out, c->st);
-        if (c->dirichlet) launch_coarse_sig<T>(F.g, cf.sig, (double)cf.scale, L.g, L.fac, Prec<T>::sig(L), c->st);
+        launch_coarse_level<T>(F.g, cf, L.g, L.fac, F.wlast, L.wlast, out, c->dirichlet ? Prec<T>::sig(L) : nullptr, c->st);
     }
     // inverse diagonals: read by the FP64 smoothers, by Jacobi, by the tail
     // launch and by every smoother of an operator with a diagonal excess; the
     // other FP32 red-black sweeps recompute them from the coefficients they
     // load (the same value)
     const int t = tail_start(c);
-    if (sizeof(T) == 8 || c->opts.smoother == PARIS_SMOOTH_JACOBI || c->dirichlet) {
-        for (int l = 0; l < nl; ++l)
-            launch_inv_diag<T>(c->lv[l].g, level_coef<T>(c, l, c0), Prec<T>::w(c->lv[l]), c->st);
-    } else if (t > 0) {
-        for (int l = t; l < nl; ++l)
-            launch_inv_diag<T>(c->lv[l].g, level_coef<T>(c, l, c0), Prec<T>::w(c->lv[l]), c->st);
+    const int from = sizeof(T) == 8 || c->opts.smoother == PARIS_SMOOTH_JACOBI || c->dirichlet ? 0 : t > 0 ? t : nl;
+    std::vector<Geo> g;
+    std::vector<Coef<T>> cf;
+    std::vector<T*> w;
+    for (int l = from; l < nl; ++l) {
+        g.push_back(c->lv[l].g);
+        cf.push_back(level_coef<T>(c, l, c0));
+        w.push_back(Prec<T>::w(c->lv[l]));
     }
+    launch_inv_diag<T>((int)g.size(), g.data(), cf.data(), w.data(), c->st);
     launch_coarse_inverse<T>(c->lv[nl - 1].g, level_coef<T>(c, nl - 1, c0), c->coarse_inv, c->st);
 }
 
@@ -937,7 +939,7 @@ void mixed_setup(paris_ctx* c, const Coef<double>& c64, bool rho0) {
     Coef<float> c32{c->b32_0[0], c->b32_0[1], c->b32_0[2], 1.0f};
     ProfScope ps(c, PARIS_K_SETUP, 0.0);
     if (!rho0) {
-        launch_convert_beta<float>(c->g0, b64, ih2, c->b32_0, c->st);
+        launch_convert_beta(c->g0, b64, ih2, c->b32_0, c->st);
         if (c->half0) launch_convert_beta_half(c->g0, b64, c->b16_0, c->st);
     }
     if (c->dirichlet) {  // the diagonal excess, scaled like the FP32 coefficients
