@@ -42,11 +42,21 @@ __device__ __forceinline__ void tail_split(unsigned t, unsigned n0, unsigned n1,
     k = (int)kk;
 }
 
+// A periodic axis of odd length joins cells of one colour across its seam: there
+// a pass takes its own colour's values as they were before it (an update in the
+// threads' order would not be undone by the reversed one, and the V-cycle would
+// not be symmetric, which conjugate gradients needs).
+__device__ __forceinline__ bool odd_seam(const Geo& g) {
+    return (!g.wx && (g.nx & 1)) || (!g.wy && (g.ny & 1)) || (!g.wz && (g.nz & 1));
+}
+
 // One colour pass of over-relaxed red-black Gauss-Seidel on a tail level (the
-// update of rbgs_kernel; zero: x taken as 0, the other colour zeroed).
+// update of rbgs_kernel; zero: x taken as 0, the other colour zeroed).  tmp: a
+// value per cell, for the new values until all are formed (odd_seam).
 template <typename T>
-__device__ void tail_pass(const TailLevel<T>& L, int color, bool zero, T omega) {
+__device__ void tail_pass(const TailLevel<T>& L, int color, bool zero, T omega, T* tmp) {
     const Geo g = L.g;
+    const bool seam = !zero && odd_seam(g);
     const int npair = (g.nx + 1) / 2;
     const int total = npair * g.ny * g.nz;
     for (int t = threadIdx.x; t < total; t += blockDim.x) {
@@ -66,19 +76,27 @@ __device__ void tail_pass(const TailLevel<T>& L, int color, bool zero, T omega) 
 #pragma unroll
                 for (int q = 0; q < 6; ++q) acc = fma(s.b[q], L.x[s.nb[q]], acc);
                 const T xc = L.x[c];
-                L.x[c] = fma(omega, fma(L.w[c], acc, -xc), xc);
+                (seam ? tmp : L.x)[c] = fma(omega, fma(L.w[c], acc, -xc), xc);
             }
         }
         if (zero && io < g.nx) L.x[g.cidx(io, j, k)] = T(0);
     }
+    if (!seam) return;
+    __syncthreads();
+    for (int t = threadIdx.x; t < total; t += blockDim.x) {
+        int tp, j, k;
+        tail_split((unsigned)t, (unsigned)npair, (unsigned)g.ny, L.mp, L.my, tp, j, k);
+        const int i = 2 * tp + ((j + k + color) & 1);
+        if (i < g.nx) L.x[g.cidx(i, j, k)] = tmp[g.cidx(i, j, k)];
+    }
 }
 
 template <typename T>
-__device__ void tail_smooth(const TailLevel<T>& L, int sweeps, bool first_zero, bool reverse, T omega) {
+__device__ void tail_smooth(const TailLevel<T>& L, int sweeps, bool first_zero, bool reverse, T omega, T* tmp) {
     for (int s = 0; s < sweeps; ++s) {
-        tail_pass<T>(L, reverse ? 1 : 0, first_zero && s == 0, omega);
+        tail_pass<T>(L, reverse ? 1 : 0, first_zero && s == 0, omega, tmp);
         __syncthreads();
-        tail_pass<T>(L, reverse ? 0 : 1, false, omega);
+        tail_pass<T>(L, reverse ? 0 : 1, false, omega, tmp);
         __syncthreads();
     }
 }
@@ -224,7 +242,7 @@ __device__ void tail_levels(TailShared<T>& ts, int n, int nu1, int nu2, T omega,
     for (int l = 0; l < n - 1; ++l) {
         const TailLevel<T> L = ts.L[l];  // in registers: the loops below store through its pointers
         if (nu1 > 0) {
-            tail_smooth<T>(L, nu1, true, false, omega);
+            tail_smooth<T>(L, nu1, true, false, omega, ts.term);
         } else {
             const int cells = L.g.nx * L.g.ny * L.g.nz;
             for (int c = threadIdx.x; c < cells; c += blockDim.x) L.x[c] = T(0);
@@ -239,7 +257,7 @@ __device__ void tail_levels(TailShared<T>& ts, int n, int nu1, int nu2, T omega,
         tail_prolong<T>(ts.L[l + 1], ts.L[l]);
         __syncthreads();
         const TailLevel<T> L = ts.L[l];
-        if (nu2 > 0) tail_smooth<T>(L, nu2, false, true, omega);
+        if (nu2 > 0) tail_smooth<T>(L, nu2, false, true, omega, ts.term);
     }
 }
 
@@ -388,7 +406,7 @@ __device__ __forceinline__ int pair_cell(const Pair<T>& o, int& xl, int& xr, T& 
 }
 
 template <int M, typename T>
-__device__ __forceinline__ void pair_pass(const Pair<T>& o, T* x, bool zero, T omega) {
+__device__ __forceinline__ void pair_pass(const Pair<T>& o, T* x, bool zero, bool seam, T omega) {
     int xl, xr;
     T bl, br;
     const int c = pair_cell<M>(o, xl, xr, bl, br);
@@ -398,29 +416,34 @@ __device__ __forceinline__ void pair_pass(const Pair<T>& o, T* x, bool zero, T o
         if (io >= 0) x[io] = T(0);
         return;
     }
-    if (c < 0) return;
-    T acc = o.f[M];
-    acc = fma(bl, x[xl], acc);
-    acc = fma(br, x[xr], acc);
-    acc = fma(o.by[M][0], x[c + o.oym], acc);
-    acc = fma(o.by[M][1], x[c + o.oyp], acc);
-    acc = fma(o.bz[M][0], x[c + o.ozm], acc);
-    acc = fma(o.bz[M][1], x[c + o.ozp], acc);
-    const T xc = x[c];
-    x[c] = fma(omega, fma(o.w[M], acc, -xc), xc);
+    T xn = T(0);
+    if (c >= 0) {
+        T acc = o.f[M];
+        acc = fma(bl, x[xl], acc);
+        acc = fma(br, x[xr], acc);
+        acc = fma(o.by[M][0], x[c + o.oym], acc);
+        acc = fma(o.by[M][1], x[c + o.oyp], acc);
+        acc = fma(o.bz[M][0], x[c + o.ozm], acc);
+        acc = fma(o.bz[M][1], x[c + o.ozp], acc);
+        const T xc = x[c];
+        xn = fma(omega, fma(o.w[M], acc, -xc), xc);
+    }
+    if (seam) __syncthreads();  // odd_seam: after all reads
+    if (c >= 0) x[c] = xn;
 }
 
 template <typename T>
-__device__ __forceinline__ void pair_smooth(const Pair<T>& o, T* x, int sweeps, bool first_zero, bool reverse, T omega) {
+__device__ __forceinline__ void pair_smooth(const Pair<T>& o, T* x, int sweeps, bool first_zero, bool reverse, bool seam,
+                                            T omega) {
     for (int s = 0; s < sweeps; ++s) {
         if (!reverse) {
-            pair_pass<0>(o, x, first_zero && s == 0, omega);
+            pair_pass<0>(o, x, first_zero && s == 0, seam, omega);
             __syncthreads();
         }
-        pair_pass<1>(o, x, false, omega);
+        pair_pass<1>(o, x, false, seam, omega);
         __syncthreads();
         if (reverse) {
-            pair_pass<0>(o, x, false, omega);
+            pair_pass<0>(o, x, false, seam, omega);
             __syncthreads();
         }
     }
@@ -475,7 +498,7 @@ __device__ __forceinline__ void small_restrict(const Geo& fg, const TailLevel<T>
         const int n2 = child_count(K, cg.nz, fg.nz, fa2);
         const T* p = term + ((K * fa2) * fg.ny + J * fa1) * fg.nx + I * fa0;
         T sum = T(0);
-        if (n0 + n1 + n2 == 6) {
+        if (n0 == 2 && n1 == 2 && n2 == 2) {
 #pragma unroll
             for (int dk = 0; dk < 2; ++dk)
 #pragma unroll
@@ -516,7 +539,8 @@ __global__ void __launch_bounds__(kSmallThreads) tail_small_kernel(const __grid_
     pair_rhs<1>(o0, a.L[0].f);
     __syncthreads();
     const bool sig = a.L[0].sig != nullptr;
-    pair_smooth(o0, x[0], a.nu1, true, false, a.omega);
+    const bool seam0 = odd_seam(a.L[0].g), seam1 = NH == 2 && odd_seam(a.L[NH - 1].g);
+    pair_smooth(o0, x[0], a.nu1, true, false, seam0, a.omega);
     pair_term<0>(o0, x[0], sig, term);
     pair_term<1>(o0, x[0], sig, term);
     __syncthreads();
@@ -525,7 +549,7 @@ __global__ void __launch_bounds__(kSmallThreads) tail_small_kernel(const __grid_
         __syncthreads();
         pair_rhs<0>(o1, f1);
         pair_rhs<1>(o1, f1);
-        pair_smooth(o1, x[NH - 1], a.nu1, true, false, a.omega);
+        pair_smooth(o1, x[NH - 1], a.nu1, true, false, seam1, a.omega);
         pair_term<0>(o1, x[NH - 1], sig, term);
         pair_term<1>(o1, x[NH - 1], sig, term);
         __syncthreads();
@@ -552,13 +576,13 @@ __global__ void __launch_bounds__(kSmallThreads) tail_small_kernel(const __grid_
         pair_prolong<0>(o1, x[NH - 1], xc);
         pair_prolong<1>(o1, x[NH - 1], xc);
         __syncthreads();
-        pair_smooth(o1, x[NH - 1], a.nu2, false, true, a.omega);
+        pair_smooth(o1, x[NH - 1], a.nu2, false, true, seam1, a.omega);
     }
     const T* up = NH == 2 ? x[NH - 1] : xc;
     pair_prolong<0>(o0, x[0], up);
     pair_prolong<1>(o0, x[0], up);
     __syncthreads();
-    pair_smooth(o0, x[0], a.nu2, false, true, a.omega);
+    pair_smooth(o0, x[0], a.nu2, false, true, seam0, a.omega);
     const int cells = a.L[0].g.nx * a.L[0].g.ny * a.L[0].g.nz;
     for (int e = threadIdx.x; e < cells; e += kSmallThreads) a.L[0].x[e] = x[0][e];
 }
