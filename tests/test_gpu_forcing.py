@@ -170,3 +170,35 @@ def test_forcing_rejects_invalid_arguments(paris):
                               (0.1, (0, 0, 0), -1e-3), (float("inf"), (0, 0, 0), 1e-3)):
             with pytest.raises(paris.ParisError):
                 ctx.predictor_forcing(C, None, 2.0, 1.0, sigma, g, tau, *u)
+
+
+@pytest.mark.parametrize("g", [(0.0, 0.0, 0.0), (0.3, 0.0, -9.81)], ids=["no_gravity", "gravity"])
+@pytest.mark.parametrize("grid", [pi.Grid(40, 18, 12, 1 / 40, (P, W, P)), pi.Grid(33, 9, 11, 0.05, (W, P, W))],
+                         ids=lambda g: f"{g.nx}x{g.ny}x{g.nz}")
+def test_cells_of_one_fluid(paris, grid, g):
+    """Regions of C exactly 0 and 1 (the cells whose FP64 arithmetic is
+    skipped), signed zeros, values next to 1 and mixed cells between them,
+    with infinite, NaN and huge curvatures inside the regions: beta and u* as
+    the oracle has them, non-finite where it is."""
+    rng = np.random.default_rng(64)
+    C = np.zeros(grid.shape)
+    C[:, : grid.ny // 2] = 1.0
+    C[: grid.nz // 3, :, : grid.nx // 2] = rng.choice([0.0, -0.0, 1.0, 1 - 2.0**-53, 0.25, 0.75],
+                                                      (grid.nz // 3, grid.ny, grid.nx // 2))
+    kappa = rng.normal(0.0, 40.0, grid.shape)
+    kappa[-2, 1, 3], kappa[-3, -2, 5], kappa[-2, -2, 9] = np.nan, np.inf, 1e300
+    rho1, rho2, sigma, tau = 1000.0, 1.2, 0.07, 2e-3
+    un = [rng.normal(size=grid.face_shape(a)) for a in range(3)]
+    with np.errstate(invalid="ignore"):
+        want = F.predictor(grid, *[x.copy() for x in un], C, kappa, sigma, g, rho1, rho2, tau)
+    beta_ref = oracle.face_coeffs(grid, C, rho1, rho2)
+    with paris.Context(grid) as ctx:
+        u = [dev(x) for x in un]
+        beta = ctx.predictor_forcing(dev(C), dev(kappa), rho1, rho2, sigma, g, tau, *u)
+        for a in range(3):
+            np.testing.assert_allclose(host(beta[a]), beta_ref[a], rtol=4e-16, atol=0)
+            fin = np.isfinite(want[a])
+            assert not fin.all()
+            np.testing.assert_array_equal(np.isfinite(host(u[a])), fin)
+            scale = np.abs(want[a][fin]).max()
+            np.testing.assert_allclose(host(u[a])[fin], want[a][fin], rtol=0, atol=2e-15 * scale)
