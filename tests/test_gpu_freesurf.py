@@ -216,3 +216,12 @@ def test_free_surface_tail_bit_identical(paris, grid, precision):
             out.append([host(p)] + [host(x) for x in u])
     for a, b in zip(*out):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("grid", [pi.Grid(128, 12, 10, 1 / 128, (P, W, W)), pi.Grid(132, 9, 7, 1 / 132, (P, P, W)),
+                                  pi.Grid(260, 8, 6, 1 / 260, (P, W, P))], ids=lambda g: f"{g.nx}x{g.ny}x{g.nz}")
+def test_long_rows_match_oracle(paris, grid):
+    """Rows of at least a warp's vectors (the product with four cells per
+    thread): a part of a block of rows, more than one block along x, walls and
+    seams in y and z; the bars of the short rows."""
+    test_free_surface_step_matches_oracle(paris, grid, "MIXED")

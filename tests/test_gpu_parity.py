@@ -537,3 +537,21 @@ def test_finest_level_boxes_bit_identical(paris, grid, nu, half):
             out.append([host(p)] + [host(x) for x in u])
     for a, b in zip(*out):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("grid", [pi.Grid(128, 11, 10, 1 / 128, (P, W, W)), pi.Grid(132, 8, 7, 1 / 132, (P, P, P)),
+                                  pi.Grid(260, 8, 6, 1 / 260, (P, W, P))], ids=lambda g: f"{g.nx}x{g.ny}x{g.nz}")
+def test_long_rows_of_face_arrays_match_oracle(paris, grid):
+    """The mixed step from FP32 face arrays with rows of at least a warp's
+    vectors, to the parity bar of the other grids."""
+    pr = pi.random_problem(grid, seed=15, rho1=100.0)
+    ref = oracle.projection_step(grid, pr.C, pr.rho1, pr.rho2, pr.dt, pr.u, pr.v, pr.w)
+    with ctx_for(paris, grid, precision=paris.MIXED, level0_density=0) as ctx:
+        u = [dev(x) for x in (pr.u, pr.v, pr.w)]
+        p = torch.zeros(grid.shape, dtype=torch.float64, device="cuda")
+        st = ctx.projection_step(dev(pr.C), pr.rho1, pr.rho2, pr.dt, *u, p)
+    assert st["converged"] == 1 and st["fell_back"] == 0, st
+    assert np.abs(host(p) - ref.p).max() <= 1e-8 * np.abs(ref.p).max()
+    umax = max(np.abs(x).max() for x in (pr.u, pr.v, pr.w))
+    for a in range(3):
+        assert np.abs(host(u[a]) - ref.u[a]).max() <= 1e-8 * umax
