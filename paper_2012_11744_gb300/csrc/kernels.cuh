@@ -592,10 +592,9 @@ void launch_check_arithmetic(const double* v, int64_t n, int shift, unsigned lon
                              cudaStream_t st);
 
 // ------------------------------------------------------------ adjoint -----
-// out = D (B g) (walls carry no flux); partials (sum, max|out|, nonfinite)
-int64_t launch_weighted_div(const Geo& g, const double* bx, const double* by, const double* bz,
-                            const double* gx, const double* gy, const double* gz, double inv_h,
-                            double* out, double* partials, cudaStream_t st);
+// out = D (B g) (walls carry no flux)
+void launch_weighted_div(const Geo& g, const double* bx, const double* by, const double* bz, const double* gx,
+                         const double* gy, const double* gz, double inv_h, double* out, cudaStream_t st);
 // dLoss/du* = g - G q and dLoss/dbeta = dt (G p)(G q - g) on non-wall faces
 void launch_adjoint_faces(const Geo& g, const double* p, const double* q, double inv_h, double dt,
                           const double* gx, const double* gy, const double* gz, double* usx,

@@ -1725,7 +1725,7 @@ paris_status paris_project_adjoint(paris_ctx* c, const double* bx, const double*
     if (c->solid) return PARIS_ERR_INVALID_ARG;  // the adjoint of the blocking is not built
     const double inv_h = 1.0 / c->grid.h;
     // right-hand side of the adjoint solve: D (B g)
-    launch_weighted_div(c->g0, bx, by, bz, gu, gv, gw, inv_h, c->rhs, c->partials, c->st);
+    launch_weighted_div(c->g0, bx, by, bz, gu, gv, gw, inv_h, c->rhs, c->st);
     CK(cudaGetLastError());
     // the adjoint solve uses the same symmetric operator L = D B G
     paris_status solve = paris_poisson_solve(c, bx, by, bz, c->rhs, q, st);
