@@ -1783,17 +1783,20 @@ __global__ void update_xr_kernel(int64_t n, const Scal* s, const T* __restrict__
     // rev: the vectors from the end (a pass that starts where the previous one ended)
     auto at = [&](int64_t e) { return rev ? nv - 1 - e : e; };
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; i + (U - 1) * stride < nv; i += U * stride) {
+    for (; i < nv; i += U * stride) {
         VT dv[U], qv[U], xv[U], rv[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if (!NOX) dv[u] = reinterpret_cast<const VT*>(d)[at(i + u * stride)];
-            qv[u] = reinterpret_cast<const VT*>(q)[at(i + u * stride)];
-            if (!NOX) xv[u] = reinterpret_cast<VT*>(x)[at(i + u * stride)];
-            rv[u] = reinterpret_cast<VT*>(r)[at(i + u * stride)];
+            if (i + u * stride < nv) {
+                if (!NOX) dv[u] = reinterpret_cast<const VT*>(d)[at(i + u * stride)];
+                qv[u] = reinterpret_cast<const VT*>(q)[at(i + u * stride)];
+                if (!NOX) xv[u] = reinterpret_cast<VT*>(x)[at(i + u * stride)];
+                rv[u] = reinterpret_cast<VT*>(r)[at(i + u * stride)];
+            }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
+            if (i + u * stride >= nv) break;
             const T* de = reinterpret_cast<const T*>(&dv[u]);
             const T* qe = reinterpret_cast<const T*>(&qv[u]);
             T* xe = reinterpret_cast<T*>(&xv[u]);
@@ -1803,23 +1806,6 @@ __global__ void update_xr_kernel(int64_t n, const Scal* s, const T* __restrict__
             if (!NOX) reinterpret_cast<VT*>(x)[at(i + u * stride)] = xv[u];
             reinterpret_cast<VT*>(r)[at(i + u * stride)] = rv[u];
         }
-    }
-    for (; i < nv; i += stride) {
-        VT dv, xv;
-        if (!NOX) {
-            dv = reinterpret_cast<const VT*>(d)[at(i)];
-            xv = reinterpret_cast<VT*>(x)[at(i)];
-        }
-        const VT qv = reinterpret_cast<const VT*>(q)[at(i)];
-        VT rv = reinterpret_cast<VT*>(r)[at(i)];
-        const T* de = reinterpret_cast<const T*>(&dv);
-        const T* qe = reinterpret_cast<const T*>(&qv);
-        T* xe = reinterpret_cast<T*>(&xv);
-        T* re = reinterpret_cast<T*>(&rv);
-#pragma unroll
-        for (int w = 0; w < W; ++w) one(de[w], qe[w], xe[w], re[w], l2[0], li[0]);
-        if (!NOX) reinterpret_cast<VT*>(x)[at(i)] = xv;
-        reinterpret_cast<VT*>(r)[at(i)] = rv;
     }
     PARIS_TAIL_FOR(c, nv * W, n) {
         T xv = NOX ? T(0) : x[c], rv = r[c];
@@ -1873,16 +1859,19 @@ __global__ void dot2_kernel(int64_t n, const T* __restrict__ a, const T* __restr
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     auto at = [&](int64_t e) { return rev ? nv - 1 - e : e; };  // rev: from the end
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; i + (U - 1) * stride < nv; i += U * stride) {
+    for (; i < nv; i += U * stride) {
         VT av[U], bv[U], cv[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            av[u] = __ldg(reinterpret_cast<const VT*>(a) + at(i + u * stride));
-            bv[u] = __ldg(reinterpret_cast<const VT*>(b) + at(i + u * stride));
-            if (c) cv[u] = __ldg(reinterpret_cast<const VT*>(c) + at(i + u * stride));
+            if (i + u * stride < nv) {
+                av[u] = __ldg(reinterpret_cast<const VT*>(a) + at(i + u * stride));
+                bv[u] = __ldg(reinterpret_cast<const VT*>(b) + at(i + u * stride));
+                if (c) cv[u] = __ldg(reinterpret_cast<const VT*>(c) + at(i + u * stride));
+            }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
+            if (i + u * stride >= nv) break;
             const T* ae = reinterpret_cast<const T*>(&av[u]);
             const T* be = reinterpret_cast<const T*>(&bv[u]);
 #pragma unroll
@@ -1892,20 +1881,6 @@ __global__ void dot2_kernel(int64_t n, const T* __restrict__ a, const T* __restr
 #pragma unroll
                 for (int w = 0; w < W; ++w) s1[u] = fma(ae[w], ce[w], s1[u]);
             }
-        }
-    }
-    for (; i < nv; i += stride) {
-        const VT av = reinterpret_cast<const VT*>(a)[at(i)];
-        const VT bv = reinterpret_cast<const VT*>(b)[at(i)];
-        const T* ae = reinterpret_cast<const T*>(&av);
-        const T* be = reinterpret_cast<const T*>(&bv);
-#pragma unroll
-        for (int w = 0; w < W; ++w) s0[0] = fma(ae[w], be[w], s0[0]);
-        if (c) {
-            const VT cv = reinterpret_cast<const VT*>(c)[at(i)];
-            const T* ce = reinterpret_cast<const T*>(&cv);
-#pragma unroll
-            for (int w = 0; w < W; ++w) s1[0] = fma(ae[w], ce[w], s1[0]);
         }
     }
     PARIS_TAIL_FOR(e, nv * W, n) {
