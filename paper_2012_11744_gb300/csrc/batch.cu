@@ -46,6 +46,7 @@ struct BLevel {
     float* b[3];  // coefficients beta/h_a^2 of this level
     float* x;     // level solution (level 0: the V-cycle output)
     float* f;     // level right-hand side (level 0: the V-cycle input)
+    float* t;     // second array of x on a level with an odd_seam (else null)
     unsigned mx, my, mp, mq;  // fast_div multipliers of nx, ny, the pairs and the quads of a row
 };
 
@@ -538,6 +539,27 @@ __device__ __noinline__ void rb_pairs(int rank, int ncta, const BLevel& L, const
     }
 }
 
+// The colour pass of a level with an odd_seam, cell by cell, from x to xo (all
+// cells written).  Same update as pass_store.
+__device__ __noinline__ void rb_seam(int rank, int ncta, const BLevel& L, const float* f, const float* x, float* xo,
+                                     int color, float omega, bool zero) {
+    const Geo g = L.g;
+    const float *bx = L.b[0], *by = L.b[1], *bz = L.b[2];
+    const unsigned mx = L.mx, my = L.my;
+    GLOOP(c, g.ncell()) {
+        PassCell p;
+        decomp(g, mx, my, c, p.i, p.j, p.k);
+        p.io = g.nx;
+        if (((p.i + p.j + p.k) & 1) != color) {
+            xo[c] = zero ? 0.f : x[c];
+            continue;
+        }
+        PassLoad d;
+        pass_load(d, g, bx, by, bz, f, x, p, zero);
+        pass_store(d, g, xo, p, omega, zero);
+    }
+}
+
 // One colour pass on a level: quads where every thread of the group gets at
 // least two planes of one, pairs otherwise.
 __device__ __forceinline__ void rb_pass(int rank, int ncta, const BLevel& L, const float* f, float* x, int color,
@@ -705,10 +727,13 @@ constexpr int64_t kSoloCells = 4096;
 __device__ bool smooth_level(Grp& cx, const BParams& P, const BLevel& L, const float* f, float* x, int sweeps,
                              bool first_zero, bool reverse, bool solo) {
     const int rank = solo ? 0 : cx.rank, ncta = solo ? 1 : cx.ncta, c0 = reverse ? 1 : 0;
+    float* t = L.t;  // an odd_seam: the first colour's pass goes there, the second's back into x
     for (int s = 0; s < sweeps; ++s) {
-        rb_pass(rank, ncta, L, f, x, c0, P.omega, first_zero && s == 0);
+        if (t) rb_seam(rank, ncta, L, f, x, t, c0, P.omega, first_zero && s == 0);
+        else rb_pass(rank, ncta, L, f, x, c0, P.omega, first_zero && s == 0);
         if (!step_sync(cx, solo)) return false;
-        rb_pass(rank, ncta, L, f, x, 1 - c0, P.omega, false);
+        if (t) rb_seam(rank, ncta, L, f, t, x, 1 - c0, P.omega, false);
+        else rb_pass(rank, ncta, L, f, x, 1 - c0, P.omega, false);
         if (!step_sync(cx, solo)) return false;
     }
     return true;
@@ -1334,6 +1359,7 @@ paris_status paris_batch_create(paris_batch** out, int n, const paris_grid* grid
             L.mq = fast_div_mul(std::max(1, L.g.nx / 4));
             L.x = l == 0 ? nullptr : balloc<float>(b, L.g.ncell(), e);
             L.f = l == 0 ? nullptr : balloc<float>(b, L.g.ncell(), e);
+            L.t = odd_seam(L.g) ? balloc<float>(b, L.g.ncell(), e) : nullptr;
         }
         const int64_t N = H.g0.ncell();
         for (int a = 0; a < 3; ++a) I.b64[a] = balloc<double>(b, H.g0.nface(a), e);

@@ -47,6 +47,15 @@ __host__ __device__ inline int parent_of(int i, int cn, int f) {
     return I < cn ? I : cn - 1;
 }
 
+// A periodic axis of odd length joins cells of one colour across its seam.  There
+// a colour pass takes its own colour's values as they were before it: updated
+// in place, a cell would meet the neighbour's old or new value depending on the
+// order of the threads, and no order is undone by the reversed one, so the V-cycle
+// would be neither reproducible nor symmetric (which conjugate gradients need).
+__host__ __device__ inline bool odd_seam(const Geo& g) {
+    return (!g.wx && (g.nx & 1)) || (!g.wy && (g.ny & 1)) || (!g.wz && (g.nz & 1));
+}
+
 // Coefficient set of one level: face arrays and a uniform scale (1/h^2 for
 // arrays holding beta itself, 1 for arrays that are already scaled), and an
 // optional per-cell diagonal excess sig in the units of the face arrays: the

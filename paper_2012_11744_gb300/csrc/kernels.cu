@@ -17,6 +17,7 @@
 #include <cmath>
 #include <climits>
 #include <cstdio>
+#include <type_traits>
 
 #include "kernels.cuh"
 
@@ -1072,13 +1073,15 @@ void launch_coarse_solve(const Geo& g, const double* inv, const T* f, T* x, cuda
 // w_c = 1/sum_f beta_f.  One thread per x-pair (2t, 2t+1) of a row updates
 // the member of colour `color` ((i+j+k) even = red = 0).  With zero_init the
 // incoming x is taken as zero and the other member of the pair is zeroed.
+// In place, or (TWO) into a second array with the other member copied, for a
+// level with an odd_seam.
 
-template <typename T, typename TB, bool USEW, bool I32>
+template <typename T, typename TB, bool USEW, bool I32, bool TWO>
 __global__ void __launch_bounds__(kTX* pass_rows<T>()) rbgs_kernel(Geo g, const TB* __restrict__ bx,
                                                        const TB* __restrict__ by,
                                                        const TB* __restrict__ bz, T scale,
                                                        const T* __restrict__ w,
-                                                       const T* __restrict__ f, T* __restrict__ x,
+                                                       const T* __restrict__ f, T* __restrict__ x, T* __restrict__ xo,
                                                        int color, T omega, int zero_init, int k0) {
     pdl_wait();
     const int t = blockIdx.x * kTX + threadIdx.x;
@@ -1111,9 +1114,13 @@ __global__ void __launch_bounds__(kTX* pass_rows<T>()) rbgs_kernel(Geo g, const 
             const T xc = x[c];
             xn = fma(omega, fma(USEW ? w[c] : inv_sum6(s.b), acc, -xc), xc);
         }
-        x[c] = xn;
+        (TWO ? xo : x)[c] = xn;
     }
-    if (zero_init && io < g.nx) x[g.cidx(io, j, k)] = T(0);
+    if ((TWO || zero_init) && io < g.nx) {
+        const int64_t co = g.cidx(io, j, k);
+        if (zero_init) (TWO ? xo : x)[co] = T(0);
+        else xo[co] = x[co];
+    }
 }
 
 // Four consecutive cells of a row as one 16-byte (FP32) or two 16-byte
@@ -1237,12 +1244,12 @@ __device__ __forceinline__ void rbgs4_row(const Geo& g, const TB* __restrict__ b
 // The row's two new values are computed before either is stored (the FP64
 // form's passes measured 4 % faster so than with the stores inside the
 // update).
-template <typename T, bool USEW, typename TB = T>
+template <typename T, bool USEW, bool TWO, typename TB = T>
 __global__ void __launch_bounds__(kTX* pass_rows<T>()) rbgs4_kernel(Geo g, const TB* __restrict__ bx,
                                                         const TB* __restrict__ by,
                                                         const TB* __restrict__ bz, T scale,
                                                         const T* __restrict__ w,
-                                                        const T* __restrict__ f, T* __restrict__ x,
+                                                        const T* __restrict__ f, T* __restrict__ x, T* __restrict__ xo,
                                                         int color, T omega, int zero_init, int k0) {
     pdl_wait();
     const int j = blockIdx.y * pass_rows<T>() + threadIdx.y;
@@ -1263,73 +1270,68 @@ __global__ void __launch_bounds__(kTX* pass_rows<T>()) rbgs4_kernel(Geo g, const
     const int c0 = (k * g.ny + j) * g.nx + i0;
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-        const int li = 2 * u + M;
-        x[c0 + li] = xn[u];
-        if (zero_init) x[c0 + li + 1 - 2 * M] = T(0);  // the other member of the pair
+        const int li = 2 * u + M, lo = li + 1 - 2 * M;  // the other member of the pair
+        (TWO ? xo : x)[c0 + li] = xn[u];
+        if (zero_init) (TWO ? xo : x)[c0 + lo] = T(0);
+        else if (TWO) xo[c0 + lo] = x[c0 + lo];
     }
 }
 
+// x and xo as the kernels take them: xo null for a pass in place
 template <typename T>
-void launch_rbgs(const Geo& g, const Coef<T>& cf, const T* w, const T* f, T* x, int color,
+void launch_rbgs(const Geo& g, const Coef<T>& cf, const T* w, const T* f, T* x, T* xo, int color,
                  double omega, bool zero_init, cudaStream_t st, int k0, int k1) {
     if (k1 < 0) k1 = g.nz;
+    const dim3 block(kTX, pass_rows<T>());
+    const int rows = (g.ny + pass_rows<T>() - 1) / pass_rows<T>(), zero = zero_init ? 1 : 0;
+    // FP32: recomputing 1/D from the coefficients already loaded is cheaper
+    // than reading it; FP64: the division costs more than the read.  A diagonal
+    // excess is in w only.
+    const bool use_w = sizeof(T) == 8 || cf.sig;
     // four cells per thread where a row fills at least a warp (shorter rows
     // would leave lanes idle: the single-pair kernel serves them)
     if (g.nx % 4 == 0 && g.nx >= 4 * kTX && !g.wx && fits_i32(g) && aligned16(cf.bx, cf.by, cf.bz, f) &&
-        aligned16(x) && ((sizeof(T) == 4 && !cf.sig) || aligned16(w))) {
-        dim3 gr((g.nx / 4 + kTX - 1) / kTX, (g.ny + pass_rows<T>() - 1) / pass_rows<T>(), k1 - k0);
-        if (sizeof(T) == 8 || cf.sig)  // w read (FP64, or a diagonal excess the coefficients do not hold)
-            launch_pdl(rbgs4_kernel<T, true>, gr, dim3(kTX, pass_rows<T>()), 0, st, g, cf.bx, cf.by, cf.bz, cf.scale, w, f,
-                x, color, (T)omega, zero_init ? 1 : 0, k0);
-        else
-            launch_pdl(rbgs4_kernel<T, false>, gr, dim3(kTX, pass_rows<T>()), 0, st, g, cf.bx, cf.by, cf.bz, cf.scale, w,
-                f, x, color, (T)omega, zero_init ? 1 : 0, k0);
+        aligned16(x, xo) && (!use_w || aligned16(w))) {
+        const dim3 gr((g.nx / 4 + kTX - 1) / kTX, rows, k1 - k0);
+        auto* k = use_w ? (xo ? rbgs4_kernel<T, true, true> : rbgs4_kernel<T, true, false>)
+                        : (xo ? rbgs4_kernel<T, false, true> : rbgs4_kernel<T, false, false>);
+        launch_pdl(k, gr, block, 0, st, g, cf.bx, cf.by, cf.bz, cf.scale, w, f, x, xo, color, (T)omega, zero, k0);
         count_launch();
         return;
     }
-    const int npair = (g.nx + 1) / 2;
-    dim3 gr((npair + kTX - 1) / kTX, (g.ny + pass_rows<T>() - 1) / pass_rows<T>(), k1 - k0);
-    // FP32: recomputing 1/D from the coefficients already loaded is cheaper
-    // than reading it; FP64: the division costs more than the read
-    const bool i32 = fits_i32(g);
-    if (sizeof(T) == 8 || cf.sig) {
-        if (i32)
-            launch_pdl(rbgs_kernel<T, T, true, true>, gr, dim3(kTX, pass_rows<T>()), 0, st, g, cf.bx, cf.by, cf.bz,
-                cf.scale, w, f, x, color, (T)omega, zero_init ? 1 : 0, k0);
-        else
-            launch_pdl(rbgs_kernel<T, T, true, false>, gr, dim3(kTX, pass_rows<T>()), 0, st, g, cf.bx, cf.by, cf.bz,
-                cf.scale, w, f, x, color, (T)omega, zero_init ? 1 : 0, k0);
-    } else {
-        if (i32)
-            launch_pdl(rbgs_kernel<T, T, false, true>, gr, dim3(kTX, pass_rows<T>()), 0, st, g, cf.bx, cf.by, cf.bz,
-                cf.scale, w, f, x, color, (T)omega, zero_init ? 1 : 0, k0);
-        else
-            launch_pdl(rbgs_kernel<T, T, false, false>, gr, dim3(kTX, pass_rows<T>()), 0, st, g, cf.bx, cf.by, cf.bz,
-                cf.scale, w, f, x, color, (T)omega, zero_init ? 1 : 0, k0);
-    }
+    const dim3 gr(((g.nx + 1) / 2 + kTX - 1) / kTX, rows, k1 - k0);
+    auto pick = [&](auto two) {
+        constexpr bool TWO = decltype(two)::value;
+        return fits_i32(g) ? (use_w ? rbgs_kernel<T, T, true, true, TWO> : rbgs_kernel<T, T, false, true, TWO>)
+                           : (use_w ? rbgs_kernel<T, T, true, false, TWO> : rbgs_kernel<T, T, false, false, TWO>);
+    };
+    launch_pdl(xo ? pick(std::true_type{}) : pick(std::false_type{}), gr, block, 0, st, g, cf.bx, cf.by, cf.bz, cf.scale,
+               w, f, x, xo, color, (T)omega, zero, k0);
     count_launch();
 }
 
-void launch_rbgs_h(const Geo& g, const __half* const b[3], float scale, const float* f, float* x,
+void launch_rbgs_h(const Geo& g, const __half* const b[3], float scale, const float* f, float* x, float* xo,
                    int color, double omega, bool zero_init, cudaStream_t st, int k0, int k1) {
     if (k1 < 0) k1 = g.nz;
+    const dim3 block(kTX, pass_rows<float>());
+    const int rows = (g.ny + pass_rows<float>() - 1) / pass_rows<float>(), zero = zero_init ? 1 : 0;
+    const float* w = nullptr;
     // four cells per thread where a row fills a warp (the update of the pair kernel)
-    if (g.nx % 4 == 0 && g.nx >= 4 * kTX && !g.wx && fits_i32(g) && aligned16(f, x) &&
+    if (g.nx % 4 == 0 && g.nx >= 4 * kTX && !g.wx && fits_i32(g) && aligned16(f, x, xo) &&
         ((((uintptr_t)b[0] | (uintptr_t)b[1] | (uintptr_t)b[2]) & 7u) == 0)) {
-        dim3 gr((g.nx / 4 + kTX - 1) / kTX, (g.ny + pass_rows<float>() - 1) / pass_rows<float>(), k1 - k0);
-        launch_pdl(rbgs4_kernel<float, false, __half>, gr, dim3(kTX, pass_rows<float>()), 0, st, g, b[0], b[1], b[2], scale,
-                   (const float*)nullptr, f, x, color, (float)omega, zero_init ? 1 : 0, k0);
+        launch_pdl(xo ? rbgs4_kernel<float, false, true, __half> : rbgs4_kernel<float, false, false, __half>,
+                   dim3((g.nx / 4 + kTX - 1) / kTX, rows, k1 - k0), block, 0, st, g, b[0], b[1], b[2], scale, w, f, x, xo,
+                   color, (float)omega, zero, k0);
         count_launch();
         return;
     }
-    const int npair = (g.nx + 1) / 2;
-    dim3 gr((npair + kTX - 1) / kTX, (g.ny + pass_rows<float>() - 1) / pass_rows<float>(), k1 - k0);
-    if (fits_i32(g))
-        launch_pdl(rbgs_kernel<float, __half, false, true>, gr, dim3(kTX, pass_rows<float>()), 0, st, g, b[0], b[1], b[2],
-            scale, nullptr, f, x, color, (float)omega, zero_init ? 1 : 0, k0);
-    else
-        launch_pdl(rbgs_kernel<float, __half, false, false>, gr, dim3(kTX, pass_rows<float>()), 0, st, g, b[0], b[1], b[2],
-            scale, nullptr, f, x, color, (float)omega, zero_init ? 1 : 0, k0);
+    auto pick = [&](auto two) {
+        constexpr bool TWO = decltype(two)::value;
+        return fits_i32(g) ? rbgs_kernel<float, __half, false, true, TWO> : rbgs_kernel<float, __half, false, false, TWO>;
+    };
+    launch_pdl(xo ? pick(std::true_type{}) : pick(std::false_type{}),
+               dim3(((g.nx + 1) / 2 + kTX - 1) / kTX, rows, k1 - k0), block, 0, st, g, b[0], b[1], b[2], scale, w, f, x, xo,
+               color, (float)omega, zero, k0);
     count_launch();
 }
 
@@ -2106,7 +2108,7 @@ cudaError_t stream_rates(const float* a, const float* b, const float* c, float* 
     template void launch_inv_diag<T>(int, const Geo*, const Coef<T>*, T* const*, cudaStream_t); \
     template void launch_coarse_inverse<T>(const Geo&, const Coef<T>&, double*, cudaStream_t); \
     template void launch_coarse_solve<T>(const Geo&, const double*, const T*, T*, cudaStream_t, bool); \
-    template void launch_rbgs<T>(const Geo&, const Coef<T>&, const T*, const T*, T*, int,     \
+    template void launch_rbgs<T>(const Geo&, const Coef<T>&, const T*, const T*, T*, T*, int, \
                                  double, bool, cudaStream_t, int, int);                        \
     template void launch_jacobi<T>(const Geo&, const Coef<T>&, const T*, const T*, const T*,  \
                                    T*, double, bool, cudaStream_t);                            \

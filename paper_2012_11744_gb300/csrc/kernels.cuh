@@ -405,11 +405,12 @@ template <typename T>
 void launch_coarse_solve(const Geo& g, const double* inv, const T* f, T* x, cudaStream_t st, bool keep_mean);
 
 // ------------------------------------------------------------ V-cycle -----
-// One red-black colour pass of over-relaxed Gauss-Seidel on A x = f, in
-// place, on the z-planes [k0, k1) (k1 < 0: all planes).
-// zero_init: x is taken as 0 on entry (the pass also zeroes the other colour).
+// One red-black colour pass of over-relaxed Gauss-Seidel on A x = f on the
+// z-planes [k0, k1) (k1 < 0: all planes): in place (xo null), or from x to a
+// second array xo (the other colour copied), which a level with an odd_seam needs.
+// zero_init: x is taken as 0 and not read (the pass also zeroes the other colour).
 template <typename T>
-void launch_rbgs(const Geo& g, const Coef<T>& cf, const T* w, const T* f, T* x, int color,
+void launch_rbgs(const Geo& g, const Coef<T>& cf, const T* w, const T* f, T* x, T* xo, int color,
                  double omega, bool zero_init, cudaStream_t st, int k0 = 0, int k1 = -1);
 // One fused red-black sweep (both colours, one pass) from xin to xout
 // (separate arrays; xin unread when zero_init).  first_color: colour
@@ -431,7 +432,7 @@ void launch_restrict_residual(const Geo& fine, const Coef<T>& cf, const T* f, co
                              const Geo& coarse, const int fac[3], T* fc, cudaStream_t st);
 // FP32 V-cycle with FP16 storage of the (unscaled) level-0 coefficients:
 // the colour pass and the residual restriction of the finest level.
-void launch_rbgs_h(const Geo& g, const __half* const b[3], float scale, const float* f, float* x,
+void launch_rbgs_h(const Geo& g, const __half* const b[3], float scale, const float* f, float* x, float* xo,
                    int color, double omega, bool zero_init, cudaStream_t st, int k0 = 0, int k1 = -1);
 void launch_restrict_residual_h(const Geo& fine, const __half* const b[3], float scale, const float* f,
                                 const float* x, const Geo& coarse, const int fac[3], float* fc,

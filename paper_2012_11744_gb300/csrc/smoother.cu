@@ -18,8 +18,9 @@
 //   * input and output are separate arrays (ping-pong), so halo reads never
 //     see another CTA's updates.
 //
-// The result is bit-identical to one in-place pass of each colour (same
-// arithmetic in the same order) when every periodic axis has even length.
+// The result is bit-identical to one pass of each colour (same arithmetic in
+// the same order), across the seam of an odd periodic axis too, where a colour
+// meets itself and takes its values as they were before the pass.
 // With ZERO the incoming solution is taken as zero and never read.
 // Indices are 32-bit: the host uses this kernel only for levels whose face
 // arrays hold fewer than 2^31 entries (rbgs_fused_fits).

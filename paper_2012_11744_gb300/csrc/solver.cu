@@ -502,7 +502,13 @@ void smooth(paris_ctx* c, int l, const Coef<T>& cf, const T* f, T* x, int sweeps
             const bool h16 = sizeof(T) == 4 && l == 0 && c->half0;
             const bool v0 = sizeof(T) == 4 && l == 0 && c->rho0;
             const double bsz = h16 ? 2.0 : (double)sz;
+            // across an odd periodic seam cells of one colour meet: the first colour's
+            // pass goes to the level's second buffer, the second's back into x
+            const bool seam = odd_seam(L.g);
             auto pass = [&](int color, bool zero, int a, int b) {
+                const bool back = seam && color != c0;
+                T* in = back ? Prec<T>::t(L) : x;
+                T* out = !seam ? nullptr : back ? x : Prec<T>::t(L);
                 if constexpr (sizeof(T) == 4) {
                     if (v0) {
                         // after a zero pass the other colour is still unwritten on the
@@ -516,16 +522,16 @@ void smooth(paris_ctx* c, int l, const Coef<T>& cf, const T* f, T* x, int sweeps
                     }
                     if (h16) {
                         // FP16 arrays hold beta itself: scale by 1/h^2 in the kernel
-                        launch_rbgs_h(L.g, c->b16_0, (float)(1.0 / (c->grid.h * c->grid.h)), f, x, color,
+                        launch_rbgs_h(L.g, c->b16_0, (float)(1.0 / (c->grid.h * c->grid.h)), f, in, out, color,
                                       o.omega, zero, c->st, a, b);
                         return;
                     }
                     if (l == 1 && c->rho0 && c->half_rho) {  // level 1 of the mixed step: FP16 coefficients
-                        launch_rbgs_h(L.g, L.b16, L.scale16, f, x, color, o.omega, zero, c->st, a, b);
+                        launch_rbgs_h(L.g, L.b16, L.scale16, f, in, out, color, o.omega, zero, c->st, a, b);
                         return;
                     }
                 }
-                launch_rbgs<T>(L.g, cf, Prec<T>::w(L), f, x, color, o.omega, zero, c->st, a, b);
+                launch_rbgs<T>(L.g, cf, Prec<T>::w(L), f, in, out, color, o.omega, zero, c->st, a, b);
             };
             auto first = [&](int a, int b) { pass(c0, z0, a, b); };
             auto second = [&](int a, int b) { pass(1 - c0, false, a, b); };

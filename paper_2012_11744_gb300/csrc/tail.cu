@@ -42,14 +42,6 @@ __device__ __forceinline__ void tail_split(unsigned t, unsigned n0, unsigned n1,
     k = (int)kk;
 }
 
-// A periodic axis of odd length joins cells of one colour across its seam: there
-// a pass takes its own colour's values as they were before it (an update in the
-// threads' order would not be undone by the reversed one, and the V-cycle would
-// not be symmetric, which conjugate gradients needs).
-__device__ __forceinline__ bool odd_seam(const Geo& g) {
-    return (!g.wx && (g.nx & 1)) || (!g.wy && (g.ny & 1)) || (!g.wz && (g.nz & 1));
-}
-
 // One colour pass of over-relaxed red-black Gauss-Seidel on a tail level (the
 // update of rbgs_kernel; zero: x taken as 0, the other colour zeroed).  tmp: a
 // value per cell, for the new values until all are formed (odd_seam).

@@ -158,3 +158,23 @@ def test_batch_quad_passes_with_walls(paris):
         for q in (i, i + 177):  # the first and the last copy
             assert st[q]["converged"] == 1, st[q]
             check_instance(pr, *out[q], ref=ref)
+
+
+def test_batch_odd_periodic_axes_bit_identical(paris):
+    """Cells of one colour that meet across an odd periodic seam are taken as
+    they were before the pass: two runs give the same bits, by groups of CTAs
+    and by one, on smoothed, coarsest and single levels."""
+    grids = [pi.Grid(33, 33, 33, 1 / 33, (P, P, P)), pi.Grid(50, 26, 34, 1 / 50, (W, P, P)),
+             pi.Grid(25, 24, 18, 1 / 25, (P, W, P)), pi.Grid(7, 5, 3, 1 / 7, (P, P, P)),
+             pi.Grid(12, 20, 28, 1 / 28, (P, P, P))]
+    probs = [pi.random_problem(g, seed=130 + i, rho1=100.0) for i, g in enumerate(grids)]
+    one, st, _ = run_batch(paris, probs)
+    two, _, _ = run_batch(paris, probs)
+    many, stm, ctas = run_batch(paris, probs * 60)
+    assert ctas < 302 + 60  # copies 10 and 59 have the same CTAs: the few left over go to the first ones
+    for i, pr in enumerate(probs):
+        assert st[i]["converged"] == 1 and stm[i]["converged"] == 1, (st[i], stm[i])
+        check_instance(pr, *one[i])
+        for x, y in ((one[i], two[i]), (many[i + 50], many[i + 295])):
+            for a, b in zip((x[0], *x[1]), (y[0], *y[1])):
+                np.testing.assert_array_equal(a, b)
