@@ -148,6 +148,7 @@ struct paris_ctx {
     bool cap_stream_broken = false;
     cudaGraphExec_t cg_exec[5] = {};
     int cg_kernels[5] = {};
+    float cg_scale16 = 0.f;  // level 1's scale16 in the graph of slot 2
 };
 
 namespace {
@@ -744,6 +745,13 @@ bool coarse_graph_launch(paris_ctx* c, const Coef<T>& c0) {
     // the two precisions with a diagonal excess
     const int slot = c->dirichlet ? (sizeof(T) == 8 ? 4 : 3) : (sizeof(T) == 8 ? 1 : ((c->rho0 && c->half_rho) ? 2 : 0));
     if (nl < 3 || !c->cap_stream) return false;
+    // the scale of level 1's FP16 coefficients follows the densities and is an
+    // argument of the captured kernels: other densities, another graph
+    if (slot == 2 && c->cg_exec[2] && c->cg_scale16 != c->lv[1].scale16) {
+        cudaStreamSynchronize(c->st);  // a V-cycle queued behind the last norms may still run
+        cudaGraphExecDestroy(c->cg_exec[2]);
+        c->cg_exec[2] = nullptr;
+    }
     if (!c->cg_exec[slot]) {
         cudaStream_t user = c->st;
         c->st = c->cap_stream;
@@ -764,6 +772,7 @@ bool coarse_graph_launch(paris_ctx* c, const Coef<T>& c0) {
             return false;
         }
         c->cg_kernels[slot] = (int)(launch_count() - before);
+        if (slot == 2) c->cg_scale16 = c->lv[1].scale16;
         count_launch(-c->cg_kernels[slot]);  // counted when replayed instead
     }
     if (cudaGraphLaunch(c->cg_exec[slot], c->st) != cudaSuccess) return false;

@@ -555,3 +555,28 @@ def test_long_rows_of_face_arrays_match_oracle(paris, grid):
     umax = max(np.abs(x).max() for x in (pr.u, pr.v, pr.w))
     for a in range(3):
         assert np.abs(host(u[a]) - ref.u[a]).max() <= 1e-8 * umax
+
+
+@pytest.mark.parametrize("grid", [pi.Grid(32, 32, 32, 1 / 32, (P, P, P)), pi.Grid(64, 48, 40, 1 / 64, (P, W, P)),
+                                  pi.Grid(128, 64, 96, 1 / 128, (P, P, W))],
+                         ids=lambda g: f"{g.nx}x{g.ny}x{g.nz}")
+def test_context_reused_with_other_densities(paris, grid):
+    """A context called again with other densities (level 1's FP16 coefficients
+    get another power of two) solves as a fresh one does, bit for bit and in
+    the same iterations."""
+    pr = pi.random_problem(grid, seed=71, rho1=100.0)
+
+    def step(ctx, rho2):
+        u = [dev(x) for x in (pr.u, pr.v, pr.w)]
+        p = torch.zeros(grid.shape, dtype=torch.float64, device="cuda")
+        st = ctx.projection_step(dev(pr.C), 100.0 * rho2, rho2, pr.dt, *u, p)
+        return st, [host(p)] + [host(x) for x in u]
+
+    with ctx_for(paris, grid, precision=paris.MIXED) as kept:
+        for rho2 in (1.0, 50.0, 1e-2, 1.0):
+            st, got = step(kept, rho2)
+            with ctx_for(paris, grid, precision=paris.MIXED) as fresh:
+                want_st, want = step(fresh, rho2)
+            assert st["iters"] == want_st["iters"] and st["fell_back"] == 0, (rho2, st, want_st)
+            for a, b in zip(got, want):
+                np.testing.assert_array_equal(a, b)
