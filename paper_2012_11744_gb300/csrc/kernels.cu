@@ -353,7 +353,8 @@ __global__ void __launch_bounds__(kTX* kTY) face_coeffs_kernel(Geo g, const doub
                         u[f] = 0.0;
                         return;
                     }
-                    if (fa.moderate && same_bits(cc, cl) && moderate(kl) && moderate(kc)) {  // no jump, no capillary force
+                    // no jump, no capillary force (a product of finite values with C_R - C_L = 0)
+                    if (fa.moderate && same_bits(cc, cl) && moderate(cc) && moderate(bf) && moderate(kl) && moderate(kc)) {
                         if (ga != 0.0) u[f] = fma(fa.tau, ga, u[f]);
                         return;
                     }

@@ -202,3 +202,23 @@ def test_cells_of_one_fluid(paris, grid, g):
             np.testing.assert_array_equal(np.isfinite(host(u[a])), fin)
             scale = np.abs(want[a][fin]).max()
             np.testing.assert_allclose(host(u[a])[fin], want[a][fin], rtol=0, atol=2e-15 * scale)
+
+
+def test_nonfinite_fractions_reach_the_predictor(paris):
+    """Neighbouring cells with the same NaN or infinite C: u* is non-finite on
+    their faces, as in the oracle, so that the step's own test sees it."""
+    grid = pi.Grid(40, 18, 12, 1 / 40, (P, W, P))
+    rng = np.random.default_rng(65)
+    C = (rng.random(grid.shape) < 0.5).astype(np.float64)
+    # the last: rho exactly 0 there, beta infinite
+    for k, v in ((1, np.nan), (4, np.inf), (7, -np.inf), (9, -0.5)):
+        C[k, 4:7, 3:6] = C[k + 1, 4:7, 3:6] = v
+    kappa = rng.normal(0.0, 40.0, grid.shape)
+    un = [rng.normal(size=grid.face_shape(a)) for a in range(3)]
+    with np.errstate(all="ignore"):
+        want = F.predictor(grid, *[x.copy() for x in un], C, kappa, 0.07, (0.0, 0.0, -9.81), 3.0, 1.0, 2e-3)
+    with paris.Context(grid) as ctx:
+        u = [dev(x) for x in un]
+        ctx.predictor_forcing(dev(C), dev(kappa), 3.0, 1.0, 0.07, (0.0, 0.0, -9.81), 2e-3, *u)
+    for a in range(3):
+        np.testing.assert_array_equal(np.isfinite(host(u[a])), np.isfinite(want[a]))
