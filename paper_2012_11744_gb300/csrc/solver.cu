@@ -1960,16 +1960,27 @@ paris_status paris_viscous_solve_mg(paris_ctx* c, int comp, const double* nu, do
     bool converged = false, nonfinite = false;
     double prev_rr = INFINITY;
     for (;;) {
-        // the scale from the residual before (|b| at first), as in the Poisson solve
-        finalize(c->partials, 0, 1, 0, c->scal, FIN_SCALE, 0.0, c->st);
-        launch_hmg_residual64(g, un, c->hmg.sig64, us, c->scal, r32, c->partials, c->st, rnorms);
-        CK(cudaGetLastError());
-        s = read_scal(c);
+        // the scale from the residual before (|b| at first)
+        auto residual = [&]() {
+            finalize(c->partials, 0, 1, 0, c->scal, FIN_SCALE, 0.0, c->st);
+            launch_hmg_residual64(g, un, c->hmg.sig64, us, c->scal, r32, c->partials, c->st, rnorms);
+            CK(cudaGetLastError());
+            return read_scal(c);
+        };
+        s = residual();
         if (s != PARIS_OK) return s;
         const Scal& h = *c->scal_h;
         if (h.nonfinite > 0) { nonfinite = true; break; }
         if (h.bnorm2 == 0.0 || met(h)) { converged = true; break; }
         if (iters >= max_iter) break;
+        // r32 far from O(1), whose squares over- or underflow in FP32 (the first residual is
+        // up to 12 tau nu/h^2 times |b|): once more, scaled by its own maximum.  Inside the
+        // window the squares of 2^31 unknowns sum to at most 2^71, the largest is at least 2^-80
+        const double top = h.rinf * h.scale;
+        if (!(top <= 0x1p20 && top >= 0x1p-40)) {
+            s = residual();
+            if (s != PARIS_OK) return s;
+        }
         if (h.rr > 0.25 * prev_rr) { if (++stalls >= 2) break; } else stalls = 0;
         prev_rr = h.rr;
         ++outer;

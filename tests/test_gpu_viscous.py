@@ -16,6 +16,7 @@ import os
 
 import numpy as np
 import pytest
+import scipy.sparse.linalg as spla
 
 import paris_inputs as pi
 from oracle import viscous as V
@@ -264,3 +265,25 @@ def test_viscous_fullsize_sampled(paris, multigrid):
             bound = tau * nu.max() * (1e-10 + rec["rel_res_linf"]) * binf + 1e-14 * rec["x_max_abs"]
             err = np.abs(x[rec["unknowns"]] - np.asarray(rec["x"])).max()
             assert err <= bound, (c, err, bound)
+
+
+@pytest.mark.parametrize("scale", [1e4, 1e30, 1e42, 1e90])
+@pytest.mark.parametrize("comp", [0, 2])
+def test_viscous_multigrid_long_time_step(paris, comp, scale):
+    """max tau nu / h^2 far above 1: the first residual (from u* = u^n) is that
+    many times the right-hand side, beyond FP32's range in its units."""
+    grid = pi.Grid(24, 20, 16, 1 / 24, (P, W, W))
+    rng = np.random.default_rng(77)
+    shape = V.unknown_shape(grid, comp)
+    nu = 10.0 ** rng.uniform(-2, 0, shape)
+    un = rng.standard_normal(shape)
+    tau = scale * grid.h ** 2 / nu.max()
+    A = V.spd_operator(grid, comp, nu, tau)
+    b = (un / (tau * nu)).ravel()
+    want = spla.spsolve(A.tocsc(), b).reshape(shape)
+    with paris.Context(grid) as ctx:
+        us, st = ctx.viscous_solve(comp, dev(V.embed(grid, comp, nu)), tau, dev(V.embed(grid, comp, un)), tol=1e-10,
+                                   multigrid=True, check=False)
+    x = V.interior(grid, comp, host(us))
+    assert st["converged"] == 1, st
+    assert np.abs(x - want).max() <= 1e-8 * np.abs(want).max()
