@@ -531,8 +531,9 @@ paris_status paris_max_divergence(paris_ctx* ctx, const double* u, const double*
 /* Self-check of the arithmetic the kernels build from integer operations, on
  * n device values v (FP64), against the GPU's own conversion and division
  * instructions: for each value the FP64->FP32 conversion of v * 2^shift
- * (round to nearest even; results below the FP32 normal range are flushed to
- * zero and not counted), the FP32->FP64 conversion back with 2^-shift, and
+ * (round to nearest even; values below the FP32 normal range are flushed to
+ * zero and not counted), the FP32->FP64 conversion back with 2^-shift, the
+ * conversions of v that keep FP32 subnormals (those of the coefficients), and
  * for 0 < v in [2^-123, 2^117) the FP64 reciprocal formed by Newton-Raphson
  * (Eq. muH's 1/rho_f), which must be within one ulp of 1.0/v.  *mismatches
  * (host) receives the number of disagreements.  stream: a cudaStream_t (may

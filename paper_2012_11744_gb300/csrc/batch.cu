@@ -198,7 +198,7 @@ __device__ __noinline__ void setup_coefficients(const BInst& I, int rank, int nc
         auto put = [&](int a, int64_t f, bool wall, int64_t left) {
             const double bt = wall ? 0.0 : recip64(rho(C[left]) + rc);
             b64[a][f] = bt;
-            b32[a][f] = d2f_scaled(bt * ih2, 0);
+            b32[a][f] = to_f32(bt * ih2);
         };
         put(0, g.fx(i, j, k), ax.wm, g.cidx(ax.m, j, k));
         put(1, g.fy(i, j, k), ay.wm, g.cidx(i, ay.m, k));
@@ -958,7 +958,7 @@ __device__ __noinline__ void accumulate(const BInst& I, int rank, int ncta, doub
     const int64_t n = I.g0.ncell();
     const float* e = I.e;
     double* p = I.p;
-    GLOOP(c, n) p[c] = fma(f2d_scaled(e[c], 0), inv, p[c]);
+    GLOOP(c, n) p[c] = fma(to_f64(e[c]), inv, p[c]);
 }
 
 __device__ bool solve(Grp& cx, const BParams& P, double bnorm2, double binf, int& iters, int& outer,

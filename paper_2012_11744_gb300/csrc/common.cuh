@@ -227,9 +227,10 @@ __device__ inline double key_value(unsigned long long k) { return __longlong_as_
 // with integer operations on the IEEE-754 fields: the hardware conversions
 // run on the FP64 pipe at about a fifth of its FMA rate on this GPU.
 //
-// float(v * 2^s): round to nearest, ties to even, for results in the FP32
-// normal range; smaller results flush to a signed zero, larger ones give a
-// signed infinity; infinities stay infinite and NaN stays NaN.
+// float(v * 2^s): round to nearest, ties to even, for v * 2^s in the FP32
+// normal range; smaller values flush to a signed zero (the last half ulp below
+// 2^-126 too), larger ones give a signed infinity; infinities stay infinite and
+// NaN stays NaN.
 __device__ inline float d2f_scaled(double v, int s) {
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
     const unsigned sign = hi & 0x80000000u;
@@ -259,6 +260,32 @@ __device__ inline double f2d_scaled(float v, int s) {
     if (e == 0 || de <= 0) return __hiloint2double((int)sign, 0);
     if (de >= 0x7ff) return __hiloint2double((int)(sign | 0x7ff00000u), 0);
     return __hiloint2double((int)(sign | ((unsigned)de << 20) | (frac >> 3)), (int)(frac << 29));
+}
+
+// The same conversions with FP32 subnormals kept, as the hardware's, for values
+// that no scaling brings to O(1): coefficients, and corrections without a power
+// of two of their own.  A heavy fluid's coefficient may be subnormal beside a
+// light fluid's normal one, and flushing it would cut its cells off (a 32^3 solve
+// with single heavy cells at 5e-39 ended non-finite).  In integers throughout: a
+// hardware conversion for the rare values alone is issued for all (the FP32
+// copies at 128^3: 24.9 us flushing, 29.5 so, 25.2 as below).
+__device__ __forceinline__ float to_f32(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), e = (hi >> 20) & 0x7ffu;
+    if (e - 1u >= 896u) return d2f_scaled(v, 0);
+    if (e < 873u) return __int_as_float((int)(hi & 0x80000000u));
+    const unsigned long long m = ((unsigned long long)__double_as_longlong(v) & 0xfffffffffffffULL) | 0x10000000000000ULL;
+    const int s = 926 - (int)e;  // 30 .. 53 bits below a unit of 2^-149
+    unsigned n = (unsigned)(m >> s);
+    const unsigned long long rem = m & ((1ULL << s) - 1), half = 1ULL << (s - 1);
+    if (rem > half || (rem == half && (n & 1u))) ++n;
+    return __int_as_float((int)(hi & 0x80000000u | n));
+}
+__device__ __forceinline__ double to_f64(float v) {
+    const unsigned b = (unsigned)__float_as_int(v), f = b & 0x7fffffffu;
+    if (f - 1u >= 0x7fffffu) return f2d_scaled(v, 0);
+    const int z = __clz((int)f) - 8;  // leading zeros of the fraction's 24 bits
+    const unsigned n = f << z, de = 897u - (unsigned)z;  // 1.xxx * 2^(-126 - z)
+    return __hiloint2double((int)((b & 0x80000000u) | (de << 20) | ((n & 0x7fffffu) >> 3)), (int)(n << 29));
 }
 
 // 1/s for s > 0 without an FP64 division and without FP64<->FP32

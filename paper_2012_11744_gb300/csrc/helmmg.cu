@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(kTX* kTY) hmg_setup_kernel(HelmGeo g, const do
             const double nv = nu[f], v = un[f];
             const double s = recip64(tau * nv);
             sig64[p] = s;
-            sig32[p] = d2f_scaled(s, 0);
+            sig32[p] = to_f32(s);
             us[f] = v;
             const double b = s * v;
             l2 = fma(b, b, l2);
@@ -671,12 +671,12 @@ __global__ void __launch_bounds__(kTX* kTY) hmg_accumulate_kernel(HelmGeo g, con
     pdl_wait();
     const int i = blockIdx.x * kTX + threadIdx.x, j = blockIdx.y * kTY + threadIdx.y;
     if (i >= g.m[0] || j >= g.m[1]) return;
-    const int se = -(int)s->scale_exp;
+    const double inv = s->inv_scale;
     const int k0 = blockIdx.z * kZ, k1 = min(k0 + kZ, g.m[2]);
     for (int k = k0; k < k1; ++k) {
         const int64_t p = ((int64_t)k * g.m[1] + j) * g.m[0] + i;
         const int64_t f = g.off + i + (int64_t)g.e[0] * (j + (int64_t)g.e[1] * k);
-        us[f] += f2d_scaled(e[p], se);
+        us[f] = fma(to_f64(e[p]), inv, us[f]);
     }
 }
 

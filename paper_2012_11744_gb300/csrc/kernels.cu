@@ -712,7 +712,7 @@ __global__ void convert_kernel(const __grid_constant__ ConvertArgs a, double sca
     const double* __restrict__ b = a.in[blockIdx.y];
     float* __restrict__ out = a.out[blockIdx.y];
     const int64_t n = a.n[blockIdx.y];
-    PARIS_EW_FOR(c, n) out[c] = d2f_scaled(b[c] * scale, 0);
+    PARIS_EW_FOR(c, n) out[c] = to_f32(b[c] * scale);
 }
 
 void launch_convert_beta(const Geo& g, const double* b64[3], double scale, float* out[3], cudaStream_t st) {
@@ -772,9 +772,9 @@ struct CoarseArgs {
     T* sig;                    // or null
 };
 
-__device__ __forceinline__ double widen(float v) { return f2d_scaled(v, 0); }
+__device__ __forceinline__ double widen(float v) { return to_f64(v); }
 __device__ __forceinline__ double widen(double v) { return v; }
-__device__ __forceinline__ void narrow(double v, float& out) { out = d2f_scaled(v, 0); }
+__device__ __forceinline__ void narrow(double v, float& out) { out = to_f32(v); }
 __device__ __forceinline__ void narrow(double v, double& out) { out = v; }
 
 template <typename T, int AXIS>
@@ -1983,10 +1983,15 @@ __global__ void check_arithmetic_kernel(const double* __restrict__ v, int64_t n,
         // FP64 -> FP32 with the scaling 2^shift (the product by p2 = 2^shift is exact)
         const float hw = __double2float_rn(x * p2);
         const float sw = d2f_scaled(x, shift);
-        const bool hw_sub = hw != 0.0f && fabsf(hw) < 1.17549435e-38f;  // flushed by design
+        const bool hw_sub = hw != 0.0f && fabs(x * p2) < 0x1p-126;  // flushed by design
         if (isnan(hw)) cnt += isnan(sw) ? 0 : 1;
         else if (hw_sub) cnt += (sw == 0.0f) ? 0 : 1;
         else cnt += (__float_as_int(hw) == __float_as_int(sw)) ? 0 : 1;
+        // the conversions that keep subnormals
+        const float hw1 = __double2float_rn(x), sw1 = to_f32(x);
+        if (isnan(hw1)) cnt += isnan(sw1) ? 0 : 1;
+        else cnt += (__float_as_int(hw1) == __float_as_int(sw1)) ? 0 : 1;
+        if (!isnan(hw1)) cnt += (__double_as_longlong((double)hw1) == __double_as_longlong(to_f64(hw1))) ? 0 : 1;
         // FP32 -> FP64 with 2^-shift (exact in both)
         if (!isnan(hw) && !hw_sub) {
             const double hw2 = (double)hw / p2;

@@ -580,3 +580,39 @@ def test_context_reused_with_other_densities(paris, grid):
             assert st["iters"] == want_st["iters"] and st["fell_back"] == 0, (rho2, st, want_st)
             for a, b in zip(got, want):
                 np.testing.assert_array_equal(a, b)
+
+
+def test_subnormal_coefficients(paris):
+    """Coefficients that are FP32 subnormals around single heavy cells, normal
+    ones elsewhere: the mixed form keeps them (range of the correction below
+    1/(6 * 5e-39) = 3.3e37 a unit of residual) and agrees with the FP64 form."""
+    grid = pi.Grid(32, 32, 32, 1.0, (P, P, P))
+    rng = np.random.default_rng(90)
+    heavy = np.zeros(grid.shape, bool)
+    heavy[4::8, 4::8, 4::8] = True
+    b = []
+    for a in range(3):
+        f = heavy | np.roll(heavy, 1, 2 - a)
+        b.append(np.where(f, 5e-39, 2e-36))
+    rhs = rng.standard_normal(grid.shape)
+    rhs -= rhs.mean()
+    out = {}
+    for prec in ("FP64", "MIXED"):
+        with ctx_for(paris, grid, precision=getattr(paris, prec)) as ctx:
+            p = torch.zeros(grid.shape, dtype=torch.float64, device="cuda")
+            st = ctx.poisson_solve(*[dev(x) for x in b], dev(rhs), p, check=False)
+            out[prec] = host(p), st
+    assert out["MIXED"][1]["converged"] == 1 and out["MIXED"][1]["fell_back"] == 0
+    assert np.abs(out["MIXED"][0] - out["FP64"][0]).max() <= 1e-8 * np.abs(out["FP64"][0]).max()
+
+
+def test_conversions_of_subnormals(paris):
+    """The integer conversions that keep FP32 subnormals: every power of two
+    from 2^-160 to 2^-120 with the neighbours of 1 and of the halfway points
+    below it, and random fractions, bit for bit the hardware's."""
+    e = 2.0 ** np.arange(-160, -119)
+    ulp = 2.0 ** -52
+    near = np.concatenate([[1.0, 1.0 + ulp, 2.0 - ulp, 1.5, 1.5 - ulp, 1.5 + ulp], 1.0 + 0.5 ** np.arange(1, 53),
+                           2.0 - 0.5 ** np.arange(1, 53), 1.0 + np.random.default_rng(5).random(4096)])
+    x = np.outer(e, near).ravel()
+    assert paris.check_arithmetic(dev(np.concatenate([x, -x]))) == 0
