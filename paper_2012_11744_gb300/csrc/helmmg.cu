@@ -813,11 +813,9 @@ static void launch_tail(const HelmPlan& P, const HelmWork& W, int l0, const floa
         T.sig = W.sig[l];
         cells += 3 * hcount(P.lv[l]);
     }
-    // at most 4096 (1 + 3 (1 + 1/8 + ...)) floats: beyond the default 48 KB, opted in once
-    constexpr int kTailSmem = 4 * 4096 * 5;
-    static const cudaError_t opted =
-        cudaFuncSetAttribute(hmg_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmem);
-    (void)opted;  // a failure shows at the launch
+    // at most 4096 (1 + 3 (1 + 1/8 + ...)) floats
+    static SmemOptIn opted;
+    allow_smem(opted, (const void*)hmg_tail_kernel, 4 * 4096 * 5);  // a failure shows at the launch
     launch_pdl(hmg_tail_kernel, 1, kTailThreads, sizeof(float) * (size_t)cells, st, a);
     count_launch();
 }

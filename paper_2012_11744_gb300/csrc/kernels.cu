@@ -124,21 +124,11 @@ inline bool fits_i32(const Geo& g) {
 }
 
 int device_sms() {
-    constexpr int kMaxDev = 64;
-    static std::atomic<int> cache[kMaxDev];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
-        cudaGetLastError();
-        return 1;
-    }
-    int n = cache[dev].load(std::memory_order_relaxed);
-    if (n > 0) return n;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) {
-        cudaGetLastError();
-        return 1;
-    }
-    cache[dev].store(n, std::memory_order_relaxed);
-    return n;
+    static DeviceValue sms;
+    return device_value(sms, [](int dev) {
+        int n = 0;
+        return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? n : 0;
+    });
 }
 
 int elementwise_blocks(int64_t n) {
@@ -1026,12 +1016,8 @@ template <typename T>
 void launch_coarse_inverse(const Geo& g, const Coef<T>& cf, double* inv, cudaStream_t st) {
     const int n = (int)g.ncell();
     const size_t bytes = sizeof(double) * ((size_t)n * n + n);
-    static bool opted = false;  // one opt-in per instantiation for more than 48 KB
-    if (!opted) {
-        cudaFuncSetAttribute(coarse_inverse_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(double) * (128 * 128 + 128)));
-        opted = true;
-    }
+    static SmemOptIn opted;
+    allow_smem(opted, (const void*)coarse_inverse_kernel<T>, sizeof(double) * (128 * 128 + 128));  // a failure shows at the launch
     // a small matrix is a chain of barriers: fewer warps, cheaper barriers (n = 8: 14.5 -> 12.3 us)
     launch_pdl(coarse_inverse_kernel<T>, dim3(1), dim3(32, n <= 16 ? 4 : 32), bytes, st, g, cf, inv);
     count_launch();

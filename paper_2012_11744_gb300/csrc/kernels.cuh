@@ -4,6 +4,7 @@
 #include <utility>
 
 #include "common.cuh"
+#include "per_device.cuh"
 
 namespace paris {
 

@@ -167,36 +167,14 @@ __device__ __forceinline__ void plane_barrier() {
 // minimises (full waves of resident blocks) x (planes per segment + 2, the
 // planes a segment loads ahead and below), so the last wave is not mostly
 // empty and short segments do not repeat too many loads.
-int segment_planes(const Geo& g, int nplanes, const void* kernel) {
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
-            cudaGetLastError();
-            sms = 1;
-        }
-    }
-    // resident blocks per SM of each kernel (asked once per kernel)
-    static const void* keys[8] = {};
-    static int vals[8] = {};
-    int per_sm = 0;
-    for (int e = 0; e < 8 && keys[e]; ++e)
-        if (keys[e] == kernel) per_sm = vals[e];
-    if (per_sm == 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBX * kVY, 0) != cudaSuccess ||
-            per_sm < 1) {
-            cudaGetLastError();
-            per_sm = 1;
-        }
-        for (int e = 0; e < 8; ++e)
-            if (!keys[e]) {
-                keys[e] = kernel;
-                vals[e] = per_sm;
-                break;
-            }
-    }
-    const int64_t resident = (int64_t)sms * per_sm;
+template <auto KERNEL>
+int segment_planes(const Geo& g, int nplanes) {
+    static DeviceValue blocks;  // resident blocks per SM
+    const int per_sm = device_value(blocks, [](int) {
+        int n = 0;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, KERNEL, kBX * kVY, 0) == cudaSuccess ? n : 0;
+    });
+    const int64_t resident = (int64_t)device_sms() * per_sm;
     const int64_t plane_blocks = (int64_t)pair_blocks_x(g) * ((g.ny + kVY - 1) / kVY);
     int best = 2;
     double best_cost = 1e300;
@@ -838,11 +816,11 @@ void launch_rbgs_rho(const Geo& g, const float* rh, double h, const float* f, fl
         return;
     }
     if (zero_init) {
-        const int seg = segment_planes(g, k1 - k0, (const void*)rbgs_rho_kernel<true>);
+        const int seg = segment_planes<rbgs_rho_kernel<true>>(g, k1 - k0);
         dim3 gr(pair_blocks_x(g), (g.ny + kVY - 1) / kVY, (k1 - k0 + seg - 1) / seg);
         rbgs_rho_kernel<true><<<gr, dim3(kBX, kVY), 0, st>>>(g, rh, h2, f, x, color, (float)omega, k0, k1, seg);
     } else {
-        const int seg = segment_planes(g, k1 - k0, (const void*)rbgs_rho_kernel<false>);
+        const int seg = segment_planes<rbgs_rho_kernel<false>>(g, k1 - k0);
         dim3 gr(pair_blocks_x(g), (g.ny + kVY - 1) / kVY, (k1 - k0 + seg - 1) / seg);
         rbgs_rho_kernel<false><<<gr, dim3(kBX, kVY), 0, st>>>(g, rh, h2, f, x, color, (float)omega, k0, k1, seg);
     }
@@ -1429,7 +1407,7 @@ int64_t launch_matvec_rho(const Geo& g, const float* rh, double h, const float* 
         count_launch();
         return (int64_t)gr.x * gr.y * gr.z;
     }
-    const int seg = segment_planes(g, g.nz, (const void*)op_rho_kernel<false>);
+    const int seg = segment_planes<op_rho_kernel<false>>(g, g.nz);
     dim3 gr(pair_blocks_x(g), (g.ny + kVY - 1) / kVY, (g.nz + seg - 1) / seg);
     op_rho_kernel<false><<<gr, dim3(kBX, kVY), 0, st>>>(g, rh, (float)(1.0 / (h * h)), d, nullptr, q, g,
                                                         partials, seg, fin);
@@ -1455,7 +1433,7 @@ void launch_restrict_rho(const Geo& g, const float* rh, double h, const float* f
         count_launch();
         return;
     }
-    const int seg = segment_planes(g, g.nz, (const void*)op_rho_kernel<true>);
+    const int seg = segment_planes<op_rho_kernel<true>>(g, g.nz);
     dim3 gr(pair_blocks_x(g), (g.ny + kVY - 1) / kVY, (g.nz + seg - 1) / seg);
     op_rho_kernel<true><<<gr, dim3(kBX, kVY), 0, st>>>(g, rh, (float)(1.0 / (h * h)), x, f, fc, cg,
                                                        nullptr, seg, no_fin());

@@ -43,6 +43,7 @@ namespace {
 #endif
 constexpr int kStageRows = PARIS_STAGE_ROWS;    // R: rows per tile, one warp each
 constexpr int kStageSlots = PARIS_STAGE_SLOTS;  // S: planes held in the ring (S - 2 in flight)
+constexpr size_t kStageSmemMax = 200 * 1024;  // the ring's shared memory
 constexpr long long kWaitCycles = 2000000000LL;  // about one second at 2 GHz
 
 __device__ __forceinline__ float rcp_approx(float v) {
@@ -353,14 +354,11 @@ cudaError_t launch_stage(StageArgs a, cudaStream_t st) {
     const SlotLayout L = slot_layout(a.g.nx, R);
     const size_t smem = (size_t)kStageSlots * L.floats * sizeof(float);
     auto kern = rbgs_rho_stage_kernel<R, ZERO, XZ>;
-    static size_t set_for = 0;
-    if (smem > set_for) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        set_for = smem;
-    }
+    static SmemOptIn opted;
+    cudaError_t e = allow_smem(opted, (const void*)kern, kStageSmemMax);
+    if (e != cudaSuccess) return e;
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, R * 32, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, R * 32, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const int ntiles = a.g.ny / R, npl = a.k1 - a.k0;
@@ -380,7 +378,7 @@ cudaError_t launch_stage(StageArgs a, cudaStream_t st) {
 bool rho0_stage_fits(const Geo& g) {
     if (g.nx % 8 != 0 || g.ny % kStageRows != 0 || g.nz < 2) return false;
     const SlotLayout L = slot_layout(g.nx, kStageRows);
-    return (size_t)kStageSlots * L.floats * sizeof(float) <= 200 * 1024;
+    return (size_t)kStageSlots * L.floats * sizeof(float) <= kStageSmemMax;
 }
 
 cudaError_t launch_rbgs_rho_stage(const Geo& g, const float* rh, double h, const float* f, float* x, int color,

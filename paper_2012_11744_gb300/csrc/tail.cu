@@ -608,16 +608,12 @@ void launch_tail_vcycle(const TailLevel<T>* levels, int n, const double* Minv, d
         count_launch();
         return;
     }
-    // stage in shared memory when it fits (opt-in beyond 48 KB, once per type)
+    // stage in shared memory when it fits
     constexpr size_t kSmemMax = 200 * 1024;
     const size_t smem = tail_smem_bytes(levels, n);
     if (smem <= kSmemMax) {
-        static bool opted = false;
-        if (!opted) {
-            cudaFuncSetAttribute(tail_vcycle_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kSmemMax);
-            opted = true;
-        }
+        static SmemOptIn opted;
+        allow_smem(opted, (const void*)tail_vcycle_kernel<T, true>, kSmemMax);  // a failure shows at the launch
         launch_pdl(tail_vcycle_kernel<T, true>, 1, kTailThreads, smem, st, a);
     } else {
         launch_pdl(tail_vcycle_kernel<T, false>, 1, kTailThreads, 0, st, a);
