@@ -248,7 +248,8 @@ __global__ void __launch_bounds__(kTX* kTY) hmg_residual4_kernel(HLev L, const f
 
 // q = A d (quads) and the partials of d . q.  A block takes zper planes of its
 // 8 rows: with one, the 8192 blocks' hand-over of their partial sums took as
-// long as the product (76 us at 256^3; 40 with 17).
+// long as the product (76 us at 256^3; 41 with 17).  A plane's four terms are
+// added in FP32, the planes' sums with their errors (CarriedSum).
 __global__ void __launch_bounds__(kTX* kTY, 6) hmg_matvec4_kernel(HLev L, const float* __restrict__ sig,
                                                                  const float* __restrict__ d, float* __restrict__ q,
                                                                  double* partials, int zper, FinSpec fin) {
@@ -261,18 +262,20 @@ __global__ void __launch_bounds__(kTX* kTY, 6) hmg_matvec4_kernel(HLev L, const 
     const bool act = qq < nq && j < L.m[1];
     const int i0 = 4 * (qq < nq ? qq : nq - 1);
     const int k0 = blockIdx.z * zper, k1 = min(k0 + zper, L.m[2]);
-    float dq = 0.f;
+    CarriedSum dq;
     for (int k = k0; k < k1; ++k) {
         float X[4], AX[4];
         hop4(L, d, sig, jc, k, i0, lane, X, AX);
         if (act) {
             const int c0 = (k * L.m[1] + jc) * L.m[0] + i0;
             *reinterpret_cast<float4*>(q + c0) = make_float4(AX[0], AX[1], AX[2], AX[3]);
+            float t = 0.f;
 #pragma unroll
-            for (int li = 0; li < 4; ++li) dq = fmaf(X[li], AX[li], dq);
+            for (int li = 0; li < 4; ++li) t = fmaf(X[li], AX[li], t);
+            dq.add(t);
         }
     }
-    double accd[1] = {(double)dq};
+    double accd[1] = {dq.value()};
     const int op[1] = {0};
     block_reduce_store<1>(accd, op, partials, ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x,
                           tid);
@@ -644,7 +647,7 @@ __global__ void __launch_bounds__(kTX* kTY) hmg_matvec32_kernel(HLev L, const fl
     pdl_wait();
     const int i = blockIdx.x * kTX + threadIdx.x, j = blockIdx.y * kTY + threadIdx.y;
     const int tid = threadIdx.y * kTX + threadIdx.x;
-    float dq = 0.f;
+    CarriedSum dq;
     if (i < L.m[0] && j < L.m[1]) {
         const int k0 = blockIdx.z * zper, k1 = min(k0 + zper, L.m[2]);
 #pragma unroll 4
@@ -655,10 +658,10 @@ __global__ void __launch_bounds__(kTX* kTY) hmg_matvec32_kernel(HLev L, const fl
             const float dc = d[c];
             const float qc = fmaf(dg, L.ih2, sig[c]) * dc - acc * L.ih2;
             q[c] = qc;
-            dq = fmaf(dc, qc, dq);
+            dq.add_product(dc, qc);
         }
     }
-    double accd[1] = {(double)dq};
+    double accd[1] = {dq.value()};
     const int op[1] = {0};
     block_reduce_store<1>(accd, op, partials, ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x,
                           tid);

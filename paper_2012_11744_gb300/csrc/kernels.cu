@@ -145,11 +145,11 @@ int elementwise_blocks(int64_t n) {
     return (int)b;
 }
 
-int march_planes(int64_t tiles, int nz, int per_sm) {
+int march_planes(int64_t tiles, int nz, int per_sm, int most) {
     const int64_t cap = (int64_t)device_sms() * per_sm;
     int best = nz;
     int64_t least = INT64_MAX;
-    for (int p = nz < 64 ? nz : 64; p >= (nz < kMinMarch ? nz : kMinMarch); --p) {
+    for (int p = nz < most ? nz : most; p >= (nz < kMinMarch ? nz : kMinMarch); --p) {
         if ((nz + p - 1) / p > 65535) break;  // gridDim.z
         const int64_t blocks = tiles * ((nz + p - 1) / p);
         const int64_t cost = ((blocks + cap - 1) / cap) * (p + 2);
@@ -1583,8 +1583,8 @@ int64_t launch_residual64(const Geo& g, const Coef<double>& cf, const double* f,
     return nblocks_of(gr);
 }
 
-// q = A d and the partial sums of d . q (accumulated per thread in T,
-// across threads and blocks in FP64).
+// q = A d and the partial sums of d . q (accumulated per thread in T, in FP32
+// with its errors, across threads and blocks in FP64).
 template <typename T, bool I32, bool SIG = false>
 __global__ void __launch_bounds__(kTX* kTY) matvec_dot_kernel(Geo g, Coef<T> cf,
                                                              const T* __restrict__ d,
@@ -1593,7 +1593,8 @@ __global__ void __launch_bounds__(kTX* kTY) matvec_dot_kernel(Geo g, Coef<T> cf,
     pdl_wait();
     const int i = blockIdx.x * kTX + threadIdx.x;
     const int j = blockIdx.y * kTY + threadIdx.y;
-    T loc = T(0);
+    CarriedSum c32;
+    double loc = 0.0;
     if (i < g.nx && j < g.ny) {
         const int k0 = blockIdx.z * zper, k1 = min(k0 + zper, g.nz);
         PARIS_ZLOOP(k0, k1, {
@@ -1611,10 +1612,11 @@ __global__ void __launch_bounds__(kTX* kTY) matvec_dot_kernel(Geo g, Coef<T> cf,
             T qc = apply_A(st, d, dc, cf.scale);
             if (SIG) qc = fma(cf.scale * cf.sig[c], dc, qc);
             q[c] = qc;
-            loc = fma(dc, qc, loc);
+            if constexpr (sizeof(T) == 4) c32.add_product(dc, qc);
+            else loc = fma(dc, qc, loc);
         })
     }
-    double acc[1] = {(double)loc};
+    double acc[1] = {sizeof(T) == 4 ? c32.value() : loc};
     const int op[1] = {0};
     block_reduce_store<1>(acc, op, partials, flat_block(), flat_tid());
     finalize_last_block(partials, (int64_t)gridDim.x * gridDim.y * gridDim.z, fin, flat_tid());
@@ -1624,9 +1626,9 @@ __global__ void __launch_bounds__(kTX* kTY) matvec_dot_kernel(Geo g, Coef<T> cf,
 // planes: every array read as 16-byte vectors, d above and the z-faces carried
 // to the next plane, the x-neighbours from the adjacent lanes.  The one-cell
 // kernel issues fifteen 4-byte loads a cell and is bound by them: 128^3 20.0 ->
-// 15.6 us.  Same arithmetic per cell; a partial sum per cell of the four, added
-// in FP64.  Needs what rbgs4_kernel needs (nx % 4 == 0, at least a warp's row,
-// no walls along x, 32-bit offsets, 16-byte alignment).
+// 15.2 us.  Same arithmetic per cell; a plane's four terms added in FP32, the
+// planes' sums with their errors.  Needs what rbgs4_kernel needs (nx % 4 == 0,
+// at least a warp's row, no walls along x, 32-bit offsets, 16-byte alignment).
 template <bool SIG>
 __global__ void __launch_bounds__(kTX* kTY) matvec_dot4_kernel(Geo g, Coef<float> cf, const float* __restrict__ d,
                                                               float* __restrict__ q, double* partials, int zper,
@@ -1652,7 +1654,7 @@ __global__ void __launch_bounds__(kTX* kTY) matvec_dot4_kernel(Geo g, Coef<float
     ld(d + k0 * pl + row, x);
     ld(cf.bz + k0 * pl + row, bz);
     if (g.wz && k0 == 0) bz[0] = bz[1] = bz[2] = bz[3] = 0.f;
-    float loc[4] = {0.f, 0.f, 0.f, 0.f};
+    CarriedSum loc;
     for (int k = k0; k < k1; ++k) {
         const int c = k * pl + row;
         float zp[4], ym[4], yp[4], bx[5], by[4], bp[4], bt[4], t[4];
@@ -1697,8 +1699,10 @@ __global__ void __launch_bounds__(kTX* kTY) matvec_dot4_kernel(Geo g, Coef<float
         }
         if (act) {
             *reinterpret_cast<float4*>(q + c) = make_float4(out[0], out[1], out[2], out[3]);
+            float t = 0.f;
 #pragma unroll
-            for (int m = 0; m < 4; ++m) loc[m] = fmaf(x[m], out[m], loc[m]);
+            for (int m = 0; m < 4; ++m) t = fmaf(x[m], out[m], t);
+            loc.add(t);
         }
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
@@ -1707,7 +1711,7 @@ __global__ void __launch_bounds__(kTX* kTY) matvec_dot4_kernel(Geo g, Coef<float
             bz[m] = bt[m];
         }
     }
-    double acc[1] = {((double)loc[0] + (double)loc[1]) + ((double)loc[2] + (double)loc[3])};
+    double acc[1] = {loc.value()};
     const int op[1] = {0};
     block_reduce_store<1>(acc, op, partials, flat_block(), flat_tid());
     finalize_last_block(partials, (int64_t)gridDim.x * gridDim.y * gridDim.z, fin, flat_tid());

@@ -198,8 +198,10 @@ int elementwise_blocks(int64_t n);
 // tiles a plane, per_sm blocks resident on an SM: the number that fills the
 // chip in the fewest, fullest waves (a block's start and its reduction count as
 // two planes' work).  A fixed number leaves the last wave nearly empty at some
-// sizes (128^3 doubles at 8 planes: 1.35 waves) and the chip at others.
-int march_planes(int64_t tiles, int nz, int per_sm);
+// sizes (128^3 doubles at 8 planes: 1.35 waves) and the chip at others.  most: for
+// kernels whose threads add up in plain FP32 over their planes, so that the
+// rounding of those sums does not grow with the grid.
+int march_planes(int64_t tiles, int nz, int per_sm, int most = 64);
 constexpr int kMinMarch = 2;  // the fewest it returns (one on a single plane)
 // Most blocks any reducing kernel launches on a grid of this size (the
 // number of partial-sum slots a caller must provide, per value).

@@ -170,7 +170,8 @@ void launch_refine_rho(const Geo& g, const float2* rh2, double h, const float* e
     const float hi = (float)ih2d;
     const float lo = (float)(ih2d - (double)hi);
     const int tx = (g.nx + kTX - 1) / kTX, ty = (g.ny + kTY - 1) / kTY;
-    const int zper = march_planes((int64_t)tx * ty, g.nz, kPerSM);
+    // 16: 347 us a launch at 256^3, with up to 64 planes 348
+    const int zper = march_planes((int64_t)tx * ty, g.nz, kPerSM, 16);
     const dim3 gr(tx, ty, (g.nz + zper - 1) / zper);
     launch_pdl(refine_rho_kernel, gr, dim3(kTX, kTY), 0, st, g, rh2, hi, lo, e, r_old, r_new, x, r32, s,
         partials, FinSpec{s, 3, 2, FIN_REFINE, 0.0}, rev ? 1 : 0, emem ? 1 : 0, dpend, zper);
