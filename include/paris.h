@@ -535,9 +535,11 @@ paris_status paris_max_divergence(paris_ctx* ctx, const double* u, const double*
  * zero and not counted), the FP32->FP64 conversion back with 2^-shift, the
  * conversions of v that keep FP32 subnormals (those of the coefficients), and
  * for 0 < v in [2^-123, 2^117) the FP64 reciprocal formed by Newton-Raphson
- * (Eq. muH's 1/rho_f), which must be within one ulp of 1.0/v.  *mismatches
- * (host) receives the number of disagreements.  stream: a cudaStream_t (may
- * be NULL); the call allocates 8 bytes of device memory and synchronises it.
+ * (Eq. muH's 1/rho_f), which must be within one ulp of 1.0/v, and the correctly
+ * rounded one; and the quotients v[i]/v[n-1-i] of positive values, correctly
+ * rounded.  *mismatches (host) receives the number of disagreements.  stream:
+ * a cudaStream_t (may be NULL); the call allocates 8 bytes of device memory
+ * and synchronises it.
  * Errors: INVALID_ARG (n < 0, |shift| > 60, null pointers), CUDA. */
 paris_status paris_check_arithmetic(const double* v, int64_t n, int shift, int64_t* mismatches,
                                     void* stream);

@@ -196,7 +196,7 @@ __device__ __noinline__ void setup_coefficients(const BInst& I, int rank, int nc
         const double rc = rho(C[c]);
         AxisNb ax = axis_nb(i, g.nx, g.wx), ay = axis_nb(j, g.ny, g.wy), az = axis_nb(k, g.nz, g.wz);
         auto put = [&](int a, int64_t f, bool wall, int64_t left) {
-            const double bt = wall ? 0.0 : recip64(rho(C[left]) + rc);
+            const double bt = wall ? 0.0 : recip64_rn(rho(C[left]) + rc);
             b64[a][f] = bt;
             b32[a][f] = to_f32(bt * ih2);
         };

@@ -299,9 +299,12 @@ __device__ __forceinline__ double to_f64(float v) {
 // result is within one ulp of the correctly rounded 1/s.  Values of s
 // outside the exponent window [2^-123, 2^117) (or s <= 0, NaN) take the
 // FP64 division.
-__device__ inline double recip64(double s) {
+__device__ __forceinline__ bool recip_window(double s) {
     const int hi = __double2hiint(s);
-    if (hi < (900 << 20) || hi >= (1140 << 20)) return 1.0 / s;
+    return !(hi < (900 << 20) || hi >= (1140 << 20));
+}
+__device__ __forceinline__ double recip_newton(double s) {  // s in the window
+    const int hi = __double2hiint(s);
     const float sf = __int_as_float((hi - (896 << 20)) << 3);
     float yf;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(sf));
@@ -309,6 +312,35 @@ __device__ inline double recip64(double s) {
     const double y0 = __hiloint2double((int)((yb >> 3) + (896u << 20)), (int)(yb << 29));
     const double e = fma(-s, y0, 1.0);
     return fma(y0, fma(e, e, e), y0);
+}
+__device__ inline double recip64(double s) {
+    if (!recip_window(s)) return 1.0 / s;
+    return recip_newton(s);
+}
+
+// 1/s correctly rounded: one more step y + (1 - s y) y from a y within one ulp
+// gives that for every s whose fraction is not all ones (Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000 processor",
+// IBM J. Res. Dev. 34, 1990); those take the division.  Two more FP64
+// instructions (the viscous set-up at 256^3: 286 -> 345 us a component).
+__device__ inline double recip64_rn(double s) {
+    const bool ones = ((unsigned)__double2hiint(s) | 0xfff00000u) == 0xffffffffu && __double2loint(s) == -1;
+    if (!recip_window(s) || ones) return 1.0 / s;
+    const double y = recip_newton(s);
+    return fma(fma(-s, y, 1.0), y, y);
+}
+
+// a / b for positive a and b: q = a y with y = 1/b to one ulp and one step with
+// the exact remainder, q + (a - b q) y, which is within 1.5 ulp times y's relative
+// error of a / b before it is rounded.  So the result is the correctly rounded
+// quotient unless a / b lies within 2^-51 ulp of the middle between two doubles.
+// 6 FP64 instructions; outside the window in which no intermediate over- or
+// underflows, the division.
+__device__ __forceinline__ double div_pos(double a, double b) {
+    const unsigned ha = (unsigned)__double2hiint(a);
+    if (ha - (700u << 20) >= (600u << 20) || !recip_window(b)) return a / b;
+    const double y = recip_newton(b), q = a * y;
+    return fma(fma(-b, q, a), y, q);
 }
 
 // p / d for p < 2^31 by the multiplier m = floor(2^32 / d) + 1 of

@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(kTX* kTY) hmg_setup_kernel(HelmGeo g, const do
             const int64_t p = ((int64_t)k * g.m[1] + j) * g.m[0] + i;
             const int64_t f = g.off + i + (int64_t)g.e[0] * (j + (int64_t)g.e[1] * k);
             const double nv = nu[f], v = un[f];
-            const double s = recip64(tau * nv);
+            const double s = recip64_rn(tau * nv);
             sig64[p] = s;
             sig32[p] = to_f32(s);
             us[f] = v;

@@ -1988,11 +1988,15 @@ __global__ void check_arithmetic_kernel(const double* __restrict__ v, int64_t n,
             const double sw2 = f2d_scaled(hw, -shift);
             cnt += (__double_as_longlong(hw2) == __double_as_longlong(sw2)) ? 0 : 1;
         }
-        // reciprocal within one ulp of the correctly rounded quotient
+        // reciprocal within one ulp of the correctly rounded quotient, and correctly rounded
         if (x > 0.0 && x >= 0x1p-123 && x < 0x1p117) {
             const long long a = __double_as_longlong(recip64(x)), b = __double_as_longlong(1.0 / x);
             cnt += (a - b <= 1 && b - a <= 1) ? 0 : 1;
+            cnt += __double_as_longlong(recip64_rn(x)) == b ? 0 : 1;
         }
+        // the quotient of two values
+        const double y = v[n - 1 - i];
+        if (x > 0.0 && y > 0.0) cnt += __double_as_longlong(div_pos(x, y)) == __double_as_longlong(x / y) ? 0 : 1;
     }
     if (cnt) atomicAdd(bad, cnt);
 }

@@ -65,9 +65,9 @@ __global__ void __launch_bounds__(kTX* kTY, kPerSM) helm_init_kernel(HelmGeo g, 
             const int64_t f = g.off + i + (int64_t)g.e[0] * (j + (int64_t)g.e[1] * k);
             const double v = un[f], nv = nu[f];
             us[f] = v;
-            const double s = recip64(tau * nv);
+            const double s = recip64_rn(tau * nv);
             sig[p] = s;
-            w[p] = recip64(fma((double)(dxy + HelmColumn::count(g.kind[2], g.m[2], k)), g.ih2, s));
+            w[p] = recip64_rn(fma((double)(dxy + HelmColumn::count(g.kind[2], g.m[2], k)), g.ih2, s));
             const double b = s * v;
             l2[0] = fma(b, b, l2[0]);
             const unsigned long long kb = abs_key(b);
@@ -243,18 +243,6 @@ __global__ void helm_direction_kernel(int64_t n, const Scal* __restrict__ s, con
         const double z = w[p] * r[p];
         d[p] = first ? z : fma(beta, d[p], z);
     }
-}
-
-// a / b for positive a and b, correctly rounded: y = 1/b to one ulp (recip64),
-// q = a y, and one step with the exact remainder, q + (a - b q) y (Markstein,
-// "Computation of elementary functions on the IBM RISC System/6000", 1990).
-// 6 FP64 instructions; outside the window in which no intermediate over- or
-// underflows, the division.
-__device__ __forceinline__ double div_pos(double a, double b) {
-    const int ha = __double2hiint(a), hb = __double2hiint(b);
-    if (ha < (700 << 20) || ha >= (1300 << 20) || hb < (900 << 20) || hb >= (1140 << 20)) return a / b;
-    const double y = recip64(b), q = a * y;
-    return fma(fma(-b, q, a), y, q);
 }
 
 // nu_f = (mu_L + mu_R) / (rho_L + rho_R) on every face of the component,

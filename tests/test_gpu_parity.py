@@ -616,3 +616,24 @@ def test_conversions_of_subnormals(paris):
                            2.0 - 0.5 ** np.arange(1, 53), 1.0 + np.random.default_rng(5).random(4096)])
     x = np.outer(e, near).ravel()
     assert paris.check_arithmetic(dev(np.concatenate([x, -x]))) == 0
+
+
+def test_reciprocals_and_quotients_correctly_rounded(paris):
+    """The FP64 reciprocal and quotient without a division, bit for bit the
+    GPU's own: random fractions over the reciprocal's range of exponents, the
+    fractions next to 1 and to 2, quotients of neighbours, exact ones and powers
+    of two (the hook divides v[i] by v[n-1-i])."""
+    rng = np.random.default_rng(31)
+    n = 1 << 20
+    a, b = ((1.0 + rng.random(n)) * 2.0 ** rng.integers(-122, 116, n) for _ in range(2))
+    assert paris.check_arithmetic(dev(np.concatenate([a, b[::-1]]))) == 0
+    k = np.arange(0, 2048)
+    edge = np.concatenate([1.0 + k * 2.0**-52, 2.0 - (k + 1) * 2.0**-52, 2.0 ** rng.integers(-122, 116, 2048),
+                           1.0 + rng.random(2048)])
+    for shift in range(0, edge.size, 61):
+        q = np.roll(edge, shift)
+        assert paris.check_arithmetic(dev(np.concatenate([edge, q[::-1]]))) == 0
+    # mixtures of two fluids as the face viscosity divides them
+    c = rng.random((2, n))
+    mu, rho = 1.0e-3 * c + 1.8e-5 * (1 - c), 1000.0 * c + 1.2 * (1 - c)
+    assert paris.check_arithmetic(dev(np.concatenate([mu[0] + mu[1], (rho[0] + rho[1])[::-1]]))) == 0
