@@ -906,11 +906,6 @@ static void hmg_vcycle_core(const HelmPlan& P, const HelmWork& W, const float* f
     }
 }
 
-int64_t helm_max_blocks(const HelmGeo& g) {
-    const dim3 gr = hgrid(g.m, kZ);
-    return (int64_t)gr.x * gr.y * gr.z;
-}
-
 }  // namespace paris
 
 namespace paris {

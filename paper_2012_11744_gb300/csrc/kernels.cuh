@@ -318,7 +318,6 @@ void launch_hmg_sigma(const HelmPlan& P, float* const* sig, cudaStream_t st);
 // (|r|^2, max |r|, non-finite) of the FP64 residual
 void launch_hmg_residual64(const HelmGeo& g, const double* un, const double* sig, const double* us, const Scal* s,
                            float* r32, double* partials, cudaStream_t st, FinSpec fin);
-int64_t helm_max_blocks(const HelmGeo& g);
 // FP32 inner iteration of the mixed form: z32 = V r32 (finest-level vectors
 // given, not the work arrays); q = A d in FP32 and d . q; u* += e / scale
 void launch_hmg_vcycle32(const HelmPlan& P, const HelmWork& W, const float* r32, float* z32, int nu1, int nu2,
