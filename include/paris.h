@@ -131,7 +131,10 @@ typedef struct {
                              the levels of at most 32^3 cells above them (8192 in FP64)
                              in one launch down and one up; 0 one launch per step and
                              level.  The same arithmetic in the same order in both:
-                             identical results (1) */
+                             identical results, except where a finest level taken from
+                             rho/2 in one launch has an odd nx/2: the z-column kernels
+                             restrict over all faces there, the launch over the coarse
+                             cells' surface faces, which differ by rounding (1) */
 } paris_opts;
 
 typedef struct {

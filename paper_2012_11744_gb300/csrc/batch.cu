@@ -34,7 +34,7 @@ namespace batch {
 
 // Threads per CTA, two CTAs per SM.  The kernel waits on memory latency, so it
 // wants warps and bytes in flight per thread, and no spills: 384 threads at
-// the 85 registers that leaves run 64 instances (20 M cells) in 17.9 ms, 256 in
+// the 85 registers that leaves ran 64 instances (20 M cells) in 17.9 ms, 256 in
 // 18.6, 512 in 19.9 (spilling); at 4 to 16 instances 256 are 6 to 8 % faster.
 constexpr int kBT = 384;
 constexpr int kMaxLev = 12;  // multigrid levels per instance

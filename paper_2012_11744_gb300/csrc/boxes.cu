@@ -12,7 +12,9 @@
 // A halo cell is updated by several blocks, each time to the same value; the
 // passes are those of rbgs_kernel, the restriction that of
 // restrict_residual_kernel, in the same arithmetic and order, so the results
-// are the same bit for bit.
+// are the same bit for bit (from rho/2: those of the plane tiles, rho0.cu; where
+// nx/2 is odd the z-column kernels stand in for these, whose restriction sums
+// all faces and differs by rounding).
 //
 // What bounds it is latency: of the launch, of one access to memory, and of
 // the dependent instructions of four passes on one SM.  So a thread owns one
