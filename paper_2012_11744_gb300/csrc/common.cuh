@@ -378,20 +378,16 @@ __device__ inline double warp_max(double v) {
 
 // An FP32 sum that carries its rounding errors (Knuth's two-sum): the sums of a
 // thread that marches through planes, so that their rounding does not grow with
-// the planes a block takes.  Seven FP32 additions a term, no FP64 (the product at
-// 250 x 255 x 245: 91 us a launch, 97 with plain sums over as many planes, 113
-// with at most eight).
+// the planes a block takes: what is left is half an ulp of each term's magnitude,
+// where a chain of n fused steps has up to n times that.  Seven FP32 additions a
+// term, no FP64 (the product at 250 x 255 x 245: 91 us a launch, 97 with plain
+// sums over as many planes, 113 with at most eight).
 struct CarriedSum {
     float sum = 0.f, err = 0.f;
     __device__ __forceinline__ void add(float t) {
         const float s = __fadd_rn(sum, t), tp = __fsub_rn(s, sum);
         err = __fadd_rn(err, __fadd_rn(__fsub_rn(sum, __fsub_rn(s, tp)), __fsub_rn(t, tp)));
         sum = s;
-    }
-    __device__ __forceinline__ void add_product(float a, float b) {
-        const float t = __fmul_rn(a, b);
-        err = __fadd_rn(err, __fmaf_rn(a, b, -t));
-        add(t);
     }
     __device__ __forceinline__ double value() const { return (double)sum + (double)err; }
 };

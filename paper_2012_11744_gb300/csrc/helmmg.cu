@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(kTX* kTY, kPerSM) hmg_residual64_kernel(HelmGe
 
 // FP32 inner iteration: q = A d on the finest level (FP32 sigma) and the
 // partials of d . q
-__global__ void __launch_bounds__(kTX* kTY) hmg_matvec32_kernel(HLev L, const float* __restrict__ sig,
+__global__ void __launch_bounds__(kTX* kTY, 6) hmg_matvec32_kernel(HLev L, const float* __restrict__ sig,
                                                                const float* __restrict__ d, float* __restrict__ q,
                                                                double* partials, int zper, FinSpec fin) {
     pdl_wait();
@@ -658,7 +658,7 @@ __global__ void __launch_bounds__(kTX* kTY) hmg_matvec32_kernel(HLev L, const fl
             const float dc = d[c];
             const float qc = fmaf(dg, L.ih2, sig[c]) * dc - acc * L.ih2;
             q[c] = qc;
-            dq.add_product(dc, qc);
+            dq.add(__fmul_rn(dc, qc));
         }
     }
     double accd[1] = {dq.value()};

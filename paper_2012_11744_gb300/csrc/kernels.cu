@@ -1612,7 +1612,7 @@ __global__ void __launch_bounds__(kTX* kTY) matvec_dot_kernel(Geo g, Coef<T> cf,
             T qc = apply_A(st, d, dc, cf.scale);
             if (SIG) qc = fma(cf.scale * cf.sig[c], dc, qc);
             q[c] = qc;
-            if constexpr (sizeof(T) == 4) c32.add_product(dc, qc);
+            if constexpr (sizeof(T) == 4) c32.add(__fmul_rn((float)dc, (float)qc));
             else loc = fma(dc, qc, loc);
         })
     }
