@@ -54,6 +54,7 @@ struct BInst {
     Geo g0;
     double h, dt, rho1, rho2;
     int nlev, ncoarse, dense;
+    unsigned seams;  // bit l: level l has an odd_seam
     BLevel lv[kMaxLev];
     const double* C;
     double *u, *v, *w, *p;
@@ -81,6 +82,7 @@ struct Grp {
     int rank, ncta;
     int* err;
     int pb;
+    unsigned seams;     // bit l: level l has an odd_seam
     unsigned arrivals;  // of the whole group up to the last barrier (thread 0)
     long long spin;
 };
@@ -515,6 +517,36 @@ __device__ __noinline__ void rb_quads(int rank, int ncta, const BLevel& L, const
     }
 }
 
+// Above the colour's bit: the pass is on a level with an odd_seam, and is the
+// second of its sweep.  In the argument, since the descriptor's loads miss L1
+// after each barrier: with a test of L.t the batches of small boxes lost 3 to 5 %.
+constexpr int kSeam = 2, kSecond = 4;
+
+// The colour pass of such a level, cell by cell: the first of a sweep from x to the
+// level's second array, the second back (all cells written).  Same update as
+// pass_store.
+__device__ __noinline__ void rb_seam(int rank, int ncta, const BLevel& L, const float* f, float* xl, int color,
+                                     float omega, bool zero) {
+    const Geo g = L.g;
+    const bool back = (color & kSecond) != 0;
+    const float* x = back ? L.t : xl;
+    float* xo = back ? xl : L.t;
+    const float *bx = L.b[0], *by = L.b[1], *bz = L.b[2];
+    const unsigned mx = L.mx, my = L.my;
+    GLOOP(c, g.ncell()) {
+        PassCell p;
+        decomp(g, mx, my, c, p.i, p.j, p.k);
+        p.io = g.nx;
+        if (((p.i + p.j + p.k + color) & 1) != 0) {
+            xo[c] = zero ? 0.f : x[c];
+            continue;
+        }
+        PassLoad d;
+        pass_load(d, g, bx, by, bz, f, x, p, zero);
+        pass_store(d, g, xo, p, omega, zero);
+    }
+}
+
 // One red-black colour pass in place on level L (zero: x taken as 0 and the
 // other colour zeroed).  x_c <- x_c + omega (w (f + sum beta x_nb) - x_c).
 // A thread takes two pairs per iteration and loads both stencils before it
@@ -522,6 +554,10 @@ __device__ __noinline__ void rb_quads(int rank, int ncta, const BLevel& L, const
 // another, so the two updates are independent.
 __device__ __noinline__ void rb_pairs(int rank, int ncta, const BLevel& L, const float* f, float* x, int color,
                                       float omega, bool zero) {
+    if (color & kSeam) {
+        rb_seam(rank, ncta, L, f, x, color, omega, zero);
+        return;
+    }
     const Geo g = L.g;  // in registers: the stores below could alias the descriptor
     const float *bx = L.b[0], *by = L.b[1], *bz = L.b[2];
     const unsigned npair = (unsigned)(g.nx + 1) / 2, mp = L.mp, my = L.my;
@@ -539,33 +575,12 @@ __device__ __noinline__ void rb_pairs(int rank, int ncta, const BLevel& L, const
     }
 }
 
-// The colour pass of a level with an odd_seam, cell by cell, from x to xo (all
-// cells written).  Same update as pass_store.
-__device__ __noinline__ void rb_seam(int rank, int ncta, const BLevel& L, const float* f, const float* x, float* xo,
-                                     int color, float omega, bool zero) {
-    const Geo g = L.g;
-    const float *bx = L.b[0], *by = L.b[1], *bz = L.b[2];
-    const unsigned mx = L.mx, my = L.my;
-    GLOOP(c, g.ncell()) {
-        PassCell p;
-        decomp(g, mx, my, c, p.i, p.j, p.k);
-        p.io = g.nx;
-        if (((p.i + p.j + p.k) & 1) != color) {
-            xo[c] = zero ? 0.f : x[c];
-            continue;
-        }
-        PassLoad d;
-        pass_load(d, g, bx, by, bz, f, x, p, zero);
-        pass_store(d, g, xo, p, omega, zero);
-    }
-}
-
 // One colour pass on a level: quads where every thread of the group gets at
 // least two planes of one, pairs otherwise.
 __device__ __forceinline__ void rb_pass(int rank, int ncta, const BLevel& L, const float* f, float* x, int color,
                                         float omega, bool zero) {
     const int nx = L.g.nx, per = nx / 4 * L.g.ny * L.g.nz / (ncta * kBT);
-    if (nx % 4 == 0 && !L.g.wx && per >= 2)
+    if (nx % 4 == 0 && !L.g.wx && per >= 2 && !(color & kSeam))
         rb_quads(rank, ncta, L, f, x, color, omega, zero, per < kQuadPlanes ? per : kQuadPlanes);
     else
         rb_pairs(rank, ncta, L, f, x, color, omega, zero);
@@ -724,16 +739,13 @@ __device__ __forceinline__ bool step_sync(Grp& cx, bool solo) {
 // a step is shorter than the barrier of the group after it.
 constexpr int64_t kSoloCells = 4096;
 
-__device__ bool smooth_level(Grp& cx, const BParams& P, const BLevel& L, const float* f, float* x, int sweeps,
+__device__ bool smooth_level(Grp& cx, const BParams& P, const BLevel& L, int l, const float* f, float* x, int sweeps,
                              bool first_zero, bool reverse, bool solo) {
     const int rank = solo ? 0 : cx.rank, ncta = solo ? 1 : cx.ncta, c0 = reverse ? 1 : 0;
-    float* t = L.t;  // an odd_seam: the first colour's pass goes there, the second's back into x
     for (int s = 0; s < sweeps; ++s) {
-        if (t) rb_seam(rank, ncta, L, f, x, t, c0, P.omega, first_zero && s == 0);
-        else rb_pass(rank, ncta, L, f, x, c0, P.omega, first_zero && s == 0);
+        rb_pass(rank, ncta, L, f, x, c0 | ((cx.seams >> l & 1) * kSeam), P.omega, first_zero && s == 0);
         if (!step_sync(cx, solo)) return false;
-        if (t) rb_seam(rank, ncta, L, f, t, x, 1 - c0, P.omega, false);
-        else rb_pass(rank, ncta, L, f, x, 1 - c0, P.omega, false);
+        rb_pass(rank, ncta, L, f, x, (1 - c0) | kSecond | ((cx.seams >> l & 1) * kSeam), P.omega, false);
         if (!step_sync(cx, solo)) return false;
     }
     return true;
@@ -753,7 +765,7 @@ __device__ bool vcycle_down(Grp& cx, const BParams& P, const float* f0, float* x
             for (int64_t c = (int64_t)rank * kBT + threadIdx.x; c < L.g.ncell(); c += (int64_t)ncta * kBT) x[c] = 0.f;
             if (!step_sync(cx, solo)) return false;
         }
-        if (!smooth_level(cx, P, L, f, x, P.nu1, true, false, solo)) return false;
+        if (!smooth_level(cx, P, L, l, f, x, P.nu1, true, false, solo)) return false;
         restrict_level(rank, ncta, L, I.lv[l + 1], f, x);
         if (!step_sync(cx, solo)) return false;
     }
@@ -768,7 +780,7 @@ __device__ bool vcycle_up(Grp& cx, const BParams& P, const float* f0, float* x0,
         float* x = l == 0 ? x0 : L.x;
         prolong_level(rank, ncta, L, I.lv[l + 1], x);
         if (!step_sync(cx, solo)) return false;
-        if (!smooth_level(cx, P, L, l == 0 ? f0 : L.f, x, P.nu2, false, true, solo)) return false;
+        if (!smooth_level(cx, P, L, l, l == 0 ? f0 : L.f, x, P.nu2, false, true, solo)) return false;
     }
     return true;
 }
@@ -816,8 +828,8 @@ __device__ bool vcycle(Grp& cx, const BParams& P, const float* f0, float* x0) {
         const BLevel& Cl = I.lv[nl - 1];
         const float* f = nl == 1 ? f0 : Cl.f;
         float* x = nl == 1 ? x0 : Cl.x;
-        if (!smooth_level(cx, P, Cl, f, x, 8, true, false, false)) return false;
-        if (!smooth_level(cx, P, Cl, f, x, 8, false, true, false)) return false;
+        if (!smooth_level(cx, P, Cl, nl - 1, f, x, 8, true, false, false)) return false;
+        if (!smooth_level(cx, P, Cl, nl - 1, f, x, 8, false, true, false)) return false;
     }
     return vcycle_up(cx, P, f0, x0, stop - 1, 0, false);
 }
@@ -1092,6 +1104,7 @@ __global__ void __launch_bounds__(kBT, 2) persistent_kernel(const BInst* __restr
     cx.ncta = cx.I->ncta;
     cx.err = err;
     cx.pb = 0;
+    cx.seams = cx.I->seams;
     cx.arrivals = 0;
     cx.spin = P.spin_limit;
     const BInst& I = *cx.I;
@@ -1359,7 +1372,11 @@ paris_status paris_batch_create(paris_batch** out, int n, const paris_grid* grid
             L.mq = fast_div_mul(std::max(1, L.g.nx / 4));
             L.x = l == 0 ? nullptr : balloc<float>(b, L.g.ncell(), e);
             L.f = l == 0 ? nullptr : balloc<float>(b, L.g.ncell(), e);
-            L.t = odd_seam(L.g) ? balloc<float>(b, L.g.ncell(), e) : nullptr;
+            L.t = nullptr;
+            if (odd_seam(L.g)) {
+                I.seams |= 1u << l;
+                L.t = balloc<float>(b, L.g.ncell(), e);
+            }
         }
         const int64_t N = H.g0.ncell();
         for (int a = 0; a < 3; ++a) I.b64[a] = balloc<double>(b, H.g0.nface(a), e);
